@@ -1062,70 +1062,54 @@ k_outer(int64_t n, Batch B, const double4_32a* __restrict__ posh,
     }
 }
 
-// After the precision 0 density kernel (k_density_df with OUTER): i joins the
-// outer part of row j for every gather entry e of row i whose bit is set in
-// omask (i is not in N_j). One thread per row; the rows' gather parts are
-// only read and their outer parts only written, so nothing overlaps.
-__global__ void __launch_bounds__(kThreads)
-k_append_outer(int64_t n, Batch B, const unsigned long long* __restrict__ omask,
-               const int32_t* __restrict__ ngather, int32_t* __restrict__ rslab,
-               int32_t* __restrict__ ocnt, unsigned* __restrict__ status) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n || (status[2] & IF_SLAB_OVF)) return;  // the CSR holds the whole rows
-    const int inst = slot_inst(B, i);
-    if (!slot_real(B, inst, i)) return;
-    // up to four appends in flight per thread: their loads, then their atomic
-    // slots, then their stores (each append is a chain of three memory steps)
-    constexpr int kBatch = 4;
-    const int32_t* row = rslab + i * kRSlab;
-    unsigned long long m0 = omask[2 * i], m1 = omask[2 * i + 1];
-    while (m0 | m1) {
-        int e[kBatch], j[kBatch], q[kBatch];
-#pragma unroll
-        for (int b = 0; b < kBatch; ++b) {
-            e[b] = -1;
-            if (m0) {
-                e[b] = __ffsll((long long)m0) - 1;
-                m0 &= m0 - 1ull;
-            } else if (m1) {
-                e[b] = 64 + __ffsll((long long)m1) - 1;
-                m1 &= m1 - 1ull;
-            }
-        }
-#pragma unroll
-        for (int b = 0; b < kBatch; ++b) j[b] = e[b] >= 0 ? row[e[b]] : 0;
-#pragma unroll
-        for (int b = 0; b < kBatch; ++b)
-            q[b] = e[b] >= 0 ? __ldg(&ngather[j[b]]) + atomicAdd(&ocnt[j[b]], 1) : 0;
-#pragma unroll
-        for (int b = 0; b < kBatch; ++b) {
-            if (e[b] < 0) continue;
-            if (q[b] < kRSlab) rslab[(int64_t)j[b] * kRSlab + q[b]] = (int32_t)i;
-            else atomicOr(&status[2], (unsigned)IF_OUTER_OVF);
-        }
-    }
-}
-
 // Row lengths, and the outer part of each row (appended in atomic order)
-// sorted by index in place, one thread per row (rows hold a few outer
-// entries): the rows, and every sum over them, become deterministic.
+// sorted by index in place: the rows, and every sum over them, become
+// deterministic. One warp per rw rows (4 to 32): the lengths are read and
+// written coalesced, one row per lane, and the rows with something to sort (two
+// outer entries or more) are taken four at a time, eight lanes each. A row's entries
+// are read once, into shared memory; the rank of an entry (the indices of a
+// row are distinct) is the number of smaller ones, and each is stored at its
+// rank. Bounded by memory latency: there is no chain of dependent memory
+// steps, as there was in the one-thread-per-row insertion sort this replaces.
+constexpr int kSortLanes = 8;
+constexpr int kSortRows = 32 / kSortLanes;  // rows a warp sorts at a time
+
 __global__ void __launch_bounds__(kThreads)
 k_rowlen_sort(int64_t n, const int32_t* __restrict__ ngather, const int32_t* __restrict__ ocnt,
-              int32_t* __restrict__ rowlen, int32_t* __restrict__ rslab,
-              const unsigned* __restrict__ status, unsigned mask) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n || (status[2] & mask)) return;
-    const int ng = ngather[i], no = ocnt[i];
-    rowlen[i] = ng + no;
-    int32_t* row = rslab + i * kRSlab + ng;
-    for (int a = 1; a < no; ++a) {  // insertion sort
-        const int32_t v = row[a];
-        int b = a - 1;
-        while (b >= 0 && row[b] > v) {
-            row[b + 1] = row[b];
-            --b;
+              int32_t* __restrict__ rowlen, int32_t* rslab, const unsigned* __restrict__ status,
+              unsigned mask, int rw) {
+    if (status[2] & mask) return;
+    __shared__ int pick[kThreads / 32][32];
+    __shared__ int32_t ents[kThreads / kSortLanes][kRSlab];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, l = lane % kSortLanes;
+    const int64_t i = ((int64_t)blockIdx.x * (kThreads / 32) + warp) * rw + lane;
+    int ng = 0, no = 0;
+    if (lane < rw && i < n) {
+        ng = ngather[i];
+        no = ocnt[i];
+        rowlen[i] = ng + no;
+    }
+    const unsigned m = __ballot_sync(kFull, no > 1);
+    if (no > 1) pick[warp][__popc(m & ((1u << lane) - 1u))] = lane;
+    __syncwarp();
+    const int rows = __popc(m);
+    int32_t* e = ents[threadIdx.x / kSortLanes];
+    for (int r = 0; r < rows; r += kSortRows) {
+        const int at = r + lane / kSortLanes;
+        const int src = at < rows ? pick[warp][at] : 0;
+        const int rng = __shfl_sync(kFull, ng, src);
+        const int rno = __shfl_sync(kFull, no, src);
+        const int cnt = at < rows ? rno : 0;
+        int32_t* row = rslab + (i - lane + src) * kRSlab + rng;
+        for (int k = l; k < cnt; k += kSortLanes) e[k] = row[k];
+        __syncwarp();
+        for (int k = l; k < cnt; k += kSortLanes) {
+            const int32_t v = e[k];
+            int rank = 0;
+            for (int q = 0; q < cnt; ++q) rank += e[q] < v ? 1 : 0;
+            row[rank] = v;
         }
-        row[b + 1] = v;
+        __syncwarp();  // e is rewritten by the next rows
     }
 }
 
@@ -1298,6 +1282,19 @@ static void csr_fallback(sph_ctx* c, cudaStream_t s, unsigned mask) {
                                                        mask);
 }
 
+static void rowlen_sort(sph_ctx* c, cudaStream_t s, unsigned mask) {
+    // a warp's rows are sorted four at a time, one round of memory latency each:
+    // fewer rows per warp while the warps do not fill the chip (measured: 4,096
+    // particles 7 us at 4 rows and 19 at 32, the 8,191-particle sphere 13 and 50;
+    // the one-thread-per-row sort took 39 and 140). At 32: 1M patch 43 us (84
+    // before), 1M sphere 78 us (182 before).
+    int rw = kSortRows;
+    while (rw < 32 && c->n >= (int64_t)c->nsm * 32 * 2 * rw) rw *= 2;
+    const int64_t per = (int64_t)(kThreads / 32) * rw;
+    k_rowlen_sort<<<(unsigned)((c->n + per - 1) / per), kThreads, 0, s>>>(
+        c->n, c->ngather, c->ocnt, c->rowlen, c->rslab, c->status, mask, rw);
+}
+
 void launch_csr(sph_ctx* c, cudaStream_t s, bool outer_later) {
     const int64_t n = c->n;
     c->csr_ready = false;
@@ -1306,7 +1303,6 @@ void launch_csr(sph_ctx* c, cudaStream_t s, bool outer_later) {
         cudaMemsetAsync(c->offsets, 0, sizeof(int64_t), s);
         return;
     }
-    const unsigned nb = (unsigned)((n + kThreads - 1) / kThreads);
     const unsigned nbw = (unsigned)((n * 32 + kThreads - 1) / kThreads);
     double4_32a* posh = c->posh[c->cur];
     const Batch B = batch_of(c);
@@ -1314,24 +1310,18 @@ void launch_csr(sph_ctx* c, cudaStream_t s, bool outer_later) {
         c->launches += 2;
         k_outer<<<nbw, kThreads, 0, s>>>(n, B, posh, c->fpos, c->tin, c->ngather, c->rslab,
                                          c->ocnt, c->status);
-        k_rowlen_sort<<<nb, kThreads, 0, s>>>(n, c->ngather, c->ocnt, c->rowlen, c->rslab,
-                                              c->status, (unsigned)IF_SLAB_OVF);
+        rowlen_sort(c, s, (unsigned)IF_SLAB_OVF);
     }
     // fallback (a row did not fit its slab): the full two-pass build into the CSR
     csr_fallback(c, s, (unsigned)IF_SLAB_OVF);
 }
 
-// After a density kernel that recorded the outer entries: append and sort
-// them, and build the CSR instead if one of them overflowed its slab.
+// After a density kernel that appended the outer entries: sort them, and build the CSR instead if one of them overflowed its slab.
 void launch_rows_finish(sph_ctx* c, cudaStream_t s) {
     const int64_t n = c->n;
     if (n == 0) return;
-    const unsigned nb = (unsigned)((n + kThreads - 1) / kThreads);
-    c->launches += 2;
-    k_append_outer<<<nb, kThreads, 0, s>>>(n, batch_of(c), c->omask, c->ngather, c->rslab,
-                                           c->ocnt, c->status);
-    k_rowlen_sort<<<nb, kThreads, 0, s>>>(n, c->ngather, c->ocnt, c->rowlen, c->rslab, c->status,
-                                          (unsigned)(IF_SLAB_OVF | IF_OUTER_OVF));
+    c->launches += 1;
+    rowlen_sort(c, s, (unsigned)(IF_SLAB_OVF | IF_OUTER_OVF));
     csr_fallback(c, s, (unsigned)IF_OUTER_OVF);
 }
 

@@ -178,10 +178,8 @@ __device__ __forceinline__ void eos_d(const KParams& kp, double rho, double u, d
 // T lanes per particle: lane s of particle i takes row entries s, s + T, ...
 // KER: the M4 spline, the Wendland C2 or the sinc kernel.
 // OUTER: the kernel also decides, for each j of N_i, whether i is in N_j --
-// r_ij^2 < (2 h_j)^2 by the defining FP64 test -- and records the entries
-// where it is not as bits of omask (bit e for gather entry e of row i);
-// k_append_outer then appends those i to the outer parts of the rows j. The
-// pair's double-float r^2 is within ~2^-45 of the defining FP64 value and
+// r_ij^2 < (2 h_j)^2 by the defining FP64 test -- and appends i to the outer
+// part of every row j where it is not (Append). The pair's double-float r^2 is within ~2^-45 of the defining FP64 value and
 // (2 h_j)^2 is packed as a float (within 2^-24), so r^2 below / above it by
 // more than 2^-20 decides; the band between takes the FP64 test itself. The
 // sets are the exact ones, as built by k_outer.
@@ -191,8 +189,7 @@ k_density_df(int64_t n, Batch B, const double4_32a* __restrict__ posh,
              const float4* __restrict__ xpk, const double* __restrict__ ue,
              Rows R, double4_32a* __restrict__ therm,
              double2* __restrict__ kern, float4* __restrict__ dpk, double* __restrict__ pint,
-             double* __restrict__ cint, unsigned* status,
-             unsigned long long* __restrict__ omask) {
+             double* __restrict__ cint, unsigned* status, OuterOut O) {
     const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / T;
     const int sub = (int)(threadIdx.x % T);
     const int inst = slot_inst(B, ((int64_t)blockIdx.x * blockDim.x) / T);
@@ -203,7 +200,6 @@ k_density_df(int64_t n, Batch B, const double4_32a* __restrict__ posh,
     const KParams& kp = B.kp[inst];
     double4_32a pi = make_double4_32a(0.0, 0.0, 0.0, 1.0);
     df acc = {0.0f, 0.0f};
-    unsigned long long om0 = 0ull, om1 = 0ull;  // OUTER: bits of the gather entries
     if (act) {
     pi = posh[i];
     const Grid& g = B.grid[inst];
@@ -216,6 +212,7 @@ k_density_df(int64_t n, Batch B, const double4_32a* __restrict__ posh,
     if (sub == 0) acc = df{I0.w, I1.w};  // self term m_i W(0, h_i): shape 1
     // rows read from the CSR (a gather set overflowed) are complete already
     const bool append = OUTER && !(R.status[2] & IF_SLAB_OVF);
+    Append ap;
     for (int e = sub; e < len; e += T) {
         const int j = __ldg(&ent[e]);
         const float4 J0 = __ldg(&xpk[3 * j]), J1 = __ldg(&xpk[3 * j + 1]);
@@ -245,28 +242,14 @@ k_density_df(int64_t n, Batch B, const double4_32a* __restrict__ posh,
                 const double Rj = 2.0 * pj.w;
                 in_j = exact_r2_def(pi, pj, per, kp.lz) < __dmul_rn(Rj, Rj);
             }
-            if (!in_j) {  // i belongs in the outer part of row j
-                if (e < 64) om0 |= 1ull << e;
-                else om1 |= 1ull << (e - 64);
-            }
+            if (!in_j) ap.add(i, j, R.ngather, O);  // i belongs in the outer part of row j
         }
     }
+    if (OUTER) ap.flush(i, O);
     }
     if (T > 1) {
         acc = dfl::lane_sum<T>(acc);
-        if (OUTER) {
-#pragma unroll
-            for (int o = 1; o < T; o <<= 1) {
-                om0 |= __shfl_xor_sync(0xffffffffu, om0, o);
-                om1 |= __shfl_xor_sync(0xffffffffu, om1, o);
-            }
-        }
         if (!act || sub != 0) return;
-    }
-    if (OUTER && !act) return;
-    if (OUTER) {
-        omask[2 * i] = om0;
-        omask[2 * i + 1] = om1;
     }
     const Grid& g = B.grid[inst];
     const double hinv = 1.0 / pi.w;
@@ -296,7 +279,7 @@ static void density_df_t(sph_ctx* c, cudaStream_t s) {
     auto go = [&](auto kernel_fn) {
         kernel_fn<<<nb, kThreads, 0, s>>>(n, batch_of(c), c->posh[b], c->xpk, c->ue[b], R,
                                           c->therm, c->kern, c->dpk, c->pint, c->cint, c->status,
-                                          c->omask);
+                                          OuterOut{c->rslab, c->ocnt, c->status});
     };
     if (c->kern_kind == KER_WENDLAND) go(k_density_df<FUSE, T, KER_WENDLAND, OUTER>);
     else if (c->kern_kind == KER_SINC) go(k_density_df<FUSE, T, KER_SINC, OUTER>);

@@ -172,8 +172,8 @@ k_pack_mx(int64_t n, Batch B, const double4_32a* __restrict__ posh,
 }
 
 // T lanes per particle: lane s of particle i takes row entries s, s + T, ...
-// OUTER: as k_density_df, the kernel also records in omask the gather entries
-// j of row i with i not in N_j. The FP32 relative coordinates put r^2 within
+// OUTER: as k_density_df, the kernel also appends i to the outer parts of the
+// rows j in N_i with i not in N_j. The FP32 relative coordinates put r^2 within
 // ~2^-21 of the defining FP64 value and 1/h_j is packed as a float, so
 // r^2 / h_j^2 below / above 4 by more than 2^-18 decides; the band between,
 // and a periodic axis shorter than 8 h_j, take the FP64 test itself.
@@ -183,7 +183,7 @@ k_density_mx(int64_t n, Batch B, const double4_32a* __restrict__ posh,
              const double* __restrict__ ue, float4* __restrict__ mpk,
              Rows R, double4_32a* __restrict__ therm,
              double* __restrict__ pint, double* __restrict__ cint, unsigned* status,
-             unsigned long long* __restrict__ omask) {
+             OuterOut O) {
     const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / T;
     const int sub = (int)(threadIdx.x % T);
     const int inst = slot_inst(B, ((int64_t)blockIdx.x * blockDim.x) / T);
@@ -193,7 +193,6 @@ k_density_mx(int64_t n, Batch B, const double4_32a* __restrict__ posh,
     if (T == 1 && !act) return;
     const KParams& kp = B.kp[inst];
     df acc = {0.0f, 0.0f};
-    unsigned long long om0 = 0ull, om1 = 0ull;  // OUTER: bits of the gather entries
     if (act) {
     const float4 a0 = mpk[5 * i], a1 = mpk[5 * i + 1];
     const float hinv = a1.w;
@@ -201,6 +200,7 @@ k_density_mx(int64_t n, Batch B, const double4_32a* __restrict__ posh,
     if (sub == 0) acc = df{a0.w, 0.0f};  // self term m_i W(0, h_i): shape 1
     // rows read from the CSR (a gather set overflowed) are complete already
     const bool append = OUTER && !(R.status[2] & IF_SLAB_OVF);
+    Append ap;
     for (int e = sub; e < len; e += T) {
         const int j = __ldg(&ent[e]);
         const float4 b0 = __ldg(&mpk[5 * j]), b1 = __ldg(&mpk[5 * j + 1]);
@@ -221,27 +221,14 @@ k_density_mx(int64_t n, Batch B, const double4_32a* __restrict__ posh,
                 const double Rj = 2.0 * pj.w;
                 in_j = exact_r2_def(posh[i], pj, zw.per, kp.lz) < __dmul_rn(Rj, Rj);
             }
-            if (!in_j) {  // i belongs in the outer part of row j
-                if (e < 64) om0 |= 1ull << e;
-                else om1 |= 1ull << (e - 64);
-            }
+            if (!in_j) ap.add(i, j, R.ngather, O);  // i belongs in the outer part of row j
         }
     }
+    if (OUTER) ap.flush(i, O);
     }
     if (T > 1) {
         acc = dfl::lane_sum<T>(acc);
-        if (OUTER) {
-#pragma unroll
-            for (int o = 1; o < T; o <<= 1) {
-                om0 |= __shfl_xor_sync(0xffffffffu, om0, o);
-                om1 |= __shfl_xor_sync(0xffffffffu, om1, o);
-            }
-        }
         if (!act || sub != 0) return;
-    }
-    if (OUTER) {
-        omask[2 * i] = om0;
-        omask[2 * i + 1] = om1;
     }
     const Grid& g = B.grid[inst];
     const double hd = posh[i].w;
@@ -377,7 +364,7 @@ static void density_mx_t(sph_ctx* c, cudaStream_t s) {
     const int b = c->cur;
     k_density_mx<FUSE, T, OUTER><<<nb, kThreads, 0, s>>>(
         n, batch_of(c), c->posh[b], c->ue[b], c->mpk, OUTER ? rows_gather(c) : rows_of(c),
-        c->therm, c->pint, c->cint, c->status, c->omask);
+        c->therm, c->pint, c->cint, c->status, OuterOut{c->rslab, c->ocnt, c->status});
 }
 
 template <bool FUSE, bool OUTER>
