@@ -1,5 +1,5 @@
 // scan.cu -- device-wide exclusive prefix sums (reduce, scan partials, apply).
-// Used for the radix-sort digit offsets and for the neighbour-list row offsets.
+// Used for the neighbour-list row offsets.
 #include "sph_internal.cuh"
 
 namespace sph {
@@ -115,15 +115,6 @@ void launch_scan_i32_i64(const int32_t* in, int64_t n, int64_t* out, int64_t* pa
     k_scan_partials<int64_t><<<1, kThreads, 0, s>>>(part, np, gate, mask);
     k_scan_apply<int32_t, int64_t><<<(unsigned)np, kThreads, 0, s>>>(in, n, part, out, 1, gate,
                                                                       mask);
-}
-
-void launch_scan_u32(uint32_t* data, int64_t n, uint32_t* part, cudaStream_t s) {
-    if (n <= 0) return;
-    const int64_t np = scan_parts(n);
-    k_scan_reduce<uint32_t, uint32_t><<<(unsigned)np, kThreads, 0, s>>>(data, n, part, nullptr, 0u);
-    k_scan_partials<uint32_t><<<1, kThreads, 0, s>>>(part, np, nullptr, 0u);
-    k_scan_apply<uint32_t, uint32_t><<<(unsigned)np, kThreads, 0, s>>>(data, n, part, data, 0,
-                                                                        nullptr, 0u);
 }
 
 }  // namespace sph

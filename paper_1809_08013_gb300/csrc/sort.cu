@@ -1,8 +1,9 @@
 // sort.cu -- Algorithm 1 step 1 (the tree build), done as Morton-sorted cell
 // lists: bounding box and cell grid on the device, 24-bit Morton key of each
 // particle's cell, a stable LSD radix sort (3 passes of 8 bits, one more for
-// the instance id of a batch), the permutation of the particle state into
-// sorted order, and the [start, end) range of every occupied cell.
+// the instance id of a batch; one kernel per pass), the permutation of the
+// particle state into sorted order with the [start, end) range of every
+// occupied cell.
 //
 // The keys are sorted in caller order (each particle at its "rank" roff[k] +
 // its index within its instance), not in the order the previous step left,
@@ -203,7 +204,12 @@ __global__ void __launch_bounds__(kBoxThreads)
 k_bbox(int64_t n, Batch B, const double4_32a* __restrict__ posh,
        const double4_32a* __restrict__ velm, const double* __restrict__ ue,
        const int32_t* __restrict__ order, const LMeta* __restrict__ lmeta,
-       double* __restrict__ part, unsigned* __restrict__ status) {
+       double* __restrict__ part, unsigned* __restrict__ status, uint32_t* __restrict__ hist,
+       int64_t nhist) {
+    // the digit counts of the sort that follows, cleared for k_keys and its passes
+    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < nhist;
+         t += (int64_t)gridDim.x * blockDim.x)
+        hist[t] = 0u;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t grp = blockIdx.x;  // group of kSlotAlign slots (< n: one block per group)
     const int64_t w0 = grp * kSlotAlign + (int64_t)warp * kBoxWarpSlots;
@@ -341,54 +347,57 @@ k_grid_setup(const double* __restrict__ part, Batch B, Grid* __restrict__ grid,
         acc = fmin_ ? (ok < acc ? ok : acc) : (ok > acc ? ok : acc);
         hsum = lane < 16 ? hsum + oh : oh + hsum;
     }
+    static_assert(kGridThreads / 32 == 32, "one lane per warp's partial below");
     __shared__ long long wk[kGridThreads / 32][16];
     __shared__ double wh[kGridThreads / 32];
     if (lane < 16) wk[warp][lane] = acc;
     if (lane == 3 + kBoxMax) wh[warp] = hsum;
     __syncthreads();
-    __shared__ double r[11];
-    __shared__ long long lk[4];  // list keys: displacement, -slack, stamp, -stamp
-    if (threadIdx.x == 0) {
-        BoxPart a;
-        box_init(a);
-        for (int w = 0; w < kGridThreads / 32; ++w) {
-            for (int d = 0; d < 3; ++d) a.mn[d] = wk[w][d] < a.mn[d] ? wk[w][d] : a.mn[d];
-            for (int d = 0; d < kBoxMax; ++d) a.mx[d] = wk[w][3 + d] > a.mx[d] ? wk[w][3 + d] : a.mx[d];
-            a.hs += wh[w];
+    // warp f combines field f over the warps by shuffles (one thread combining
+    // all of them in turn took half of this kernel's time at small sizes); the
+    // sum of h in the order of the warps
+    __shared__ long long fk[3 + kBoxMax];
+    __shared__ double hs;
+    if (warp < 3 + kBoxMax) {
+        long long v = wk[lane][warp];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const long long u = __shfl_xor_sync(0xffffffffu, v, o);
+            v = warp < 3 ? (u < v ? u : v) : (u > v ? u : v);
         }
-        // the layout the grid derivation below reads: min x, y, z, -max x, y, z, -max h, sum h
-        for (int d = 0; d < 3; ++d) {
-            r[d] = okey_inv(a.mn[d]);
-            r[3 + d] = -okey_inv(a.mx[d]);
-        }
-        r[6] = -okey_inv(a.mx[3]);
-        r[7] = a.hs;
-        r[8] = okey_inv(a.mx[4]);   // max m
-        r[9] = okey_inv(a.mx[5]);   // max |v| component
-        r[10] = okey_inv(a.mx[6]);  // max u
-        for (int q = 0; q < 4; ++q) lk[q] = a.mx[BX_D + q];
+        if (lane == 0) fk[warp] = v;
+    } else if (warp == 3 + kBoxMax && lane == 0) {
+        double a = 0.0;
+        for (int w = 0; w < kGridThreads / 32; ++w) a += wh[w];
+        hs = a;
     }
     __syncthreads();
-    if (threadIdx.x != 0) return;
-    const KParams kp = B.kp[inst];
+    if (warp != 0) return;
+    // The rest is one warp: lane d (0 to 2) takes axis d, the others repeat
+    // axis 2; the divisions of the three axes and of the mean run side by side.
+    const int d = lane < 2 ? lane : 2;
+    const long long* lk = fk + 3 + BX_D;  // list keys: displacement, -slack, stamp, -stamp
+    const KParams& kp = B.kp[inst];
     Grid* g = grid + inst;
-    const long long cellcap = g->cap;
-    double mn[3] = {r[0], r[1], r[2]};
-    double mx[3] = {-r[3], -r[4], -r[5]};
-    for (int d = 0; d < 3; ++d)  // no particle, or none inside the geometry range
-        if (n == 0 || !(mn[d] <= mx[d])) { mn[d] = 0.0; mx[d] = 0.0; }
-    if (inst == 0) {
+    const bool per = kp.periodic_z != 0;
+    const double lz = kp.lz;
+    double mn = okey_inv(fk[d]), mx = okey_inv(fk[3 + d]);
+    // no particle, or none inside the geometry range
+    if (n == 0 || !__all_sync(0xffffffffu, mn <= mx)) {
+        if (n == 0 || !(mn <= mx)) { mn = 0.0; mx = 0.0; }
+    }
+    if (inst == 0 && lane == 0) {
         status[2] = 0u;
         status[3] = 0u;
         wctr[0] = 0ull;
     }
-    const double hmean = n > 0 ? r[7] / (double)n : 1.0;
+    const double hmean = n > 0 ? hs / (double)n : 1.0;
     double w = 2.0 * hmean * kp.cell_scale;
     if (!(w > 0.0) || !isfinite(w)) w = 1.0;
-    const bool per = kp.periodic_z != 0;
-    double X = 0.0;
-    for (int d = 0; d < 3; ++d) X = fmax(X, fmax(fabs(mn[d]), fabs(mx[d])));
-    if (per) X = fmax(X, 0.5 * kp.lz);
+    double X = fmax(fabs(mn), fabs(mx));
+    X = fmax(X, __shfl_xor_sync(0xffffffffu, X, 1));
+    X = fmax(__shfl_sync(0xffffffffu, X, 0), __shfl_sync(0xffffffffu, X, 2));
+    if (per) X = fmax(X, 0.5 * lz);
     // Candidate lists of the h search. The instance keeps its lists while
     // every particle carries the same build stamp and twice the largest
     // displacement since that build (bounded with the truncation errors of
@@ -399,6 +408,7 @@ k_grid_setup(const double* __restrict__ part, Batch B, Grid* __restrict__ grid,
     // its cells, whose walks then reach further by the displacement bound.
     bool keep = false;
     float dm2 = CUDART_INF_F;
+    int stamp = 0;
     if (kp.list_skin > 0.0 && n > 0) {
         const long long smax = lk[2], smin = -lk[3];
         const bool epoch = smax == smin && smin > 0;
@@ -407,88 +417,99 @@ k_grid_setup(const double* __restrict__ part, Batch B, Grid* __restrict__ grid,
         dm2 = (float)(2.0 * Dm * (1.0 + 0x1p-20));
         const float slack = lk[1] == kKeyMin ? CUDART_INF_F : -fkey_inv(lk[1]);
         keep = epoch && g->gvalid && dm2 < slack;  // false for a NaN displacement
-        g->lstamp = keep ? (int)smin : (int)((atomicAdd(lctr, 1u) & 0x3fffffffu) + 1u);
-    } else {
-        g->lstamp = 0;
+        if (keep) stamp = (int)smin;
+        else if (lane == 0) stamp = (int)((atomicAdd(lctr, 1u) & 0x3fffffffu) + 1u);
     }
+    int cnt = 1;
+    double ww = 1.0, lo = mn;
+    if (!keep) {
+        const long long cellcap = g->cap;
+        long long cells = 1;
+        for (int tries = 0; tries < 200; ++tries) {
+            if (per && d == 2) {
+                double c = floor(lz / w);
+                if (c < 1.0) c = 1.0;
+                if (c > (double)kMaxCellsPerAxis) c = (double)kMaxCellsPerAxis;
+                cnt = (int)c;
+                lo = -0.5 * lz;
+                ww = lz / c;
+            } else {
+                cnt = grid_count(mx - mn, w, &ww);
+            }
+            cells = (long long)__shfl_sync(0xffffffffu, cnt, 0) *
+                    __shfl_sync(0xffffffffu, cnt, 1) * __shfl_sync(0xffffffffu, cnt, 2);
+            if (cells <= cellcap) break;
+            w *= 1.25;
+        }
+        if (lane < 3) {
+            const double inv = 1.0 / ww;
+            g->lo[d] = lo;
+            g->w[d] = ww;
+            g->inv_w[d] = inv;
+            g->n[d] = cnt;
+            g->lof[d] = (float)lo;
+            g->wf[d] = (float)ww;
+            g->invwf[d] = (float)inv;
+        }
+        if (lane == 0) {
+            // (an empty instance has no cells: no block clears or marks them)
+            g->ncells = n > 0 ? cells : 0;
+            g->gvalid = 1;
+        }
+    } else {
+        ww = g->w[d];
+    }
+    if (lane < 3)
+        g->slop[d] = (float)(1e-3 * ww + 1.2e-7 * X + (keep ? 0.5 * 1.001 * dm2 : 0.0));
+    if (lane != 0) return;
+    g->lstamp = stamp;
     g->lbuild = kp.list_skin > 0.0 && n > 0 && !keep ? 1 : 0;
     g->dm2 = dm2;
-    int cnt[3];
-    double ww[3], lo[3];
-    for (int tries = 0; tries < 200 && !keep; ++tries) {
-        for (int d = 0; d < 3; ++d) {
-            lo[d] = mn[d];
-            cnt[d] = grid_count(mx[d] - mn[d], w, &ww[d]);
-        }
-        if (per) {
-            double c = floor(kp.lz / w);
-            if (c < 1.0) c = 1.0;
-            if (c > (double)kMaxCellsPerAxis) c = (double)kMaxCellsPerAxis;
-            cnt[2] = (int)c;
-            lo[2] = -0.5 * kp.lz;
-            ww[2] = kp.lz / c;
-        }
-        if ((long long)cnt[0] * cnt[1] * cnt[2] <= cellcap) break;
-        w *= 1.25;
-    }
-    if (!keep) {
-        for (int d = 0; d < 3; ++d) {
-            g->lo[d] = lo[d];
-            g->w[d] = ww[d];
-            g->inv_w[d] = 1.0 / ww[d];
-            g->n[d] = cnt[d];
-            g->lof[d] = (float)lo[d];
-            g->wf[d] = (float)ww[d];
-            g->invwf[d] = (float)(1.0 / ww[d]);
-        }
-        g->ncells = (long long)cnt[0] * cnt[1] * cnt[2];
-        g->gvalid = 1;
-    }
-    for (int d = 0; d < 3; ++d)
-        g->slop[d] = (float)(1e-3 * g->w[d] + 1.2e-7 * X + (keep ? 0.5 * 1.001 * dm2 : 0.0));
     g->periodic_z = per ? 1 : 0;
-    g->lz = kp.lz;
-    g->lzf = (float)kp.lz;
-    g->halflzf = (float)(0.5 * kp.lz);
+    g->lz = lz;
+    g->lzf = (float)lz;
+    g->halflzf = (float)(0.5 * lz);
     g->X = X;
     // |fl32 difference - FP64 difference| <= 2^-24 (4X + 2.02R + 2 lz) per
     // component (conversions of both coordinates, the FP32 subtraction, the
     // periodic shift); 1.0001 and the upward rounding keep it an upper bound
     const double u24 = 5.9604644775390625e-08;
-    g->eC = __double2float_ru(u24 * (4.0 * X + (per ? 2.0 * kp.lz : 0.0)) * 1.0001 + 1e-37);
+    g->eC = __double2float_ru(u24 * (4.0 * X + (per ? 2.0 * lz : 0.0)) * 1.0001 + 1e-37);
     g->eR = __double2float_ru(u24 * 2.02 * 1.0001);
     // Units of the pair kernels (Grid::uL, uM, uV): the power of two at or
     // just above the mean h, the largest mass and a velocity scale (the
     // largest |v| component, or the sound speed the parameters imply if that
     // is larger: c0 for Tait, sqrt(gamma (gamma - 1) max u) for an ideal gas).
-    auto unit_exp = [](double v) {
-        int e = 0;
+    // The exponents come from the bits (v < 2^e; a subnormal ends at the
+    // clamp).
+    auto exp2_of = [](double v) { return (int)((__double_as_longlong(v) >> 52) & 0x7ff) - 1022; };
+    auto unit_exp = [&](double v) {
         if (!(v > 0.0) || !isfinite(v)) return 0;
-        frexp(v, &e);  // v < 2^e
+        const int e = exp2_of(v);
         return e < -300 ? -300 : (e > 300 ? 300 : e);
     };
-    double vs = n > 0 ? r[9] : 0.0;
+    const double umax = okey_inv(fk[3 + 6]);
+    double vs = n > 0 ? okey_inv(fk[3 + 5]) : 0.0;
     if (kp.eos == 0) vs = fmax(vs, fabs(kp.c0));
-    else if (n > 0 && r[10] > 0.0) vs = fmax(vs, sqrt(kp.gamma * (kp.gamma - 1.0) * r[10]));
-    g->uL = unit_exp(hmean);
-    g->uM = unit_exp(n > 0 ? r[8] : 0.0);
+    else if (n > 0 && umax > 0.0) vs = fmax(vs, sqrt(kp.gamma * (kp.gamma - 1.0) * umax));
+    const int uL = unit_exp(hmean);
+    g->uL = uL;
+    g->uM = unit_exp(n > 0 ? okey_inv(fk[3 + 4]) : 0.0);
     g->uV = unit_exp(vs);
     // fixed-point exponent of the coordinate chunks (dfl::to_fx): |x| 2^k < 2^61,
     // and the chunks' float exponent k + uL must keep them normal floats
-    int ex = 0;
-    frexp(X, &ex);  // X < 2^ex
-    int k = X > 0.0 && isfinite(X) ? 61 - ex : 61;
+    int k = X > 0.0 && isfinite(X) ? 61 - exp2_of(X) : 61;
     k = k < -1000 ? -1000 : (k > 1000 ? 1000 : k);
-    if (k + g->uL > 100 || k + g->uL < -60) {  // coordinates out of all proportion to h
-        k = k + g->uL > 100 ? 100 - g->uL : -60 - g->uL;
+    if (k + uL > 100 || k + uL < -60) {  // coordinates out of all proportion to h
+        k = k + uL > 100 ? 100 - uL : -60 - uL;
         if (kp.precision == PREC_FP64) atomicOr(&status[0], (unsigned)ST_RANGE);
     }
     g->fxk = k;
-    const dfl::fx3 L = dfl::to_fx(per ? kp.lz : 0.0, k, k + g->uL);
+    const dfl::fx3 L = dfl::to_fx(per ? lz : 0.0, k, k + uL);
     g->lzc[0] = L.c2;
     g->lzc[1] = L.c1;
     g->lzc[2] = L.c0;
-    g->hlzc = (float)(0.5 * kp.lz * p2d(-g->uL));
+    g->hlzc = (float)(0.5 * lz * p2d(-uL));
     g->hmean = hmean;
     g->hmax_bits = 0ull;
 }
@@ -530,15 +551,22 @@ __device__ __forceinline__ int cell_coord(double v, float lo, float inv, int n) 
 // While the instance keeps its candidate lists, the code is the particle's
 // code at the list build, so the sort gives every particle its slot of then;
 // a build step records the codes it sorts by.
+// Also counts the keys' first digits (a chained sort) and clears the cells.
 __global__ void __launch_bounds__(kThreads)
 k_keys(int64_t n, Batch B, const int64_t* __restrict__ coff, const int64_t* __restrict__ roff,
        const double4_32a* __restrict__ posh, const int32_t* __restrict__ order,
-       uint32_t* __restrict__ keys, int32_t* __restrict__ vals, LMeta* __restrict__ lmeta) {
+       uint32_t* __restrict__ keys, int32_t* __restrict__ vals, LMeta* __restrict__ lmeta,
+       RadixGeom R, uint32_t* __restrict__ hist, int2* __restrict__ cells) {
     const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n) return;
-    const int inst = slot_inst(B, k);
-    if (!slot_real(B, inst, k)) return;
+    const int inst = slot_inst(B, (int64_t)blockIdx.x * blockDim.x);
     const Grid* g = B.grid + inst;
+    {
+        const int64_t all = (__ldg(&B.icnt[inst]) + kThreads - 1) / kThreads * kThreads;
+        const long long nc = g->ncells, cb = g->cbase;
+        for (long long c = k - __ldg(&B.ioff[inst]); c < nc; c += all) cells[cb + c] = make_int2(0, 0);
+    }
+    if (k >= n) return;
+    if (!slot_real(B, inst, k)) return;
     const bool lists = B.kp[inst].list_skin > 0.0;
     const int32_t id = order[k];
     uint32_t code;
@@ -555,46 +583,99 @@ k_keys(int64_t n, Batch B, const int64_t* __restrict__ coff, const int64_t* __re
     const int64_t q = __ldg(&roff[inst]) + ((int64_t)id - __ldg(&coff[inst]));
     keys[q] = ((uint32_t)inst << 24) | code;
     vals[q] = (int32_t)k;
+    if (R.chained) R.count(hist, q >> R.tile_shift, code & 255u, 1u);
 }
 
 // --------------------------------------------------------- stable radix sort
+// The blocks of a pass need, for every digit, the number of keys with a
+// smaller digit and of keys with that digit in earlier tiles; both come from
+// counts per tile and per group of tiles. Small sorts (RadixGeom::chained) are
+// one kernel per pass: whoever writes a key to its place for a pass (k_keys,
+// or the pass before) knows the tile it lands in and its next digit, and
+// counts it by atomic additions (integers: the order does not matter). Large
+// ones, where those additions cost more than reading the keys once more
+// (measured at 1M: 35 us a pass against 8), count in a kernel of their own.
+// Either way no scan kernels: a histogram kernel and the three kernels of a
+// scan in each pass made 15 launches of 3-7 us each in a 27k-particle step.
 __global__ void __launch_bounds__(kThreads)
-k_radix_hist(const uint32_t* __restrict__ keys, int64_t n, int shift, uint32_t* __restrict__ hist,
-             int nblocks) {
+k_radix_hist(const uint32_t* __restrict__ keys, int64_t n, int shift, RadixGeom R,
+             uint32_t* __restrict__ hist) {
     __shared__ uint32_t h[256];
     h[threadIdx.x] = 0;
     __syncthreads();
-    const int64_t base = (int64_t)blockIdx.x * kRadixTile;
+    const int64_t base = (int64_t)blockIdx.x * kThreads * kRadixItems;
 #pragma unroll
     for (int k = 0; k < kRadixItems; ++k) {
         const int64_t i = base + k * kThreads + threadIdx.x;
         if (i < n) atomicAdd(&h[(keys[i] >> shift) & 255u], 1u);
     }
     __syncthreads();
-    hist[(int64_t)threadIdx.x * nblocks + blockIdx.x] = h[threadIdx.x];
+    R.count(hist, blockIdx.x, threadIdx.x, h[threadIdx.x]);
 }
 
-// Each warp ranks a contiguous run of 256 keys in (iteration, lane) order, so
-// the rank of a key among equal digits follows its input position: stable.
+// Each warp ranks a contiguous run of keys in (iteration, lane) order, so the
+// rank of a key among equal digits follows its input position: stable.
+template <int ITEMS, bool NEXT>
 __global__ void __launch_bounds__(kThreads)
 k_radix_scatter(const uint32_t* __restrict__ kin, const int32_t* __restrict__ vin, int64_t n,
-                int shift, const uint32_t* __restrict__ hist, int nblocks,
-                uint32_t* __restrict__ kout, int32_t* __restrict__ vout) {
+                int shift, RadixGeom R, const uint32_t* __restrict__ hist,
+                uint32_t* __restrict__ next, uint32_t* __restrict__ kout,
+                int32_t* __restrict__ vout) {
     __shared__ uint32_t cnt[kThreads / 32][256];
+    __shared__ uint32_t wtot[kThreads / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t base = (int64_t)blockIdx.x * (kThreads * ITEMS) + warp * (32 * ITEMS);
+    uint32_t key[ITEMS];
+    int32_t val[ITEMS];
+    uint32_t rank[ITEMS];
+#pragma unroll
+    for (int it = 0; it < ITEMS; ++it) {
+        const int64_t i = base + it * 32 + lane;
+        key[it] = i < n ? kin[i] : 0u;
+        val[it] = i < n ? vin[i] : 0;
+    }
+    // thread d: keys of digit d in all tiles, and in the tiles before this one
+    uint32_t total = 0, before = 0;
+    {
+        static_assert(kThreads == 256, "one digit per thread");
+        const int d = threadIdx.x;
+        const int tile = (int)blockIdx.x;
+        if (R.groups == 1) {
+#pragma unroll 8
+            for (int t = 0; t < R.tiles; ++t) {
+                const uint32_t v = __ldg(&hist[t * 256 + d]);
+                total += v;
+                before += t < tile ? v : 0u;
+            }
+        } else {
+            const int grp = tile >> R.group_shift;
+            const uint32_t* groups = hist + (int64_t)R.tiles * 256;
+#pragma unroll 8
+            for (int g = 0; g < R.groups; ++g) {
+                const uint32_t v = __ldg(&groups[g * 256 + d]);
+                total += v;
+                before += g < grp ? v : 0u;
+            }
+#pragma unroll 8
+            for (int t = grp << R.group_shift; t < tile; ++t)
+                before += __ldg(&hist[(int64_t)t * 256 + d]);
+        }
+    }
+    uint32_t inc = total;  // inclusive scan of the totals over the digits
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t v = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += v;
+    }
+    if (lane == 31) wtot[warp] = inc;
     for (int q = threadIdx.x; q < (kThreads / 32) * 256; q += kThreads) (&cnt[0][0])[q] = 0;
     __syncthreads();
-    const int64_t base = (int64_t)blockIdx.x * kRadixTile + warp * (32 * kRadixItems);
-    uint32_t key[kRadixItems];
-    int32_t val[kRadixItems];
-    uint32_t rank[kRadixItems];
+    uint32_t start = before + inc - total;  // place of this tile's first key of digit d
+    for (int w = 0; w < warp; ++w) start += wtot[w];
     const uint32_t lt = (1u << lane) - 1u;
 #pragma unroll
-    for (int it = 0; it < kRadixItems; ++it) {
-        const int64_t i = base + it * 32 + lane;
-        const bool ok = i < n;
-        key[it] = ok ? kin[i] : 0u;
-        val[it] = ok ? vin[i] : 0;
+    for (int it = 0; it < ITEMS; ++it) {
+        const bool ok = base + it * 32 + lane < n;
         const uint32_t d = ok ? ((key[it] >> shift) & 255u) : 256u;
         const uint32_t peers = __match_any_sync(0xffffffffu, d);
         const uint32_t b = ok ? cnt[warp][d] : 0u;
@@ -605,8 +686,8 @@ k_radix_scatter(const uint32_t* __restrict__ kin, const int32_t* __restrict__ vi
     }
     __syncthreads();
     {
-        const int d = threadIdx.x;  // one digit per thread
-        uint32_t run = 0;
+        const int d = threadIdx.x;
+        uint32_t run = start;
 #pragma unroll
         for (int w = 0; w < kThreads / 32; ++w) {
             const uint32_t c = cnt[w][d];
@@ -616,19 +697,19 @@ k_radix_scatter(const uint32_t* __restrict__ kin, const int32_t* __restrict__ vi
     }
     __syncthreads();
 #pragma unroll
-    for (int it = 0; it < kRadixItems; ++it) {
-        const int64_t i = base + it * 32 + lane;
-        if (i < n) {
-            const uint32_t d = (key[it] >> shift) & 255u;
-            const uint32_t pos = hist[(int64_t)d * nblocks + blockIdx.x] + cnt[warp][d] + rank[it];
+    for (int it = 0; it < ITEMS; ++it) {
+        if (base + it * 32 + lane < n) {
+            const uint32_t pos = cnt[warp][(key[it] >> shift) & 255u] + rank[it];
             kout[pos] = key[it];
             vout[pos] = val[it];
+            if (NEXT) R.count(next, pos >> R.tile_shift, (key[it] >> (shift + 8)) & 255u, 1u);
         }
     }
 }
 
 // ------------------------------------------------------ permute and cells
-// Sorted rank p of instance i goes to slot ioff[i] + (p - roff[i]).
+// Sorted rank p of instance i goes to slot ioff[i] + (p - roff[i]); the first
+// and the last particle of a cell write its range (in slots).
 __global__ void __launch_bounds__(kThreads)
 k_permute(int64_t ntot, Batch B, const int64_t* __restrict__ roff,
           const uint32_t* __restrict__ keys, const int32_t* __restrict__ perm,
@@ -637,12 +718,24 @@ k_permute(int64_t ntot, Batch B, const int64_t* __restrict__ roff,
           const int32_t* __restrict__ order_in, double4_32a* __restrict__ posh_out,
           double4_32a* __restrict__ velm_out, double* __restrict__ u_out,
           int32_t* __restrict__ order_out, float4* __restrict__ fpos, float4* __restrict__ xpk,
-          float4* __restrict__ vpa, float2* __restrict__ vpb) {
+          float4* __restrict__ vpa, float2* __restrict__ vpb, int2* __restrict__ cells) {
     const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= ntot) return;
-    const int inst = (int)(keys[r] >> 24);
-    const int64_t k = __ldg(&B.ioff[inst]) + (r - __ldg(&roff[inst]));
     const int64_t o = perm[r];
+    const uint32_t key = keys[r];
+    const int inst = (int)(key >> 24);
+    const int64_t a = __ldg(&roff[inst]), e = a + __ldg(&B.icnt[inst]);
+    const int64_t k = __ldg(&B.ioff[inst]) + (r - a);
+    const bool first = (r == a) || keys[r - 1] != key;
+    const bool last = (r == e - 1) || keys[r + 1] != key;
+    if (first || last) {
+        const Grid* g = B.grid + inst;
+        const uint32_t code = key & 0xffffffu;
+        const int kx = compact3(code), ky = compact3(code >> 1), kz = compact3(code >> 2);
+        const long long lin = g->cbase + ((long long)kz * g->n[1] + ky) * g->n[0] + kx;
+        if (first) cells[lin].x = (int)k;
+        if (last) cells[lin].y = (int)(k + 1);
+    }
     const double4_32a p = posh_in[o];
     posh_out[k] = p;
     const double4_32a v = velm_in[o];
@@ -654,43 +747,42 @@ k_permute(int64_t ntot, Batch B, const int64_t* __restrict__ roff,
     fpos[k] = make_float4((float)p.x, (float)p.y, (float)p.z, 0.0f);
 }
 
-// Clear each instance's cells (blockIdx.y = instance).
-__global__ void __launch_bounds__(kThreads)
-k_cells_clear(Batch B, int2* __restrict__ cells, unsigned long long* __restrict__ cell_hmax) {
-    const Grid* g = B.grid + blockIdx.y;
-    const long long nc = g->ncells, cb = g->cbase;
-    for (long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x; c < nc;
-         c += (long long)gridDim.x * blockDim.x) {
-        cells[cb + c] = make_int2(0, 0);
-        cell_hmax[cb + c] = 0ull;
-    }
+// Tiles of the sort for nt keys. Up to kRadixSmallN a chained sort with tiles
+// of 512 keys, so that there are blocks enough for the chip: keys and passes
+// take 39 us at 104k keys and 45 us at 200k against 50 and 58 us with a
+// histogram kernel per pass and tiles of 2048; at 1M the additions contend
+// and it is 147 us against 73.
+static RadixGeom radix_geom(int64_t nt) {
+    RadixGeom R;
+    R.chained = nt <= kRadixSmallN;
+    R.items = R.chained ? kRadixItemsSmall : kRadixItems;
+    const int64_t tile = (int64_t)kThreads * R.items;
+    R.tile_shift = 0;
+    while ((int64_t)1 << R.tile_shift < tile) R.tile_shift += 1;
+    R.tiles = (int)((nt + tile - 1) / tile);
+    // up to 64 tiles: a block reads the counts of every tile; more: groups of
+    // about sqrt(tiles), one count per group and one per earlier tile of its own
+    R.group_shift = 4;
+    while (((int64_t)4 << (2 * R.group_shift)) < R.tiles) R.group_shift += 1;
+    if (R.tiles <= 64) R.group_shift = 6;
+    R.groups = ((R.tiles - 1) >> R.group_shift) + 1;
+    return R;
 }
 
-// Cell ranges (in slots) from the sorted keys (in ranks).
-__global__ void __launch_bounds__(kThreads)
-k_cells_mark(int64_t ntot, Batch B, const int64_t* __restrict__ roff,
-             const uint32_t* __restrict__ keys, int2* __restrict__ cells) {
-    const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= ntot) return;
-    const uint32_t key = keys[r];
-    const int inst = (int)(key >> 24);
-    const int64_t a = __ldg(&roff[inst]), e = a + __ldg(&B.icnt[inst]);
-    const bool first = (r == a) || keys[r - 1] != key;
-    const bool last = (r == e - 1) || keys[r + 1] != key;
-    if (!(first || last)) return;
-    const int64_t k = __ldg(&B.ioff[inst]) + (r - a);
-    const Grid* g = B.grid + inst;
-    const uint32_t code = key & 0xffffffu;
-    const int kx = compact3(code), ky = compact3(code >> 1), kz = compact3(code >> 2);
-    const long long lin = g->cbase + ((long long)kz * g->n[1] + ky) * g->n[0] + kx;
-    if (first) cells[lin].x = (int)k;
-    if (last) cells[lin].y = (int)(k + 1);
+// Counts of one pass for at most n keys.
+int64_t radix_counts(int64_t n) {
+    const int64_t a = radix_geom(n).counts();
+    const int64_t b = radix_geom(n < kRadixSmallN ? n : kRadixSmallN).counts();
+    return a > b ? a : b;
 }
 
 void launch_build_cells(sph_ctx* c, cudaStream_t s) {
     const int64_t n = c->n;
     const unsigned nb = (unsigned)((n + kThreads - 1) / kThreads);
     const Batch B = batch_of(c);
+    const int64_t nt = c->ntot;
+    const RadixGeom R = radix_geom(nt);
+    const int passes = c->ninst > 1 ? 4 : 3;
     c->launches += 1;
     if (nb > 0) {  // one block per group of kSlotAlign slots
         c->launches += 1;
@@ -698,40 +790,49 @@ void launch_build_cells(sph_ctx* c, cudaStream_t s) {
         if (c->any_lists)
             k_bbox<true><<<gb, kBoxThreads, 0, s>>>(n, B, c->posh[c->cur], c->velm[c->cur],
                                                  c->ue[c->cur], c->order[c->cur], c->lmeta,
-                                                 c->red_part, c->status);
+                                                 c->red_part, c->status, c->hist,
+                                                 passes * R.counts());
         else
             k_bbox<false><<<gb, kBoxThreads, 0, s>>>(n, B, c->posh[c->cur], c->velm[c->cur],
                                                   c->ue[c->cur], c->order[c->cur], c->lmeta,
-                                                  c->red_part, c->status);
+                                                  c->red_part, c->status, c->hist,
+                                                  passes * R.counts());
     }
     k_grid_setup<<<c->ninst, kGridThreads, 0, s>>>(c->red_part, B, c->grid, c->status, c->wctr,
                                                     c->lctr);
     if (n == 0) return;
-    const int64_t nt = c->ntot;
     if (nt == 0) return;
     const unsigned nbt = (unsigned)((nt + kThreads - 1) / kThreads);
-    const int passes = c->ninst > 1 ? 4 : 3;
-    c->launches += 1 + passes * 5 + 3;
+    c->launches += 2 + passes;
     k_keys<<<nb, kThreads, 0, s>>>(n, B, c->coff, c->roff, c->posh[c->cur], c->order[c->cur],
-                                   c->keys[0], c->vals[0], c->lmeta);
-    const int nsb = (int)((nt + kRadixTile - 1) / kRadixTile);
+                                   c->keys[0], c->vals[0], c->lmeta, R, c->hist, c->cells);
     int src = 0;
     for (int pass = 0; pass < passes; ++pass) {
-        const int shift = 8 * pass;
-        k_radix_hist<<<nsb, kThreads, 0, s>>>(c->keys[src], nt, shift, c->hist, nsb);
-        launch_scan_u32(c->hist, (int64_t)256 * nsb, c->hist_part, s);
-        k_radix_scatter<<<nsb, kThreads, 0, s>>>(c->keys[src], c->vals[src], nt, shift, c->hist,
-                                                  nsb, c->keys[1 - src], c->vals[1 - src]);
+        const uint32_t* h = c->hist + pass * R.counts();
+        auto go = [&](auto fn) {
+            fn<<<(unsigned)R.tiles, kThreads, 0, s>>>(c->keys[src], c->vals[src], nt, 8 * pass, R, h,
+                                                      c->hist + (pass + 1) * R.counts(),
+                                                      c->keys[1 - src], c->vals[1 - src]);
+        };
+        if (!R.chained) {
+            c->launches += 1;
+            k_radix_hist<<<(unsigned)R.tiles, kThreads, 0, s>>>(
+                c->keys[src], nt, 8 * pass, R, c->hist + pass * R.counts());
+            go(k_radix_scatter<kRadixItems, false>);
+        } else if (pass + 1 < passes) {
+            go(k_radix_scatter<kRadixItemsSmall, true>);
+        } else {
+            go(k_radix_scatter<kRadixItemsSmall, false>);
+        }
         src = 1 - src;
     }
     // sorted keys / permutation now in keys[src], vals[src]
     const int a = c->cur, b = 1 - c->cur;
     k_permute<<<nbt, kThreads, 0, s>>>(nt, B, c->roff, c->keys[src], c->vals[src], c->posh[a],
                                         c->velm[a], c->ue[a], c->order[a], c->posh[b], c->velm[b],
-                                        c->ue[b], c->order[b], c->fpos, c->xpk, c->vpa, c->vpb);
+                                        c->ue[b], c->order[b], c->fpos, c->xpk, c->vpa, c->vpb,
+                                        c->cells);
     c->cur = b;
-    k_cells_clear<<<dim3(64, (unsigned)c->ninst), kThreads, 0, s>>>(B, c->cells, c->cell_hmax);
-    k_cells_mark<<<nbt, kThreads, 0, s>>>(nt, B, c->roff, c->keys[src], c->cells);
 }
 
 }  // namespace sph

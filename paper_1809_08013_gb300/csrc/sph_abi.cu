@@ -144,8 +144,7 @@ sph_status ensure_lists(sph_ctx* c) {
 void free_all(sph_ctx* c) {
     void* ptrs[] = {c->posh[0], c->posh[1], c->velm[0], c->velm[1], c->ue[0], c->ue[1],
                     c->therm, c->kern, c->acc, c->pint, c->cint, c->dpk, c->mpk, c->mumax, c->fpos, c->tin, c->order[0],
-                    c->order[1], c->keys[0], c->keys[1], c->vals[0], c->vals[1], c->hist,
-                    c->hist_part, c->cells, c->cell_hmax, c->nnb, c->ngather, c->rowlen,
+                    c->order[1], c->keys[0], c->keys[1], c->vals[0], c->vals[1], c->hist, c->cells, c->cell_hmax, c->nnb, c->ngather, c->rowlen,
                     c->offsets, c->row_part, c->idx, c->rslab, c->ocnt, c->hs_lo, c->hs_hi, c->hs_it, c->wl, c->red_part, c->dt_part, c->grid,
                     c->status, c->scratch_scalar, c->blk, c->ioff, c->icnt, c->coff, c->kpi,
                     c->tune_dt, c->roff, c->wctr, c->recs, c->iad_a, c->iad_b, c->vol, c->xpk, c->vpa, c->vpb,
@@ -204,7 +203,6 @@ bool allocate_all(sph_ctx* c, int64_t nslots, Allocator& al) {
     const int64_t max_instances = c->maxinst;
     const int64_t nnzcap = c->nnzcap;
     const size_t N = (size_t)std::max<int64_t>(nslots, 1);
-    const size_t nsb = (N + kRadixTile - 1) / kRadixTile;
     const size_t nfb = (N + kThreads - 1) / kThreads;
     bool ok = true;
     for (int b = 0; b < 2; ++b) {
@@ -217,7 +215,7 @@ bool allocate_all(sph_ctx* c, int64_t nslots, Allocator& al) {
          al(&c->mumax, N) && al(&c->iad_a, N) && al(&c->iad_b, N) && al(&c->vol, N) && al(&c->vdf, N) &&
          al(&c->cpk, 3 * N) &&
          al(&c->fpos, N) && al(&c->tin, N) &&
-         al(&c->hist, 256 * nsb) && al(&c->hist_part, (size_t)scan_parts(256 * nsb) + 1) &&
+         al(&c->hist, 4 * (size_t)radix_counts((int64_t)N)) &&
          al(&c->cells, (size_t)c->cellcap) && al(&c->cell_hmax, (size_t)c->cellcap) &&
          al(&c->nnb, N) && al(&c->ngather, N) && al(&c->rowlen, N) &&
          al(&c->offsets, N + 1) && al(&c->row_part, (size_t)scan_parts(N) + 1) &&

@@ -26,7 +26,8 @@ constexpr int kMortonBits = 8;                      // bits per axis -> 24-bit k
 constexpr int kMaxCellsPerAxis = 1 << kMortonBits;  // 256
 constexpr int kThreads = 256;
 constexpr int kRadixItems = 8;                      // keys per thread in the sort
-constexpr int kRadixTile = kThreads * kRadixItems;  // 2048 keys per block
+constexpr int kRadixItemsSmall = 2;                 // ... of at most kRadixSmallN keys
+constexpr int64_t kRadixSmallN = 262144;
 constexpr int kScanTile = kThreads * 8;             // elements per block in scans
 constexpr int kReduceBlocks = 304;                  // 2 x 152 SMs
 constexpr int kMaxPairThreads = 8;                  // lanes per particle in the pair kernels
@@ -248,6 +249,23 @@ inline KParams kparams(const sph_params* p) {
     return k;
 }
 
+// Tiling of the radix sort, and the digit counts of one of its passes: per
+// tile [tiles][256], then per group of 2^group_shift tiles [groups][256].
+struct RadixGeom {
+    bool chained;  // each pass counts for the next (else a histogram kernel does)
+    int items, tiles, groups, tile_shift, group_shift;
+    __host__ __device__ int64_t counts() const { return (int64_t)(tiles + groups) * 256; }
+    // c keys of tile t have `digit`
+    __device__ __forceinline__ void count(uint32_t* hist, int64_t t, uint32_t digit,
+                                          uint32_t c) const {
+        if (c == 0) return;
+        atomicAdd(&hist[t * 256 + digit], c);
+        if (groups > 1)
+            atomicAdd(&hist[((int64_t)tiles + (t >> group_shift)) * 256 + digit], c);
+    }
+};
+int64_t radix_counts(int64_t n);  // counts of one pass for at most n keys
+
 }  // namespace sph
 
 struct sph_ctx {
@@ -290,8 +308,7 @@ struct sph_ctx {
     int32_t* order[2];
     uint32_t* keys[2];
     int32_t* vals[2];
-    uint32_t* hist;         // 256 x sort blocks
-    uint32_t* hist_part;    // scan partials of hist
+    uint32_t* hist;         // digit counts of the sort's passes (RadixGeom)
     int2* cells;            // (start, end) per linear cell id
     unsigned long long* cell_hmax;  // per cell, bits of max h (h > 0)
     int32_t *nnb, *ngather, *rowlen;
@@ -505,8 +522,6 @@ enum : unsigned {
 // when *gate & mask is set on the device when the kernels run
 void launch_scan_i32_i64(const int32_t* in, int64_t n, int64_t* out, int64_t* part,
                          cudaStream_t s, const unsigned* gate = nullptr, unsigned mask = 0u);
-// exclusive scan in place over n uint32
-void launch_scan_u32(uint32_t* data, int64_t n, uint32_t* part, cudaStream_t s);
 int64_t scan_parts(int64_t n);
 
 }  // namespace sph
