@@ -100,8 +100,10 @@ typedef struct {
                              sums round differently for each value */
     int32_t defer_lanes;  /* h search: a warp of 32 particles hands its particles still
                              searching to one warp each once at most this many remain
-                             (0 selects 16; at most 32). A tuning knob: h and the
-                             neighbour sets do not depend on it */
+                             (0 selects 16; at most 32; an instance of fewer than
+                             100,000 particles without candidate lists hands over every
+                             particle that a first count leaves searching). A tuning
+                             knob: h and the neighbour sets do not depend on it */
     double rho0, c0;     /* Tait: p = c0^2 rho0 / 7 ((rho/rho0)^7 - 1), c = c0 (rho/rho0)^3 */
     double gamma;        /* ideal gas: p = (gamma - 1) rho u, c = sqrt(gamma (gamma - 1) u) */
     double alpha, beta;  /* Monaghan artificial viscosity */

@@ -26,6 +26,7 @@
 #include <math_constants.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "df.cuh"
 #include "sph_internal.cuh"
@@ -167,20 +168,53 @@ __device__ __forceinline__ float wmax(float v) {
     return v;
 }
 
+// A flat list of the particles of up to 32 cells, one cell per lane (num
+// particles from slot start on): place t of the list is slot t + delta[k] of
+// the k-th occupied cell. The warp's 32 places t0 .. t0 + 31 find their cells
+// from the number of cells that start before t0 and a word of the places where
+// cells start after it, both by warp votes: no search in memory.
+struct FlatCells {
+    int pl, total;  // place of this lane's cell (INT_MAX: empty), length of the list
+    __device__ __forceinline__ FlatCells(int num, int start, int* delta) {
+        const int lane = threadIdx.x & 31;
+        int inc = num;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(kFull, inc, o);
+            if (lane >= o) inc += v;
+        }
+        total = __shfl_sync(kFull, inc, 31);
+        const int place = inc - num;
+        const unsigned occ = __ballot_sync(kFull, num > 0);
+        if (num > 0) delta[__popc(occ & ((1u << lane) - 1u))] = start - place;
+        pl = num > 0 ? place : 0x7fffffff;
+        __syncwarp();
+    }
+    // slot of place t0 + lane, -1 from place `end` on (t0 < total)
+    __device__ __forceinline__ int slot(int t0, int end, const int* delta) const {
+        const int lane = threadIdx.x & 31;
+        const unsigned before = __ballot_sync(kFull, pl < t0);
+        unsigned bit;  // (shl gives 0 for a shift of 32 or more, as of a negative one)
+        asm("shl.b32 %0, 1, %1;" : "=r"(bit) : "r"(pl - t0));
+        const unsigned starts = __reduce_or_sync(kFull, bit);
+        const int k = __popc(before) + __popc(starts & (0xffffffffu >> (31 - lane))) - 1;
+        return t0 + lane < end ? t0 + lane + delta[k] : -1;
+    }
+};
+
 // One warp, one particle: enumerate the candidates of every cell overlapping
-// the box [q - R, q + R] as one flat list. Up to 32 cells are fetched at once
-// (one per lane), a warp scan of their sizes gives each cell's offset, and the
-// list is handed out 32 candidates at a time: chunk(valid, j) is called by
-// all lanes together, lane l receiving candidate j (valid = false past the
-// end). PRUNE = 1 drops a cell whose box lies farther than R from the
+// the box [q - R, q + R] as one flat list, the cells 32 at a time. The list is
+// handed out 32 candidates at a time: chunk(valid, j, f) is called by all
+// lanes together, lane l receiving candidate j at f = fpos[j] (valid = false
+// past the end); the next candidates load meanwhile. PRUNE = 1 drops a cell whose box lies farther than R from the
 // particle; PRUNE = 2 drops it unless its box lies within
 // 2 max(h_i, max h of the cell) of the particle (hib = bits of h_i).
 template <int PRUNE, class Chunk>
 __device__ __forceinline__ void particle_pass(const Grid* __restrict__ g,
                                               const int2* __restrict__ cells,
                                               const unsigned long long* __restrict__ cell_hmax,
-                                              const float4& q, float R, long long hib,
-                                              int* s_start, int* s_pref, Chunk&& chunk) {
+                                              const float4* __restrict__ fpos, const float4& q,
+                                              float R, long long hib, int* delta, Chunk&& chunk) {
     const int lane = threadIdx.x & 31;
     int x0, x1, y0, y1, z0, z1;
     axis_range(q.x, R, g, 0, x0, x1);
@@ -203,7 +237,7 @@ __device__ __forceinline__ void particle_pass(const Grid* __restrict__ g,
             const long long lin = ((long long)cz * ny + ky) * nx + kx;
             const int2 se = __ldg(&cells[lin]);
             start = se.x;
-            cnt = se.y - se.x;
+            cnt = max(se.y - se.x, 0);
             if (PRUNE && cnt > 0) {
                 float reach = R;
                 if (PRUNE == 2) {
@@ -215,29 +249,147 @@ __device__ __forceinline__ void particle_pass(const Grid* __restrict__ g,
                 if (fmaf(gz, gz, fmaf(gy, gy, gx * gx)) >= reach * reach) cnt = 0;
             }
         }
-        int inc = cnt;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int v = __shfl_up_sync(kFull, inc, o);
-            if (lane >= o) inc += v;
-        }
-        const int total = __shfl_sync(kFull, inc, 31);
-        s_start[lane] = start;
-        s_pref[lane] = inc - cnt;  // exclusive offset; lanes past C hold total
-        __syncwarp();
-        for (int t0 = 0; t0 < total; t0 += 32) {
-            const int t = t0 + lane;
-            const bool valid = t < total;
-            int j = -1;
-            if (valid) {
-                int k = 0;  // last cell whose offset is <= t
-#pragma unroll
-                for (int step = 16; step > 0; step >>= 1)
-                    if (s_pref[k + step] <= t) k += step;
-                j = s_start[k] + (t - s_pref[k]);
+        const FlatCells F(cnt, start, delta);
+        int jn = F.total > 0 ? F.slot(0, F.total, delta) : -1;
+        float4 fn = jn >= 0 ? __ldg(&fpos[jn]) : make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int t0 = 0; t0 < F.total; t0 += 32) {
+            const int j = jn;
+            const float4 f = fn;
+            if (t0 + 32 < F.total) {
+                jn = F.slot(t0 + 32, F.total, delta);
+                if (jn >= 0) fn = __ldg(&fpos[jn]);
             }
-            chunk(valid, j);
+            chunk(j >= 0, j, f);
         }
+        __syncwarp();
+    }
+}
+
+// A cluster of a warp's lanes (the first remaining lane and every remaining
+// lane whose cell is within one cell of it: a warp whose particles straddle a
+// jump of the Morton curve searches two compact boxes instead of one spanning
+// both places): the box around its particles, with centre o and half extents
+// e, the largest reach Rm of its lanes, and the cells within reach of the box.
+struct Cluster {
+    float x0, x1, y0, y1, z0, z1;  // the box (z in the first lane's periodic image)
+    float ox, oy, oz, ex, ey, ez;
+    float Rm, reach, L;  // reach: of the box, with slop; L >= |p|, |q| from the centre
+    float D;             // bound on the norm of (q - p) in floats minus in FP64
+    int kx0, ky0, kz0, nxr, nyr, C;
+    bool ok, wraps, zgap;
+};
+
+// mine: the lanes of the cluster; z in the image of its first lane; Rq >= 2 h
+// of the lane's search (widened, reach_f32).
+// Per component q - p differs from its FP64 value by u |x| (u = 2^-24) from
+// each conversion to float, u L from each subtraction of the centre, and along
+// z, where the box's reach crosses the end of a periodic axis (wraps), the
+// shifts of both by lz: u (|x| + lz) and the error of lz as a float each.
+__device__ __forceinline__ Cluster make_cluster(bool mine, float x, float y, float z, float Rq,
+                                                const Grid* __restrict__ g) {
+    Cluster K;
+    const float inf = CUDART_INF_F;
+    const bool per = g->periodic_z != 0;
+    const float lzf = g->lzf, hlz = g->halflzf;
+    const float sl = fmaxf(g->slop[0], fmaxf(g->slop[1], g->slop[2]));
+    K.x0 = wmin(mine ? x : inf);
+    K.x1 = wmax(mine ? x : -inf);
+    K.y0 = wmin(mine ? y : inf);
+    K.y1 = wmax(mine ? y : -inf);
+    K.z0 = wmin(mine ? z : inf);
+    K.z1 = wmax(mine ? z : -inf);
+    K.Rm = wmax(mine ? Rq : 0.0f);
+    K.ox = 0.5f * K.x0 + 0.5f * K.x1;
+    K.oy = 0.5f * K.y0 + 0.5f * K.y1;
+    K.oz = 0.5f * K.z0 + 0.5f * K.z1;
+    K.ex = fmaxf(K.x1 - K.ox, K.ox - K.x0);
+    K.ey = fmaxf(K.y1 - K.oy, K.oy - K.y0);
+    K.ez = fmaxf(K.z1 - K.oz, K.oz - K.z0);
+    K.reach = (K.Rm + sl) * 1.0001f;
+    K.L = sqrtf(fmaf(K.ez, K.ez, fmaf(K.ey, K.ey, K.ex * K.ex))) * 1.0001f + K.reach;
+    // Not ok: scales whose squares leave the normal floats, and a periodic
+    // axis so short that a candidate within reach of a lane might not be at its
+    // image nearest the centre (R + ez < lz/2 is needed), or that the wrap could
+    // decide differently in FP32 (R > lz/4).
+    K.ok = K.L < 4.0e18f && K.Rm > 1.0e-15f &&
+           !(per && (K.Rm > 0.25f * lzf || K.Rm + K.ez > 0.49f * lzf));
+    K.wraps = per && (K.z0 - K.reach < -hlz || K.z1 + K.reach > hlz);
+    const float dxy = 1.2e-7f * (g->Xf + K.L);
+    const float dz = dxy + (K.wraps ? 1.2e-7f * (g->Xf + lzf) + 2.0f * g->lzerr : 0.0f);
+    K.D = sqrtf(fmaf(dz, dz, 2.0f * dxy * dxy)) * 1.0001f;
+    int kx1, ky1, kz1;
+    box_range(K.x0 - K.Rm, K.x1 + K.Rm, g, 0, K.kx0, kx1);
+    box_range(K.y0 - K.Rm, K.y1 + K.Rm, g, 1, K.ky0, ky1);
+    box_range(K.z0 - K.Rm, K.z1 + K.Rm, g, 2, K.kz0, kz1);
+    K.nxr = kx1 - K.kx0 + 1;
+    K.nyr = ky1 - K.ky0 + 1;
+    const int nzr = kz1 - K.kz0 + 1;
+    K.C = K.nxr > 0 && K.nyr > 0 && nzr > 0 ? K.nxr * K.nyr * nzr : 0;
+    K.zgap = !per || nzr < g->n[2];  // (the whole periodic axis: no distance along z)
+    return K;
+}
+
+// Particles of cell c of the cluster's range, 0 if the cell is out of its reach.
+__device__ __forceinline__ int cluster_cell(const Cluster& K, const Grid* __restrict__ g,
+                                            const int2* __restrict__ cells, int c, int& start) {
+    start = 0;
+    if (c >= K.C) return 0;
+    const int kx = K.kx0 + c % K.nxr, rr = c / K.nxr;
+    const int ky = K.ky0 + rr % K.nyr, kz = K.kz0 + rr / K.nyr;
+    const int cz = g->periodic_z ? wrapi(kz, g->n[2]) : kz;
+    const int2 se = __ldg(&cells[((long long)cz * g->n[1] + ky) * g->n[0] + kx]);
+    start = se.x;
+    auto gap = [&](int k, int d, float v0, float v1) {
+        const float c0 = g->lof[d] + (float)k * g->wf[d] - g->slop[d];
+        const float c1 = g->lof[d] + (float)(k + 1) * g->wf[d] + g->slop[d];
+        return fmaxf(0.0f, fmaxf(c0 - v1, v0 - c1));
+    };
+    const float gx = gap(kx, 0, K.x0, K.x1), gy = gap(ky, 1, K.y0, K.y1);
+    const float gz = K.zgap ? gap(kz, 2, K.z0, K.z1) : 0.0f;
+    return fmaf(gz, gz, fmaf(gy, gy, gx * gx)) < K.Rm * K.Rm ? max(se.y - se.x, 0) : 0;
+}
+
+// The places [first, last) of the cluster's flat list of candidates, 32 at a
+// time: f(ok, q, j) is called by all lanes together, lane l with candidate j at
+// q from the centre (q.w = |q|^2), ok when it lies within reach of the box. The
+// next candidates load while these are worked on.
+template <class F>
+__device__ __forceinline__ void cluster_walk(const Cluster& K, const Grid* __restrict__ g,
+                                             const int2* __restrict__ cells,
+                                             const float4* __restrict__ fpos, int* delta,
+                                             int first, int last, F&& f) {
+    const int lane = threadIdx.x & 31;
+    const float lzf = g->lzf, hlz = g->halflzf;
+    int seen = 0;  // candidates before this batch of cells
+    for (int c0 = 0; c0 < K.C; c0 += 32) {
+        int start;
+        const int num = cluster_cell(K, g, cells, c0 + lane, start);
+        const FlatCells cl(num, start, delta);
+        const int ta = max(first - seen, 0), tb = min(last - seen, cl.total);
+        int jn = ta < tb ? cl.slot(ta, tb, delta) : -1;
+        float4 qn = jn >= 0 ? __ldg(&fpos[jn]) : make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int t0 = ta; t0 < tb; t0 += 32) {
+            const int j = jn;
+            float4 q = qn;
+            if (t0 + 32 < tb) {
+                jn = cl.slot(t0 + 32, tb, delta);
+                if (jn >= 0) qn = __ldg(&fpos[jn]);
+            }
+            if (K.wraps) {
+                const float d = q.z - K.oz;
+                if (d > hlz) q.z -= lzf;
+                else if (d < -hlz) q.z += lzf;
+            }
+            q.x -= K.ox;
+            q.y -= K.oy;
+            q.z -= K.oz;
+            const float gx = fmaxf(fabsf(q.x) - K.ex, 0.0f), gy = fmaxf(fabsf(q.y) - K.ey, 0.0f);
+            const float gz = fmaxf(fabsf(q.z) - K.ez, 0.0f);
+            const bool ok = j >= 0 && fmaf(gz, gz, fmaf(gy, gy, gx * gx)) <= K.reach * K.reach;
+            q.w = fmaf(q.z, q.z, fmaf(q.y, q.y, q.x * q.x));
+            f(ok, q, j);
+        }
+        seen += cl.total;
         __syncwarp();
     }
 }
@@ -407,8 +559,9 @@ __device__ int count_records(const int2* recb, int nrec, double hh, const Grid* 
 }
 
 // The 32 particles i0 .. i0 + 31 (one per lane; all of one instance).
-// LISTS: the batch has instances with candidate lists (else their code is
-// compiled out).
+// LISTS: the batch has instances with candidate lists; the search starts here.
+// Else k_h_count has made the first count, and the lanes with hs_it > 0 go on
+// from the bracket it left.
 template <bool LISTS>
 __device__ __forceinline__ void union_group(
     int64_t i0, int64_t n, const Batch& B, double4_32a* posh, const float4* __restrict__ fpos,
@@ -439,6 +592,15 @@ __device__ __forceinline__ void union_group(
     const int defer = kp.defer_lanes;
     int cnt = 0, it = 0;
     bool active = geo && max_it > 0, conv = false, deferred = false;
+    if (!LISTS) {
+        it = valid ? hs_it[i] : -1;
+        active = it > 0;
+        if (active) {
+            lo = hs_lo[i];
+            hi = hs_hi[i];
+        }
+    }
+    const bool entered = LISTS || active;
     int32_t* slab = rslab + (valid ? i : 0) * kRSlab;
     const bool per = g->periodic_z != 0;
     const int nx = g->n[0], ny = g->n[1], nz = g->n[2];
@@ -462,7 +624,7 @@ __device__ __forceinline__ void union_group(
         listed = true;
         active = false;
     }
-    for (int pass = 0;; ++pass) {  // pass is warp-uniform; it (per lane) stops at convergence
+    for (int pass = LISTS ? 0 : 1;; ++pass) {  // warp-uniform; it (per lane) stops at convergence
         const unsigned am = __ballot_sync(kFull, active);
         if (!am) break;
         // Pass 0 counts N_i(h). Later passes record every candidate within 2 hs,
@@ -662,6 +824,7 @@ __device__ __forceinline__ void union_group(
             if (!active) count_records(recb, nrec, h, g, posh, i, slab, cbase);  // N_i(final h)
         }
     }
+    if (!entered) return;
     if (!valid) {
         if (inb) {  // empty slot: empty row
             nnb[i] = 0;
@@ -752,6 +915,354 @@ k_h_lists(int64_t n, Batch B, double4_32a* posh, const float4* __restrict__ fpos
     }
 }
 
+// ------------------------------------------------------------ first count
+// The first count of every particle (without candidate lists): N_i(h) at the
+// h the particle comes with, which is the last one needed for ~98% of the
+// particles of a running simulation. One block of W warps per 32 consecutive
+// (Morton-sorted) particles, one lane per particle in every warp; the
+// candidates of a cluster of lanes (as in union_group) are split between the
+// W warps in W contiguous parts.
+//
+// A warp takes the cells around the cluster 32 at a time (one per lane), lists
+// their particles flat, 32 at a time, and keeps those within reach of the box
+// around the cluster's particles. Every lane tests every kept candidate: with
+// positions q, p relative to the box's centre, the sign of
+//     d = |q|^2 - 2 p.q + (|p|^2 - t)        (one addition, three FMAs)
+// tells r^2 < t, t the middle of the FP32 thresholds of (2h)^2; a neighbour is
+// appended to the lane's column in shared memory. A chunk of 32 candidates
+// whose smallest |d| is within the band w, a bound on every rounding of d
+// (below), is done again with the candidates in the band decided by the
+// defining FP64 test: the sets are exact. The columns go to the rows four
+// entries at a time, in the order of the candidates, which does not depend on
+// W.
+//
+// Bound: instruction issue. Against testing, collecting bits and appending bit
+// by bit in one loop (the record passes of k_h_union), a candidate costs ~10
+// instead of ~16 instructions, the appends do not diverge chunk by chunk, and
+// a row takes a quarter of the stores. Measured (ncu, a steady step): 17.6k
+// warp instructions a group on the 70^3 patch (24.7k before); 1M patch 641 us
+// (940), 1M sphere 848 us (1,227), 8,191-particle sphere 46 us (232). Tried:
+// sign bits of a chunk shifted into a word and walked bit by bit at the end
+// (825 us: the walk diverges); columns of 96 or 128 entries with 16-bit places
+// and 16 to 22 warps resident (701 to 757 us; more warps beat fewer writes).
+//
+// The band. With D the bound of make_cluster on the float error of q - p, T_out
+// = (2h + D)^2 rounded up and T_in = (2h - D)^2 rounded down, |q - p|^2 >= T_out
+// is out and < T_in is in. d rounds by at most u (21 L^2 + 8 t) (|q|^2: 3 L^2;
+// |p|^2 - t: 4 L^2 + 4 t; the sum: 2 L^2 + t; the FMAs: 3 (4 L^2 + t)), so with t
+// the middle of T_in and T_out, w = half their difference plus that.
+// Per warp, for W warps: chunks of 32 candidates kept, entries of a column.
+template <int W>
+constexpr int kCountChunks = W == 1 || W == 8 ? 8 : (W == 2 ? 24 : 16);
+template <int W>
+constexpr int kCountCap = W == 1 ? 96 : kGSlab;
+constexpr int kCountWarps = 28;  // W = 1: resident warps per SM
+
+// (the places of 256 candidates fit a byte)
+template <int W>
+using CountPlace = typename std::conditional<(kCountChunks<W> <= 8), uint8_t, uint16_t>::type;
+
+template <int W>
+struct CountSmem {  // per warp
+    float4 st[32];                        // the chunk being filled: q and |q|^2
+    int idx[kCountChunks<W> * 32];        // the candidates kept
+    int delta[32];                        // cells of the walk: first slot - place in the list
+    int self[32];                         // place in the open chunk of particle i0 + l
+    CountPlace<W> col[kCountCap<W>][32];  // per lane: its neighbours' places in idx
+};
+
+template <int W>
+__global__ void __launch_bounds__(32 * W, W == 1 ? kCountWarps : 16 / W)
+k_h_count(int64_t n, Batch B, double4_32a* posh, const float4* __restrict__ fpos,
+          const int2* __restrict__ cells, int32_t* __restrict__ nnb, int32_t* __restrict__ ngather,
+          int32_t* __restrict__ rslab, double* __restrict__ hs_lo, double* __restrict__ hs_hi,
+          int32_t* __restrict__ hs_it, int32_t* __restrict__ wl, int32_t* __restrict__ gwl,
+          unsigned* __restrict__ status, unsigned long long* __restrict__ wctr) {
+    constexpr int kCh = kCountChunks<W>, kCap = kCountCap<W>;
+    __shared__ CountSmem<W> s_w[W];
+    __shared__ int s_cnt[W][32];
+    const int lane = threadIdx.x & 31, warp = W > 1 ? (int)(threadIdx.x >> 5) : 0;
+    CountSmem<W>& S = s_w[warp];
+    const int64_t i0 = (int64_t)blockIdx.x * 32, i = i0 + lane;
+    const int inst = slot_inst(B, i0);
+    const Grid* __restrict__ g = B.grid + inst;
+    const KParams& kp = B.kp[inst];
+    cells += g->cbase;
+    const bool inb = i < n;
+    const bool valid = inb && slot_real(B, inst, i);
+    float4 fi = make_float4(0.f, 0.f, 0.f, 0.f);
+    double h = 1.0, lo = 0.0, hi = CUDART_INF;
+    if (valid) {
+        h = posh[i].w;
+        fi = fpos[i];
+    }
+    // a particle outside the geometry range (reported by the bounding box)
+    // does not search: no neighbours, h unchanged
+    const bool geo = valid && isfinite(fi.x) && isfinite(fi.y) && isfinite(fi.z) && h_ok(h);
+    const int max_it = kp.max_h_iter;
+    bool active = geo && max_it > 0;  // still searching
+    bool conv = false, handed = false;
+    int cnt = 0, it = 0;
+    int32_t* row = rslab + (valid ? i : 0) * kRSlab;
+    const bool per = g->periodic_z != 0;
+    const float lzf = g->lzf, hlz = g->halflzf;
+    const int nz = g->n[2];
+    const unsigned lt = (1u << lane) - 1u;
+    const int i0s = (int)i0;
+    const int mcx = lane_cell(fi.x, g, 0), mcy = lane_cell(fi.y, g, 1), mcz = lane_cell(fi.z, g, 2);
+    const float Rq = active ? reach_f32(h) : 0.0f;
+    unsigned todo = __ballot_sync(kFull, active);
+    while (todo) {  // clusters of lanes, as in union_group
+        const int a = __ffs(todo) - 1;
+        const int acx = __shfl_sync(kFull, mcx, a), acy = __shfl_sync(kFull, mcy, a);
+        const int acz = __shfl_sync(kFull, mcz, a);
+        const float fza = __shfl_sync(kFull, fi.z, a);
+        int dzc = abs(mcz - acz);
+        if (per) dzc = min(dzc, nz - dzc);
+        const bool mine = ((todo >> lane) & 1u) && abs(mcx - acx) <= 1 && abs(mcy - acy) <= 1 &&
+                          dzc <= 1;
+        todo &= ~__ballot_sync(kFull, mine);
+        // z in the periodic image of the first lane
+        float pz = fi.z;
+        if (per) {
+            const float d = pz - fza;
+            if (d > hlz) pz -= lzf;
+            else if (d < -hlz) pz += lzf;
+        }
+        const Cluster K = make_cluster(mine, fi.x, fi.y, pz, Rq, g);
+        if (!K.ok) {
+            if (mine) {
+                handed = true;
+                active = false;
+            }
+            continue;
+        }
+        float ax = 0.0f, ay = 0.0f, az = 0.0f, b = 1.0e38f, w = -1.0f;  // (finds nothing)
+        if (mine) {
+            const float px = fi.x - K.ox, py = fi.y - K.oy, pzr = pz - K.oz;
+            float Rl, Rh;
+            f32_bounds(2.0 * h, Rl, Rh);
+            const float ro = __fadd_ru(__fmul_ru(Rh, 1.00000024f), K.D);
+            const float ri = __fsub_rd(__fmul_rd(Rl, 0.99999976f), K.D);
+            const float To = __fmul_ru(__fmul_ru(ro, ro), 1.0000003f);
+            const float Ti = ri > 0.0f ? __fmul_rd(__fmul_rd(ri, ri), 0.9999997f) : -To;
+            const float t = 0.5f * (Ti + To);
+            ax = -2.0f * px;
+            ay = -2.0f * py;
+            az = -2.0f * pzr;
+            b = fmaf(pzr, pzr, fmaf(py, py, px * px)) - t;
+            w = 0.50001f * (To - Ti) + 1.3e-6f * (K.L * K.L) + 6.0e-7f * To;
+        }
+        int flat = 0;  // W > 1: length of the flat list
+        if (W > 1) {
+            for (int c0 = 0; c0 < K.C; c0 += 32) {
+                int st;
+                flat += cluster_cell(K, g, cells, c0 + lane, st);
+            }
+            flat = __reduce_add_sync(kFull, flat);
+        }
+        int nch = 0, fill = 0;  // chunks kept, candidates in the open one
+        int e = 0;              // entries of this lane's column (past kCap: only counted)
+        int written = 0;        // entries written to the row
+        bool own = false;       // the open chunk holds some of the 32 particles themselves
+        constexpr unsigned kRow = sizeof S.col[0];
+        const unsigned col0 = (unsigned)__cvta_generic_to_shared(&S.col[0][lane]);
+        // test the open chunk (its slots past `count` padded) and close it
+        auto close = [&](int count) {
+            const int id = nch * 32;
+            if (lane >= count) {
+                S.st[lane] = make_float4(0.0f, 0.0f, 0.0f, 3.0e38f);
+                S.idx[id + lane] = -1;
+            }
+            __syncwarp();
+            bool again = own || (W > 1 && __any_sync(kFull, e > kCap - 32));
+            if (!again) {
+                float mn = CUDART_INF_F;
+                unsigned at = col0 + (unsigned)e * kRow;
+#pragma unroll
+                for (int k0 = 0; k0 < 32; k0 += 8) {  // eight tests in flight, then their appends
+                    float d[8];
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) {
+                        const float4 q = S.st[k0 + k];
+                        d[k] = fmaf(az, q.z, fmaf(ay, q.y, fmaf(ax, q.x, q.w + b)));
+                    }
+#pragma unroll
+                    for (int k = 0; k < 8; k += 2) mn = fminf(mn, fminf(fabsf(d[k]), fabsf(d[k + 1])));
+                    // (predicated instructions: left to the compiler, each was a branch)
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) {
+                        if (sizeof(CountPlace<W>) == 2)
+                            asm volatile("{.reg .pred p; setp.lt.f32 p, %1, 0f00000000;\n\t"
+                                         "@p st.shared.u16 [%0], %2;\n\t@p add.u32 %0, %0, %3;}"
+                                         : "+r"(at) : "f"(d[k]), "r"(id + k0 + k), "n"(kRow));
+                        else
+                            asm volatile("{.reg .pred p; setp.lt.f32 p, %1, 0f00000000;\n\t"
+                                         "@p st.shared.u8 [%0], %2;\n\t@p add.u32 %0, %0, %3;}"
+                                         : "+r"(at) : "f"(d[k]), "r"(id + k0 + k), "n"(kRow));
+                    }
+                }
+                again = __any_sync(kFull, !(mn > w));  // a candidate in some lane's band
+                if (!again) e = (int)((at - col0) / kRow);
+            }
+            if (again) {
+                // the signs of d and of |d| - w as bits (candidate k: bit 31 - k); the
+                // band decided in FP64, the particle itself taken out, the rest appended
+                unsigned in = 0u, bd = 0u;
+#pragma unroll
+                for (int k = 0; k < 32; ++k) {
+                    const float4 q = S.st[k];
+                    const float d = fmaf(az, q.z, fmaf(ay, q.y, fmaf(ax, q.x, q.w + b)));
+                    in = __funnelshift_l((unsigned)__float_as_int(d), in, 1);
+                    bd = __funnelshift_l((unsigned)__float_as_int(fabsf(d) - w), bd, 1);
+                }
+                S.self[lane] = 32;
+                __syncwarp();
+                const int js = S.idx[id + lane];
+                if (js >= 0 && (unsigned)(js - i0s) < 32u) S.self[js - i0s] = lane;
+                __syncwarp();
+                while (bd) {
+                    const int k = __clz((int)bd);
+                    const unsigned bit = 0x80000000u >> k;
+                    bd ^= bit;
+                    const double R = 2.0 * h;
+                    if (exact_r2(posh[i], posh[S.idx[id + k]], g) < __dmul_rn(R, R)) in |= bit;
+                    else in &= ~bit;
+                }
+                const int sp = S.self[lane];
+                if (sp < 32) in &= ~(0x80000000u >> sp);
+                if (!mine) in = 0u;
+                while (in) {
+                    const int k = __clz((int)in);
+                    in ^= 0x80000000u >> k;
+                    if (W == 1 || e < kCap) S.col[e][lane] = (CountPlace<W>)(id + k);
+                    ++e;
+                }
+            }
+            ++nch;
+            own = false;
+            __syncwarp();
+        };
+        // the first `num` entries of the column to entries from, from + 1, ... of the row
+        auto put = [&](int from, int num) {
+            auto entry = [&](int p) { return S.idx[S.col[p][lane]]; };
+            int p = 0;
+            for (const int head = min((4 - (from & 3)) & 3, num); p < head; ++p)
+                if (from + p < kGSlab) row[from + p] = entry(p);
+            for (; p + 4 <= num; p += 4) {
+                const int4 v = make_int4(entry(p), entry(p + 1), entry(p + 2), entry(p + 3));
+                if (from + p + 4 <= kGSlab) *reinterpret_cast<int4*>(row + from + p) = v;
+            }
+            for (; p < num; ++p)
+                if (from + p < kGSlab) row[from + p] = entry(p);
+        };
+        // One warp takes the whole list. Several take it in rounds of at most
+        // as many candidates as they can keep, each warp a contiguous part of
+        // the round; all but the last round write their entries at once (a row
+        // holds kGSlab gather entries, so a column needs no more).
+        constexpr int kRound = W * kCh * 32;
+        for (int base = 0;; base += kRound) {
+            const bool final_round = W == 1 || base + kRound >= flat;
+            int first = 0, last = 0x7fffffff;  // this warp's part of the flat list
+            if (W > 1) {
+                const int len = min(kRound, flat - base);
+                first = base + len * warp / W;
+                last = base + len * (warp + 1) / W;
+                e = nch = fill = 0;
+            }
+            cluster_walk(K, g, cells, fpos, S.delta, first, last, [&](bool ok, const float4& q, int j) {
+                const unsigned m = __ballot_sync(kFull, ok);
+                if (!m) return;
+                const int r = __popc(m & lt), room = 32 - fill, got = __popc(m);
+                const bool self = ok && (unsigned)(j - i0s) < 32u;
+                if (ok && r < room) {
+                    S.st[fill + r] = q;
+                    S.idx[nch * 32 + fill + r] = j;
+                }
+                own = own || __any_sync(kFull, self && r < room);
+                if (got < room) {
+                    fill += got;
+                    return;
+                }
+                close(32);
+                // (a round of several warps has no more than they keep)
+                if (W == 1 && (nch == kCh || __any_sync(kFull, e > kCap - 32))) {
+                    put(written, e);
+                    written += e;
+                    e = nch = 0;
+                    __syncwarp();
+                }
+                if (ok && r >= room) {
+                    S.st[r - room] = q;
+                    S.idx[nch * 32 + r - room] = j;
+                }
+                own = __any_sync(kFull, self && r >= room);
+                fill = got - room;
+            });
+            if (fill > 0) close(fill);
+            int tot = written + e, from = written;
+            if (W > 1) {
+                s_cnt[warp][lane] = e;
+                __syncthreads();
+                tot = written;
+#pragma unroll
+                for (int v = 0; v < W; ++v) {
+                    if (v == warp) from = tot;
+                    tot += s_cnt[v][lane];
+                }
+            }
+            if (mine && final_round) {
+                cnt = tot;
+                it = 1;
+                if (cnt >= kp.n_target - kp.n_tol && cnt <= kp.n_target + kp.n_tol) {
+                    conv = true;
+                    active = false;
+                } else if (it >= max_it) {
+                    active = false;
+                } else if (cnt < kp.n_target - kp.n_tol) {
+                    lo = h;
+                    h = __dmul_rn(h, 1.25);  // no upper bound yet
+                } else {
+                    hi = h;
+                    h = __dmul_rn(h, 0.8);  // no lower bound yet
+                }
+            }
+            if (mine && !(final_round && active)) put(from, W == 1 ? e : min(e, kCap));
+            if (W > 1) __syncthreads();  // the counts and the columns are reused
+            else __syncwarp();
+            if (final_round) break;
+            written = tot;
+        }
+    }
+    if (warp != 0) return;
+    // searches to go on with: few in a warp, or of a small instance, one warp
+    // each (k_h_iterate); else the group together (k_h_union)
+    const unsigned am = __ballot_sync(kFull, active);
+    const bool few = __popc(am) <= kp.defer_lanes || __ldg(&B.icnt[inst]) < kGroupSearchN;
+    if (handed || active) {
+        posh[i].w = h;
+        hs_lo[i] = lo;
+        hs_hi[i] = hi;
+        if (handed || few) {
+            hs_it[i] = it;
+            wl[atomicAdd(&status[3], 1u)] = (int32_t)i;
+        }
+    }
+    if (!few) {
+        if (inb && !handed) hs_it[i] = active ? it : -1;
+        if (lane == 0) gwl[atomicAdd(&wctr[1], 1ull)] = (int32_t)blockIdx.x;
+    }
+    if (!inb || handed || active) return;
+    nnb[i] = cnt;
+    ngather[i] = cnt;
+    if (!valid) return;
+    if (cnt > kGSlab) atomicOr(&status[2], (unsigned)IF_SLAB_OVF);
+    if (!conv) {
+        atomicOr(&status[0], (unsigned)ST_HNOCONV);
+        atomicAdd(&status[1], 1u);
+    }
+}
+
 // Persistent: warps take groups of 32 particles from a counter, so a group
 // whose particles straddle far-apart cells (a jump of the Morton curve: a
 // large query box, many candidates) delays one warp, not a whole wave.
@@ -764,17 +1275,18 @@ k_h_union(int64_t n, Batch B, double4_32a* posh, const float4* __restrict__ fpos
           int32_t* __restrict__ wl, unsigned* __restrict__ status,
           unsigned long long* __restrict__ wctr, int2* __restrict__ recs,
           const int32_t* __restrict__ order, int32_t* __restrict__ lst,
-          LMeta* __restrict__ lmeta) {
+          LMeta* __restrict__ lmeta, const int32_t* __restrict__ gwl) {
     __shared__ float4 s_f[kThreads / 32][32];
     __shared__ int s_i[kThreads / 32][32];
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
-    const long long ngroups = (n + 31) / 32;
+    const long long ngroups = LISTS ? (n + 31) / 32 : (long long)wctr[1];
     for (;;) {
         long long gi = 0;
         if (lane == 0) gi = (long long)atomicAdd(wctr, 1ull);
         gi = __shfl_sync(kFull, gi, 0);
         if (gi >= ngroups) break;
+        if (!LISTS) gi = gwl[gi];
         union_group<LISTS>(gi * 32, n, B, posh, fpos, cells, nnb, ngather, rslab, hs_lo, hs_hi, hs_it,
                     wl, status, s_f[warp], s_i[warp],
                     recs + ((int64_t)(blockIdx.x * (kThreads / 32) + warp) * 32 + lane) * kRec,
@@ -783,31 +1295,55 @@ k_h_union(int64_t n, Batch B, double4_32a* posh, const float4* __restrict__ fpos
 }
 
 // The candidates of a list (ln entries 32 apart from L on), 32 at a time:
-// chunk(valid, j) is called by all lanes together, lane l receiving entry
+// chunk(valid, j, f) is called by all lanes together, lane l receiving entry
 // e0 + l (valid = false past the end), as particle_pass hands out a walk's.
 template <class Chunk>
-__device__ __forceinline__ void list_pass(const int32_t* __restrict__ L, int ln, Chunk&& chunk) {
+__device__ __forceinline__ void list_pass(const int32_t* __restrict__ L, int ln,
+                                          const float4* __restrict__ fpos, Chunk&& chunk) {
     const int lane = threadIdx.x & 31;
     for (int e0 = 0; e0 < ln; e0 += 32) {
         const int e = e0 + lane;
-        const bool valid = e < ln;
-        chunk(valid, valid ? __ldg(&L[e * 32]) : -1);
+        const int j = e < ln ? __ldg(&L[e * 32]) : -1;
+        chunk(j >= 0, j, j >= 0 ? __ldg(&fpos[j]) : make_float4(0.f, 0.f, 0.f, 0.f));
     }
 }
 
-// Phase 2: one warp per handed-over particle (persistent grid over the
-// worklist), continuing its bisection where phase 1 stopped. A walk over the
-// cells records, in shared memory and in walk order, every candidate that may
-// lie within 2 hs, hs = the largest h the bisection can still test without a
-// new walk (hi once bracketed; 1.25 h, the next growth step, before); the
-// counts at every h <= hs then come from the records with the same FP32 /
-// exact FP64 decisions as a walk, and the gather set is written in the order
-// a walk at h would find it. Only growth beyond hs (or more candidates than
-// the record buffer holds) walks the cells again.
+// One warp per particle that goes on searching (persistent grid over the
+// worklist), from the bracket its first count left. hs, the largest h the
+// bisection can still test without growing (hi once bracketed; before, h, or
+// 1.25 h for a first count), bounds the counts: one walk over the cells writes
+// the candidates certainly within 2 lo to the row and records those that may
+// lie within 2 hs in shared memory; the counts at every h <= hs come from the
+// records, with a walk's FP32 / exact FP64 decisions. Every bracket update
+// takes records out: those within 2 lo join the row, those beyond 2 hi are
+// dropped; 32 or fewer are held one per lane. Only growth beyond hs walks the
+// cells again, and more candidates than the buffer holds are counted by
+// walking. Bound: issue (72% in a first step) and, with one particle per warp
+// in flight, latency (issue 52% in a steady step). Measured: a steady step of
+// the 1M patch 144 us (293 when the records kept everything within 1.25 times
+// the next h and the row was written with every count), 27,000 particles from a
+// poor h 172 us (300).
 constexpr int kRecW = 512;  // records per warp
 
+// h / 2 and 2 h of a normal h by its exponent (exact; no FP64 pipe, which
+// serves one warp instruction in 16 cycles an SM)
+__device__ __forceinline__ double scale_exp(double v, int e) {
+    return __longlong_as_double(__double_as_longlong(v) + ((long long)e << 52));
+}
+
+// non-negative doubles order like their bits
+__device__ __forceinline__ long long dbits(double v) { return __double_as_longlong(v); }
+constexpr long long kInfBits = 0x7ff0000000000000LL;
+constexpr long long kTinyBits = 0x0020000000000000LL;  // 2^-1021: halves and doubles are normal
+
+// (a + b) / 2, both operations rounded
+__device__ __forceinline__ double half_sum(double a, double b) {
+    const double s = __dadd_rn(a, b);
+    return dbits(s) > kTinyBits && dbits(s) < kInfBits ? scale_exp(s, -1) : __dmul_rn(0.5, s);
+}
+
 template <bool LISTS>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, 4)
 k_h_iterate(Batch B, double4_32a* posh, const float4* __restrict__ fpos,
             const int2* __restrict__ cells,
             int32_t* __restrict__ nnb, int32_t* __restrict__ ngather,
@@ -816,7 +1352,7 @@ k_h_iterate(Batch B, double4_32a* posh, const float4* __restrict__ fpos,
             const int32_t* __restrict__ wl, unsigned* __restrict__ status,
             const int32_t* __restrict__ order, const int32_t* __restrict__ lst,
             const LMeta* __restrict__ lmeta) {
-    __shared__ int s_start[kThreads / 32][32], s_pref[kThreads / 32][32];
+    __shared__ int s_delta[kThreads / 32][32];
     __shared__ int2 s_rec[kThreads / 32][kRecW];  // (FP32 r^2 bits, j)
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
@@ -825,21 +1361,23 @@ k_h_iterate(Batch B, double4_32a* posh, const float4* __restrict__ fpos,
     const unsigned lt = (1u << lane) - 1u;
     int2* rec = s_rec[warp];
     for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < count; w += nwarps) {
-        const int64_t i = wl[w];
+        const int i = wl[w];
         const int inst = slot_inst(B, i);
         const Grid* __restrict__ g = B.grid + inst;
         const KParams& kp = B.kp[inst];
         const int2* __restrict__ cl = cells + g->cbase;
         const int lowb = kp.n_target - kp.n_tol, highb = kp.n_target + kp.n_tol;
         const int max_it = kp.max_h_iter;
-        const double4_32a pi = posh[i];
         const float4 fi = fpos[i];
-        double h = pi.w, lo = hs_lo[i], hi = hs_hi[i];
+        double h = posh[i].w, lo = hs_lo[i], hi = hs_hi[i];
         int cnt = 0;
         bool conv = false;
-        int32_t* slab = rslab + i * kRSlab;
-        double hs = -1.0;  // radius / 2 the records cover (none yet)
-        int nrec = 0;
+        int32_t* slab = rslab + (int64_t)i * kRSlab;
+        long long hsb = -1;  // bits of hs, radius / 2 the records cover (-1: none)
+        int nrec = 0;      // records: in shared memory, or one per lane (in_regs)
+        int base = 0;      // row entries: certain neighbours at every h still to come
+        bool in_regs = false;
+        int2 own = make_int2(0x7f800000, -1);  // this lane's record (in_regs): r^2 = inf if none
         // the particle's kept candidate list, while it covers a radius 2 hq
         // (then it replaces the cell walk: the same candidates within 2 hq)
         const bool lists = LISTS && kp.list_skin > 0.0 && !g->lbuild;
@@ -847,95 +1385,110 @@ k_h_iterate(Batch B, double4_32a* posh, const float4* __restrict__ fpos,
         const float lrad = ln > 0 ? lmeta[order[i]].rad : 0.0f;
         const int32_t* L = lst + (i >> 5) * (int64_t)kList * 32 + (i & 31);
         auto list_covers = [&](double hq) { return ln > 0 && reach_f32(hq) + g->dm2 <= lrad; };
+        // append j of the lanes with `in` to the row after its first c entries
+        auto append = [&](bool in, int j, int c) {
+            const unsigned m = __ballot_sync(kFull, in);
+            const int q = c + __popc(m & lt);
+            if (in && q < kGSlab) slab[q] = j;
+            return __popc(m);
+        };
         for (int it = hs_it[i]; it < max_it; ++it) {
-            const double R = 2.0 * h;
+            const double R = dbits(h) > kTinyBits ? scale_exp(h, 1) : 2.0 * h;
             const Thr t = thresholds(R, g);
-            double R2 = -1.0;  // (2h)^2 in FP64, formed on first use
+            // r < 2h, decided as by a walk
+            auto within = [&](float r2f, int j) {
+                bool in = r2f < t.tin;
+                const bool bd = !in && r2f <= t.tout && j >= 0;
+                if (__any_sync(kFull, bd) && bd)
+                    in = exact_r2(posh[i], posh[j], g) < __dmul_rn(R, R);
+                return in;
+            };
             int c = 0;
-            if (!(h <= hs)) {
-                // walk the cells once more and record everything that may lie
-                // within 2 hs of the particle
-                hs = isinf(hi) ? __dmul_rn(h, 1.25) : hi;
+            unsigned bits = 0u;  // the decisions of this count: bit q / 32 of lane q % 32
+            static_assert(kRecW <= 32 * 32, "one bit per word of records");
+            if (!(dbits(h) <= hsb)) {
+                // walk the cells once more: what is certainly within 2 lo to the
+                // row, what may lie within 2 hs to the records
+                const double hs = dbits(hi) != kInfBits ? hi : (dbits(lo) > 0 ? h : __dmul_rn(h, 1.25));
+                hsb = dbits(hs);
                 const float tout_s = thresholds(2.0 * hs, g).tout;
-                nrec = 0;
-                auto record = [&](bool valid, int j) {
-                    float r2f = 0.0f;
-                    bool keep = false;
-                    if (valid && j != i) {
-                        r2f = f_r2(fi, __ldg(&fpos[j]), g);
-                        keep = r2f <= tout_s;
-                    }
+                const float tin_lo = dbits(lo) > 0 ? thresholds(2.0 * lo, g).tin : -1.0f;
+                nrec = base = 0;
+                in_regs = false;
+                auto record = [&](bool valid, int j, const float4& f) {
+                    const float r2f = valid && j != i ? f_r2(fi, f, g) : CUDART_INF_F;
+                    base += append(r2f < tin_lo, j, base);
+                    const bool keep = r2f >= tin_lo && r2f <= tout_s && valid && j != i;
                     const unsigned m = __ballot_sync(kFull, keep);
-                    if (keep) {
-                        const int q = nrec + __popc(m & lt);
-                        if (q < kRecW) rec[q] = make_int2(__float_as_int(r2f), j);
-                    }
+                    const int q = nrec + __popc(m & lt);
+                    if (keep && q < kRecW) rec[q] = make_int2(__float_as_int(r2f), j);
                     nrec += __popc(m);
                 };
-                if (list_covers(hs)) list_pass(L, ln, record);
-                else particle_pass<1>(g, cl, nullptr, fi, reach_f32(hs), 0, s_start[warp], s_pref[warp],
-                                      record);
+                if (list_covers(hs)) list_pass(L, ln, fpos, record);
+                else particle_pass<1>(g, cl, nullptr, fpos, fi, reach_f32(hs), 0, s_delta[warp], record);
                 __syncwarp();
-                if (nrec > kRecW) hs = -1.0;  // too many to keep: count by walking
+                if (nrec > kRecW) hsb = -1;  // too many to keep: count by walking
             }
-            if (h <= hs) {
-                for (int q0 = 0; q0 < nrec; q0 += 32) {
-                    const int q = q0 + lane;
-                    bool in = false, bd = false;
-                    int j = -1;
-                    if (q < nrec) {
-                        const int2 e = rec[q];
-                        const float r2f = __int_as_float(e.x);
-                        j = e.y;
-                        in = r2f < t.tin;
-                        bd = !in && r2f <= t.tout;
+            const bool kept = dbits(h) <= hsb;
+            if (kept) {
+                c = base;
+                if (!in_regs && nrec <= 32) {
+                    in_regs = true;
+                    own = lane < nrec ? rec[lane] : make_int2(0x7f800000, -1);
+                    __syncwarp();
+                }
+                if (in_regs) {
+                    bits = within(__int_as_float(own.x), own.y) ? 1u : 0u;
+                    c += __popc(__ballot_sync(kFull, bits != 0u));
+                } else {
+                    for (int q0 = 0; q0 < nrec; q0 += 32) {
+                        const int2 e = q0 + lane < nrec ? rec[q0 + lane] : make_int2(0x7f800000, -1);
+                        const bool in = within(__int_as_float(e.x), e.y);
+                        bits |= in ? 1u << (q0 >> 5) : 0u;
+                        c += __popc(__ballot_sync(kFull, in));
                     }
-                    if (__any_sync(kFull, bd) && bd) {
-                        if (R2 < 0.0) R2 = __dmul_rn(R, R);
-                        in = exact_r2(pi, posh[j], g) < R2;
-                    }
-                    const unsigned m = __ballot_sync(kFull, in);
-                    if (in) {
-                        const int qq = c + __popc(m & lt);
-                        if (qq < kGSlab) slab[qq] = j;
-                    }
-                    c += __popc(m);
                 }
             } else {
-                auto count = [&](bool valid, int j) {
-                    bool in = false, bd = false;
-                    if (valid && j != i) {
-                        const float r2f = f_r2(fi, __ldg(&fpos[j]), g);
-                        in = r2f < t.tin;
-                        bd = !in && r2f <= t.tout;
-                    }
-                    if (__any_sync(kFull, bd) && bd) {
-                        if (R2 < 0.0) R2 = __dmul_rn(R, R);
-                        in = exact_r2(pi, posh[j], g) < R2;
-                    }
-                    const unsigned m = __ballot_sync(kFull, in);
-                    if (in) {
-                        const int q = c + __popc(m & lt);
-                        if (q < kGSlab) slab[q] = j;
-                    }
-                    c += __popc(m);
+                auto walk = [&](bool valid, int j, const float4& f) {
+                    const float r2f = valid && j != i ? f_r2(fi, f, g) : CUDART_INF_F;
+                    c += append(within(r2f, valid && j != i ? j : -1) && valid && j != i, j, c);
                 };
-                if (list_covers(h)) list_pass(L, ln, count);
-                else particle_pass<1>(g, cl, nullptr, fi, reach_f32(h), 0, s_start[warp], s_pref[warp],
-                                      count);
+                if (list_covers(h)) list_pass(L, ln, fpos, walk);
+                else particle_pass<1>(g, cl, nullptr, fpos, fi, reach_f32(h), 0, s_delta[warp], walk);
             }
             cnt = c;
-            if (cnt >= lowb && cnt <= highb) {
-                conv = true;
-                break;
+            conv = cnt >= lowb && cnt <= highb;
+            const bool last = conv || it == max_it - 1, low = cnt < lowb;
+            if (kept) {
+                // members join the row when this is the last count or lo rises to h;
+                // the rest of the records stay while they lie between lo and hi
+                if (in_regs) {
+                    const bool in = bits != 0u;
+                    if (last || low) base += append(in, own.y, base);
+                    if (in == low) own = make_int2(0x7f800000, -1);
+                } else {
+                    int keep = 0;
+                    for (int q0 = 0; q0 < nrec; q0 += 32) {
+                        const int2 e = q0 + lane < nrec ? rec[q0 + lane] : make_int2(0x7f800000, -1);
+                        const bool in = (bits >> (q0 >> 5)) & 1u;
+                        if (last || low) base += append(in, e.y, base);
+                        const bool stay = in != low && e.y >= 0;
+                        const unsigned m = __ballot_sync(kFull, stay);
+                        __syncwarp();  // (keep <= q0: the places written have been read)
+                        if (stay) rec[keep + __popc(m & lt)] = e;
+                        keep += __popc(m);
+                    }
+                    nrec = keep;
+                    __syncwarp();
+                }
             }
-            if (it == max_it - 1) break;
-            if (cnt < lowb) {
+            if (last) break;
+            if (low) {
                 lo = h;
-                h = isinf(hi) ? __dmul_rn(h, 1.25) : __dmul_rn(0.5, __dadd_rn(lo, hi));
+                h = dbits(hi) == kInfBits ? __dmul_rn(h, 1.25) : half_sum(lo, hi);
             } else {
                 hi = h;
-                h = (lo == 0.0) ? __dmul_rn(h, 0.8) : __dmul_rn(0.5, __dadd_rn(lo, hi));
+                h = dbits(lo) == 0 ? __dmul_rn(h, 0.8) : half_sum(lo, hi);
             }
         }
         __syncwarp();  // the records are reused by this warp's next particle
@@ -1145,7 +1698,7 @@ k_csr(int64_t n, Batch B, const double4_32a* __restrict__ posh,
       int32_t* __restrict__ rowlen, int32_t* __restrict__ ngather,
       const int64_t* __restrict__ offsets, int32_t* __restrict__ idx, int64_t nnzcap,
       unsigned* __restrict__ status, unsigned mask) {
-    __shared__ int s_start[kThreads / 32][32], s_pref[kThreads / 32][32];
+    __shared__ int s_delta[kThreads / 32][32];
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
     if (!(status[2] & mask)) return;  // the slab path built the list
@@ -1182,11 +1735,10 @@ k_csr(int64_t n, Batch B, const double4_32a* __restrict__ posh,
         po_end = offsets[i + 1];
     }
     int cg = 0, co = 0;
-    particle_pass<2>(g, cl, chm, fi, Rbig, hib, s_start[warp], s_pref[warp],
-                        [&](bool valid, int j) {
+    particle_pass<2>(g, cl, chm, fpos, fi, Rbig, hib, s_delta[warp],
+                        [&](bool valid, int j, const float4& fj) {
         bool in_i = false, in_j = false;
         if (valid && j != i) {
-            const float4 fj = __ldg(&fpos[j]);
             const float r2f = f_r2(fi, fj, g);
             bool bd_i = false;
             if (r2f < tin_i) in_i = true;
@@ -1235,7 +1787,7 @@ void launch_h_search(sph_ctx* c, cudaStream_t s) {
     const unsigned nb = (unsigned)((n + kThreads - 1) / kThreads);
     double4_32a* posh = c->posh[c->cur];
     const Batch B = batch_of(c);
-    c->launches += 4;
+    c->launches += 4;  // the first count, k_h_iterate, k_finalize_h, k_cell_hmax
     if (c->any_lists) {
         c->launches += 1;
         k_h_lists<<<nb, kThreads, 0, s>>>(n, B, posh, c->fpos, c->nnb, c->ngather, c->rslab,
@@ -1246,14 +1798,33 @@ void launch_h_search(sph_ctx* c, cudaStream_t s) {
     if (c->any_lists) {
         k_h_union<true><<<(unsigned)nbu, kThreads, 0, s>>>(
             n, B, posh, c->fpos, c->cells, c->nnb, c->ngather, c->rslab, c->hs_lo, c->hs_hi,
-            c->hs_it, c->wl, c->status, c->wctr, c->recs, c->order[c->cur], c->lst, c->lmeta);
+            c->hs_it, c->wl, c->status, c->wctr, c->recs, c->order[c->cur], c->lst, c->lmeta, c->gwl);
         k_h_iterate<true><<<kReduceBlocks * 4, kThreads, 0, s>>>(
             B, posh, c->fpos, c->cells, c->nnb, c->ngather, c->rslab, c->hs_lo, c->hs_hi,
             c->hs_it, c->wl, c->status, c->order[c->cur], c->lst, c->lmeta);
     } else {
-        k_h_union<false><<<(unsigned)nbu, kThreads, 0, s>>>(
-            n, B, posh, c->fpos, c->cells, c->nnb, c->ngather, c->rslab, c->hs_lo, c->hs_hi,
-            c->hs_it, c->wl, c->status, c->wctr, c->recs, c->order[c->cur], c->lst, c->lmeta);
+        const int64_t groups = (n + 31) / 32;
+        auto count = [&](auto fn, int warps) {
+            fn<<<(unsigned)groups, 32 * warps, 0, s>>>(n, B, posh, c->fpos, c->cells, c->nnb,
+                                                       c->ngather, c->rslab, c->hs_lo, c->hs_hi,
+                                                       c->hs_it, c->wl, c->gwl, c->status, c->wctr);
+        };
+        // Warps per group: as many as fill the chip once. Measured (first count,
+        // us, with 8 / 4 / 2 / 1 warps): 4,096 particles 24 / 31 / 48 / 86, the
+        // 8,191-particle sphere 45 / 51 / 71 / 126, 27,000 45 / 38 / 38 / 80, 104k
+        // 174 / 129 / 122 / 118, the 200k sphere 446 / 321 / 289 / 270.
+        const int64_t room = (int64_t)c->nsm * 24;
+        if (groups * 2 > room) count(k_h_count<1>, 1);
+        else if (groups * 4 > room) count(k_h_count<2>, 2);
+        else if (groups * 8 > room) count(k_h_count<4>, 4);
+        else count(k_h_count<8>, 8);
+        if (c->group_search) {
+            c->launches += 1;
+            k_h_union<false><<<(unsigned)nbu, kThreads, 0, s>>>(
+                n, B, posh, c->fpos, c->cells, c->nnb, c->ngather, c->rslab, c->hs_lo, c->hs_hi,
+                c->hs_it, c->wl, c->status, c->wctr, c->recs, c->order[c->cur], c->lst, c->lmeta,
+                c->gwl);
+        }
         k_h_iterate<false><<<kReduceBlocks * 4, kThreads, 0, s>>>(
             B, posh, c->fpos, c->cells, c->nnb, c->ngather, c->rslab, c->hs_lo, c->hs_hi,
             c->hs_it, c->wl, c->status, c->order[c->cur], c->lst, c->lmeta);

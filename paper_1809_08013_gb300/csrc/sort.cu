@@ -390,6 +390,7 @@ k_grid_setup(const double* __restrict__ part, Batch B, Grid* __restrict__ grid,
         status[2] = 0u;
         status[3] = 0u;
         wctr[0] = 0ull;
+        wctr[1] = 0ull;
     }
     const double hmean = n > 0 ? hs / (double)n : 1.0;
     double w = 2.0 * hmean * kp.cell_scale;
@@ -470,6 +471,8 @@ k_grid_setup(const double* __restrict__ part, Batch B, Grid* __restrict__ grid,
     g->lzf = (float)lz;
     g->halflzf = (float)(0.5 * lz);
     g->X = X;
+    g->Xf = __double2float_ru(X);
+    g->lzerr = __double2float_ru(fabs(lz - (double)(float)lz));
     // |fl32 difference - FP64 difference| <= 2^-24 (4X + 2.02R + 2 lz) per
     // component (conversions of both coordinates, the FP32 subtraction, the
     // periodic shift); 1.0001 and the upward rounding keep it an upper bound

@@ -145,7 +145,7 @@ void free_all(sph_ctx* c) {
     void* ptrs[] = {c->posh[0], c->posh[1], c->velm[0], c->velm[1], c->ue[0], c->ue[1],
                     c->therm, c->kern, c->acc, c->pint, c->cint, c->dpk, c->mpk, c->mumax, c->fpos, c->tin, c->order[0],
                     c->order[1], c->keys[0], c->keys[1], c->vals[0], c->vals[1], c->hist, c->cells, c->cell_hmax, c->nnb, c->ngather, c->rowlen,
-                    c->offsets, c->row_part, c->idx, c->rslab, c->ocnt, c->hs_lo, c->hs_hi, c->hs_it, c->wl, c->red_part, c->dt_part, c->grid,
+                    c->offsets, c->row_part, c->idx, c->rslab, c->ocnt, c->hs_lo, c->hs_hi, c->hs_it, c->wl, c->gwl, c->red_part, c->dt_part, c->grid,
                     c->status, c->scratch_scalar, c->blk, c->ioff, c->icnt, c->coff, c->kpi,
                     c->tune_dt, c->roff, c->wctr, c->recs, c->iad_a, c->iad_b, c->vol, c->xpk, c->vpa, c->vpb,
                     c->stage, c->stage_nnb, c->vdf, c->cpk, c->lst, c->lmeta, c->lctr};
@@ -226,7 +226,7 @@ bool allocate_all(sph_ctx* c, int64_t nslots, Allocator& al) {
          al(&c->coff, (size_t)max_instances + 1) && al(&c->kpi, (size_t)max_instances) &&
          al(&c->roff, (size_t)max_instances + 1) &&
          al(&c->rslab, N * kRSlab) && al(&c->ocnt, N) &&
-         al(&c->hs_lo, N) && al(&c->hs_hi, N) && al(&c->hs_it, N) && al(&c->wl, N) &&
+         al(&c->hs_lo, N) && al(&c->hs_hi, N) && al(&c->hs_it, N) && al(&c->wl, N) && al(&c->gwl, (N + 31) / 32) &&
          al(&c->scratch_scalar, 2) && al(&c->tune_dt, 2 * (size_t)max_instances) &&
          al(&c->wctr, 4) &&
          al(&c->recs, (size_t)c->nsm * kUnionBlocksPerSM * kThreads * kRec);
@@ -343,6 +343,7 @@ void launch_set_single(sph_ctx* c, const KParams& kp, int64_t n, cudaStream_t s)
     const int64_t zero = 0;
     lists_for_layout(c, 1, &zero, &n, s);
     c->any_lists = kp.list_skin > 0.0;
+    c->group_search = n >= kGroupSearchN;
     c->n = n;
     c->ntot = n;
     c->cext = n;
@@ -395,8 +396,9 @@ void drop_step_graphs(sph_ctx* c) {
 // them, so the results are the same bits.
 bool step_graph(sph_ctx* c, double* dt, double* time, cudaStream_t s) {
     const int par = c->cur;
-    const int64_t key[10] = {c->n, c->ntot, c->ninst, c->prec, c->tpp, c->kern_kind, c->grad_kind,
-                             (int64_t)(intptr_t)dt, (int64_t)(intptr_t)time, c->any_lists ? 1 : 0};
+    const int64_t key[11] = {c->n, c->ntot, c->ninst, c->prec, c->tpp, c->kern_kind, c->grad_kind,
+                             (int64_t)(intptr_t)dt, (int64_t)(intptr_t)time, c->any_lists ? 1 : 0,
+                             c->group_search ? 1 : 0};
     sph_ctx::StepGraph& g = c->sg[par];
     if (!g.valid || memcmp(g.key, key, sizeof key) != 0) {
         if (g.valid) cudaGraphExecDestroy(g.exec);
@@ -1042,8 +1044,11 @@ static sph_status batch_set(sph_ctx* c, int32_t ninst, const int64_t* counts, co
     DeviceGuard dg(c->device);
     cudaStream_t s = (cudaStream_t)stream;
     lists_for_layout(c, ninst, coff.data(), icnt.data(), s);
-    c->any_lists = false;
-    for (int k = 0; k < ninst; ++k) c->any_lists = c->any_lists || kpi[k].list_skin > 0.0;
+    c->any_lists = c->group_search = false;
+    for (int k = 0; k < ninst; ++k) {
+        c->any_lists = c->any_lists || kpi[k].list_skin > 0.0;
+        c->group_search = c->group_search || icnt[k] >= kGroupSearchN;
+    }
     cudaError_t e = cudaMemcpyAsync(c->ioff, ioff.data(), (ninst + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(c->coff, coff.data(), (ninst + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(c->icnt, icnt.data(), ninst * sizeof(int64_t), cudaMemcpyHostToDevice, s);

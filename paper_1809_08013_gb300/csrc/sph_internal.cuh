@@ -101,6 +101,14 @@ enum : unsigned {
 };
 constexpr int kGSlab = 128;  // gather-set slots per particle (>= n_target + n_tol)
 constexpr int kRec = 256;    // h search: candidates recorded per lane in flight
+// Instances of at least this many particles go on with a search that many
+// lanes of a warp have not finished in groups of 32 (k_h_union), the others one
+// warp per particle (k_h_iterate): a small problem has too few groups to hide
+// the latency of one. Measured for the first step of a patch (us): 104k
+// particles 641 in groups, 645 one by one; 1M 3,934 and 6,100; below that a
+// group has the chip to itself (27,000: 172 one by one). By the instance, not the batch: the two leave a row in another order,
+// and an instance gives the same bits alone and in a batch.
+constexpr int64_t kGroupSearchN = 100000;
 constexpr int kUnionBlocksPerSM = 4;  // resident blocks of the persistent h search
 // Candidate lists of the h search, kept across steps (neighbors.cu). While an
 // instance keeps its lists, its particles keep the slots of the list build:
@@ -139,6 +147,7 @@ struct Grid {
     float lof[3], wf[3], invwf[3];
     float lzf, halflzf;
     float slop[3];   // absolute slack added to query boxes (FP32 rounding cover)
+    float Xf, lzerr; // X rounded up; |lz - lzf| rounded up
     float eC, eR;    // FP32-error bound of a coordinate difference: e(R) <= eC + eR * R
     int fxk;         // fixed-point exponent of the coordinate chunks: |x| 2^fxk < 2^61
     float lzc[3];    // lz as chunks, in the pair kernels' length unit
@@ -323,16 +332,19 @@ struct sph_ctx {
     double *hs_lo, *hs_hi;  // bisection bracket of particles handed to the per-particle search
     int32_t* hs_it;         // counts already done for them
     int32_t* wl;            // their indices (count in status[3])
+    int32_t* gwl;           // groups of 32 that go on searching together (count in wctr[1])
     double* red_part;       // bbox partials: kBoxStride per group of kSlotAlign slots
     double* dt_part;        // per force block (kMaxPairThreads per kThreads slots)
     sph::Grid* grid;        // per instance
-    unsigned long long* wctr;  // work counters of persistent kernels (zeroed per build)
+    unsigned long long* wctr;  // [0] work counter of k_h_union, [1] length of gwl (zeroed
+                               // per build)
     int2* recs;             // h search records: kRec per lane of the persistent grid
     int64_t nslots;         // slot capacity (particles plus the gaps between instances)
     int32_t* lst;           // candidate lists: kList per slot (warp-interleaved); these
     sph::LMeta* lmeta;      // three are allocated by the first call that turns lists on;
     unsigned* lctr;         // their records per caller index; list builds so far
     bool any_lists;         // some instance of the current batch uses candidate lists
+    bool group_search;      // some instance has kGroupSearchN particles or more
     int lay_n;              // instances of the last batch layout (first, count) ...
     int64_t lay_first[sph::kMaxInstances], lay_cnt[sph::kMaxInstances];  // ... and theirs
     int nsm;                // streaming multiprocessors of the device
@@ -358,8 +370,8 @@ struct sph_ctx {
     // sph_step / sph_batch_step instead of its ~35 separate launches.
     struct StepGraph {
         bool valid;
-        int64_t key[10];         // what the launches bake in (sizes, kinds, dt/time pointers,
-                                 // the bounding-box variant)
+        int64_t key[11];         // what the launches bake in (sizes, kinds, dt/time pointers,
+                                 // the bounding-box and h-search variants)
         cudaGraphExec_t exec;
         int64_t launches;        // kernels of one step
     } sg[2];
