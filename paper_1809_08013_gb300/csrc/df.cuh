@@ -61,6 +61,12 @@ __device__ __forceinline__ df addf(df x, float b) {
     return fast_two_sum(s.hi, __fadd_rn(s.lo, x.lo));
 }
 
+// addf for |b| >= |x.hi|: the exact sum by Fast2Sum, the same bits as addf.
+__device__ __forceinline__ df addf_larger(df x, float b) {
+    const df s = fast_two_sum(b, x.hi);
+    return fast_two_sum(s.hi, __fadd_rn(s.lo, x.lo));
+}
+
 // Products return (p, e) without the final Fast2Sum: that step is exact (it
 // does not change hi + lo), and every consumer here -- another product, a
 // sum, a sign or range test of hi, the conversion to double -- accepts a low

@@ -490,12 +490,14 @@ k_forces_iad(int64_t n, Batch B, const double4_32a* __restrict__ posh,
 
 // One block per instance: dt[k] = cfl_k * min over the instance's block
 // partials; time[k] += dt[k] when time is given. The force kernel ran with
-// tpp lanes per particle, so a block covered kThreads / tpp particles.
+// tpp lanes per particle in blocks of `threads`, so a block covered threads /
+// tpp particles.
 __global__ void __launch_bounds__(kThreads)
-k_dt_finish(const double* __restrict__ part, Batch B, int tpp, double* __restrict__ dt_out,
+k_dt_finish(const double* __restrict__ part, Batch B, int tpp, int threads,
+            double* __restrict__ dt_out,
             double* __restrict__ time) {
     const int inst = blockIdx.x;
-    const int64_t per_block = kThreads / tpp;
+    const int64_t per_block = threads / tpp;
     const int64_t b0 = B.ioff[inst] / per_block;
     const int64_t nbk = (B.icnt[inst] + per_block - 1) / per_block;
     double m = CUDART_INF;
@@ -520,6 +522,7 @@ void launch_forces(sph_ctx* c, double* dt_out, double* time_inout, cudaStream_t 
     const int b = c->cur;
     const Batch B = batch_of(c);
     c->launches += 1;
+    c->dt_block = kThreads;  // (unless the force kernel below takes smaller blocks)
     if (c->prec == PREC_MIXED)
         launch_forces_mx(c, s);
     else if (!native_pairs(c) && c->grad_kind == 1)
@@ -550,7 +553,7 @@ void launch_forces(sph_ctx* c, double* dt_out, double* time_inout, cudaStream_t 
         else go(k_forces<KER_M4>);
     }
     k_dt_finish<<<c->ninst, kThreads, 0, s>>>(c->dt_part, B, native_pairs(c) ? 1 : c->tpp,
-                                              dt_out, time_inout);
+                                              c->dt_block, dt_out, time_inout);
 }
 
 // ------------------------------------------------------------ leapfrog

@@ -28,17 +28,22 @@ using dfl::df;
 
 namespace {
 
-// pi h^3 W as a function of q >= 0 (cubic spline). In the outer piece,
-// 1 <= q.hi <= 2, 2 - q.hi is exact (Sterbenz) and a multiple of ulp(q.hi),
-// so Fast2Sum with -q.lo gives 2 - q exactly, normalised.
+// pi h^3 W as a function of q >= 0 (cubic spline). Both pieces are
+// u^2 (a u + b) + c with the coefficients of q's piece, so that no branch
+// splits the code (neighbours are evaluated several at a time):
+//   q < 1:      1 + q^2 (0.75 q - 1.5)    u = q
+//   1 <= q < 2: t^2 (0.25 t)              u = t = 2 - q
+// For 1 <= q.hi <= 2, 2 - q.hi is exact (Sterbenz) and a multiple of ulp(q.hi),
+// so Fast2Sum with -q.lo gives 2 - q exactly, normalised. The constants are the
+// larger operands of their sums (0.75 q < 1.5, |q^2 (0.75 q - 1.5)| <= 0.75 for
+// q < 1; a sum with 0 is exact).
 __device__ __forceinline__ df w_shape(df q) {
-    const df q2 = dfl::sqr(q);
-    const df a = dfl::addf(dfl::mulf(q, 0.75f), -1.5f);
-    const df win = dfl::addf(dfl::mul(q2, a), 1.0f);  // 1 - 1.5 q^2 + 0.75 q^3
+    const bool in = q.hi < 1.0f;
     const df t = dfl::fast_two_sum(__fsub_rn(2.0f, q.hi), -q.lo);
-    const df wout = dfl::scale2(dfl::mul(dfl::sqr(t), t), 0.25f);  // (2 - q)^3 / 4
-    const df zero = {0.0f, 0.0f};
-    return q.hi < 1.0f ? win : (q.hi < 2.0f ? wout : zero);
+    const df u = {in ? q.hi : t.hi, in ? q.lo : t.lo};
+    const df a = dfl::addf_larger(dfl::mulf(u, in ? 0.75f : 0.25f), in ? -1.5f : 0.0f);
+    const df w = dfl::addf_larger(dfl::mul(dfl::sqr(u), a), in ? 1.0f : 0.0f);
+    return {q.hi < 2.0f ? w.hi : 0.0f, q.hi < 2.0f ? w.lo : 0.0f};
 }
 
 // pi h^4 dW/dr as a function of q >= 0. Both pieces are one product
@@ -52,7 +57,8 @@ __device__ __forceinline__ df w_shape(df q) {
 __device__ __forceinline__ df dw_shape(df q) {
     const bool in = q.hi < 1.0f;
     const df u = in ? q : dfl::fast_two_sum(__fsub_rn(q.hi, 2.0f), q.lo);
-    const df v = dfl::addf(dfl::mulf(q, in ? 2.25f : -0.75f), in ? -3.0f : 1.5f);
+    // (|2.25 q| < 3 for q < 1, 0.75 q <= 1.5 for q <= 2; beyond, f is not used)
+    const df v = dfl::addf_larger(dfl::mulf(q, in ? 2.25f : -0.75f), in ? -3.0f : 1.5f);
     const df f = dfl::mul(u, v);
     const df zero = {0.0f, 0.0f};
     return q.hi < 2.0f ? f : zero;
@@ -183,8 +189,11 @@ __device__ __forceinline__ void eos_d(const KParams& kp, double rho, double u, d
 // (2 h_j)^2 is packed as a float (within 2^-24), so r^2 below / above it by
 // more than 2^-20 decides; the band between takes the FP64 test itself. The
 // sets are the exact ones, as built by k_outer.
+// The next neighbour's loads go out before one is evaluated, in blocks of 64
+// threads: 1M patch 681 us (732 without, in blocks of 256; the branch-free shape
+// gave 38 us of that).
 template <bool FUSE, int T, int KER, bool OUTER>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kPairBlockMin)
 k_density_df(int64_t n, Batch B, const double4_32a* __restrict__ posh,
              const float4* __restrict__ xpk, const double* __restrict__ ue,
              Rows R, double4_32a* __restrict__ therm,
@@ -213,10 +222,21 @@ k_density_df(int64_t n, Batch B, const double4_32a* __restrict__ posh,
     // rows read from the CSR (a gather set overflowed) are complete already
     const bool append = OUTER && !(R.status[2] & IF_SLAB_OVF);
     Append ap;
+    int jn = (int)i;
+    float4 N0 = I0, N1 = I1, N2 = I2;
+    auto fetch = [&](int e) {
+        if (e < len) {
+            jn = __ldg(&ent[e]);
+            N0 = __ldg(&xpk[3 * jn]);
+            N1 = __ldg(&xpk[3 * jn + 1]);
+            N2 = __ldg(&xpk[3 * jn + 2]);
+        }
+    };
+    fetch(sub);
     for (int e = sub; e < len; e += T) {
-        const int j = __ldg(&ent[e]);
-        const float4 J0 = __ldg(&xpk[3 * j]), J1 = __ldg(&xpk[3 * j + 1]);
-        const float4 J2 = __ldg(&xpk[3 * j + 2]);
+        const int j = jn;
+        const float4 J0 = N0, J1 = N1, J2 = N2;
+        fetch(e + T);
         const df mj = {J0.w, J1.w};
         float z2 = __fsub_rn(I0.z, J0.z), z1 = __fsub_rn(I1.z, J1.z), z0 = __fsub_rn(I2.z, J2.z);
         if (per) wrap_fx(z2, z1, z0, hlz, L2, L1, L0);
@@ -225,7 +245,11 @@ k_density_df(int64_t n, Batch B, const double4_32a* __restrict__ posh,
         const df Z = dfl::fx_sum(z2, z1, z0);
         const df r2 = dfl::add(dfl::add_same(dfl::sqr(X), dfl::sqr(Y)), dfl::sqr(Z));
         df w = {1.0f, 0.0f};  // coincident particles: q = 0
-        if (r2.hi > 0.0f) {
+        if (KER == KER_M4) {
+            const df v = w_shape(dfl::mul(dfl::mul(r2, dfl::rsqrt(r2)), Hi));
+            w.hi = r2.hi > 0.0f ? v.hi : w.hi;
+            w.lo = r2.hi > 0.0f ? v.lo : w.lo;
+        } else if (r2.hi > 0.0f) {
             const df q = dfl::mul(dfl::mul(r2, dfl::rsqrt(r2)), Hi);
             w = w_shape_k<KER>(q, sn);
         }
@@ -273,13 +297,13 @@ k_density_df(int64_t n, Batch B, const double4_32a* __restrict__ posh,
 template <bool FUSE, int T, bool OUTER>
 static void density_df_t(sph_ctx* c, cudaStream_t s) {
     const int64_t n = c->n;
-    const unsigned nb = (unsigned)((n * T + kThreads - 1) / kThreads);
     const int b = c->cur;
     const Rows R = OUTER ? rows_gather(c) : rows_of(c);
     auto go = [&](auto kernel_fn) {
-        kernel_fn<<<nb, kThreads, 0, s>>>(n, batch_of(c), c->posh[b], c->xpk, c->ue[b], R,
-                                          c->therm, c->kern, c->dpk, c->pint, c->cint, c->status,
-                                          OuterOut{c->rslab, c->ocnt, c->status});
+        const unsigned tb = kPairBlockMin;
+        kernel_fn<<<(unsigned)((n * T + tb - 1) / tb), tb, 0, s>>>(
+            n, batch_of(c), c->posh[b], c->xpk, c->ue[b], R, c->therm, c->kern, c->dpk, c->pint,
+            c->cint, c->status, OuterOut{c->rslab, c->ocnt, c->status});
     };
     if (c->kern_kind == KER_WENDLAND) go(k_density_df<FUSE, T, KER_WENDLAND, OUTER>);
     else if (c->kern_kind == KER_SINC) go(k_density_df<FUSE, T, KER_SINC, OUTER>);
@@ -310,8 +334,18 @@ void launch_density_df(sph_ctx* c, bool fuse_eos, cudaStream_t s, bool outer) {
 // viscosity, mu = hb v.r rhob R, 1/rhob = (r^2 + eta2 hb^2) R. Every sum is
 // linear in Fbar, so its constant factor (0.5/pi, or dnorm/2) is applied once
 // per particle, in FP64, when the sums are written out.
-template <int T, int KER>
-__global__ void __launch_bounds__(kThreads, KER == KER_SINC ? 2 : 3)
+// U: neighbours evaluated at a time, their terms added in the order of the row
+// (the same bits for every U); with U > 1 the viscosity is evaluated for every
+// pair and selected, so that no branch keeps the U evaluations apart.
+// Bound: instruction dispatch (550 warp instructions a pair, mostly FP32 with
+// three register operands, which this GPU issues at 0.62 of the rate of the
+// others). U = 4 in blocks of 64 (160 registers, 12 warps an SM) against U = 1
+// in blocks of 256 (80 registers, 24 warps): 4,096 particles 44 us (91), 27,000
+// 70 (108), 104k 216 (247), 1M 1,795 (1,893); the Wendland kernel at 216,000
+// 427 (457). U = 3: 1,860 at 1M; 5 or 6: 2,330. The sinc shapes, with a loop
+// over terms, are faster one at a time (1,076 against 1,410 at 216,000).
+template <int T, int KER, int U>
+__global__ void __launch_bounds__(kPairBlock<U>, U > 1 ? 1 : (KER == KER_SINC ? 2 : 3))
 k_forces_df(int64_t n, Batch B, const double4_32a* __restrict__ posh,
             const float4* __restrict__ vpa, const float2* __restrict__ vpb,
             const float4* __restrict__ dpk,
@@ -343,49 +377,113 @@ k_forces_df(int64_t n, Batch B, const double4_32a* __restrict__ posh,
         const int sn = kp.sinc_n;
         const df eta2 = dfl::from_double_fp64(kp.eta2);
         const df betad = dfl::from_double_fp64(kp.beta);
-        for (int e = sub; e < len; e += T) {
-            const int j = __ldg(&ent[e]);
-            const float4 J0 = __ldg(&xpk[3 * j]), J1 = __ldg(&xpk[3 * j + 1]);
-            const float4 J2 = __ldg(&xpk[3 * j + 2]);
-            const float4 wa = __ldg(&vpa[j]);
-            const float2 wb = __ldg(&vpb[j]);
-            const float4 b0 = __ldg(&dpk[3 * j]), b1 = __ldg(&dpk[3 * j + 1]);
-            const float4 b2 = __ldg(&dpk[3 * j + 2]);
-            float z2 = __fsub_rn(I0.z, J0.z), z1 = __fsub_rn(I1.z, J1.z), z0 = __fsub_rn(I2.z, J2.z);
-            if (per) wrap_fx(z2, z1, z0, hlz, L2, L1, L0);
-            const df X = dfl::fx_sum(__fsub_rn(I0.x, J0.x), __fsub_rn(I1.x, J1.x), __fsub_rn(I2.x, J2.x));
-            const df Y = dfl::fx_sum(__fsub_rn(I0.y, J0.y), __fsub_rn(I1.y, J1.y), __fsub_rn(I2.y, J2.y));
-            const df Z = dfl::fx_sum(z2, z1, z0);
-            const df r2 = dfl::add(dfl::add_same(dfl::sqr(X), dfl::sqr(Y)), dfl::sqr(Z));
-            if (!(r2.hi > 0.0f)) continue;  // coincident particles exert no force
-            const df rinv = dfl::rsqrt(r2);
-            const df r = dfl::mul(r2, rinv);
-            const df fa = dw_shape_k<KER>(dfl::mul(r, Hi), sn);
-            const df fb = dw_shape_k<KER>(dfl::mul(r, df{b0.x, b0.y}), sn);
-            const df Fb = dfl::mul(dfl::add(dfl::mul(Ki, fa), dfl::mul(df{b0.z, b0.w}, fb)), rinv);
-            const df WX = dfl::sub(VXi, df{wa.x, wa.y}), WY = dfl::sub(VYi, df{wa.z, wa.w});
-            const df WZ = dfl::sub(VZi, df{wb.x, wb.y});
-            const df vr = dfl::add(dfl::add(dfl::mul(WX, X), dfl::mul(WY, Y)), dfl::mul(WZ, Z));
-            df Pi = {0.f, 0.f};
-            if (vr.hi < 0.0f) {
-                const df hb = dfl::add(hhi, df{b1.z, b1.w});
-                const df d1 = dfl::add(r2, dfl::mul(dfl::mul(eta2, hb), hb));
-                const df rb = dfl::add(rhi, df{b2.x, b2.y});
-                const df R = dfl::rcp(dfl::mul(d1, rb));
-                const df mu = dfl::mul(dfl::mul(dfl::mul(hb, vr), rb), R);
-                const df cb = dfl::add(cai, df{b2.z, b2.w});
-                const df t = dfl::add(dfl::mul(betad, mu), dfl::neg(cb));
-                Pi = dfl::mul(dfl::mul(mu, t), dfl::mul(d1, R));
-                if (-mu.hi > mumx.hi) mumx = dfl::neg(mu);
+        if constexpr (U == 1) {
+            for (int e = sub; e < len; e += T) {
+                const int j = __ldg(&ent[e]);
+                const float4 J0 = __ldg(&xpk[3 * j]), J1 = __ldg(&xpk[3 * j + 1]);
+                const float4 J2 = __ldg(&xpk[3 * j + 2]);
+                const float4 wa = __ldg(&vpa[j]);
+                const float2 wb = __ldg(&vpb[j]);
+                const float4 b0 = __ldg(&dpk[3 * j]), b1 = __ldg(&dpk[3 * j + 1]);
+                const float4 b2 = __ldg(&dpk[3 * j + 2]);
+                float z2 = __fsub_rn(I0.z, J0.z), z1 = __fsub_rn(I1.z, J1.z), z0 = __fsub_rn(I2.z, J2.z);
+                if (per) wrap_fx(z2, z1, z0, hlz, L2, L1, L0);
+                const df X = dfl::fx_sum(__fsub_rn(I0.x, J0.x), __fsub_rn(I1.x, J1.x), __fsub_rn(I2.x, J2.x));
+                const df Y = dfl::fx_sum(__fsub_rn(I0.y, J0.y), __fsub_rn(I1.y, J1.y), __fsub_rn(I2.y, J2.y));
+                const df Z = dfl::fx_sum(z2, z1, z0);
+                const df r2 = dfl::add(dfl::add_same(dfl::sqr(X), dfl::sqr(Y)), dfl::sqr(Z));
+                if (!(r2.hi > 0.0f)) continue;  // coincident particles exert no force
+                const df rinv = dfl::rsqrt(r2);
+                const df r = dfl::mul(r2, rinv);
+                const df fa = dw_shape_k<KER>(dfl::mul(r, Hi), sn);
+                const df fb = dw_shape_k<KER>(dfl::mul(r, df{b0.x, b0.y}), sn);
+                const df Fb = dfl::mul(dfl::add(dfl::mul(Ki, fa), dfl::mul(df{b0.z, b0.w}, fb)), rinv);
+                const df WX = dfl::sub(VXi, df{wa.x, wa.y}), WY = dfl::sub(VYi, df{wa.z, wa.w});
+                const df WZ = dfl::sub(VZi, df{wb.x, wb.y});
+                const df vr = dfl::add(dfl::add(dfl::mul(WX, X), dfl::mul(WY, Y)), dfl::mul(WZ, Z));
+                df Pi = {0.f, 0.f};
+                if (vr.hi < 0.0f) {
+                    const df hb = dfl::add(hhi, df{b1.z, b1.w});
+                    const df d1 = dfl::add(r2, dfl::mul(dfl::mul(eta2, hb), hb));
+                    const df rb = dfl::add(rhi, df{b2.x, b2.y});
+                    const df R = dfl::rcp(dfl::mul(d1, rb));
+                    const df mu = dfl::mul(dfl::mul(dfl::mul(hb, vr), rb), R);
+                    const df cb = dfl::add(cai, df{b2.z, b2.w});
+                    const df t = dfl::add(dfl::mul(betad, mu), dfl::neg(cb));
+                    Pi = dfl::mul(dfl::mul(mu, t), dfl::mul(d1, R));
+                    if (-mu.hi > mumx.hi) mumx = dfl::neg(mu);
+                }
+                const df mF = dfl::mul(df{J0.w, J1.w}, Fb);
+                const df g = dfl::mul(mF, dfl::add(dfl::add(Ai, df{b1.x, b1.y}), Pi));
+                sx = dfl::add(sx, dfl::mul(g, X));
+                sy = dfl::add(sy, dfl::mul(g, Y));
+                sz = dfl::add(sz, dfl::mul(g, Z));
+                const df mFv = dfl::mul(mF, vr);
+                sp = dfl::add(sp, mFv);
+                sv = dfl::add(sv, dfl::mul(mFv, Pi));
             }
-            const df mF = dfl::mul(df{J0.w, J1.w}, Fb);
-            const df g = dfl::mul(mF, dfl::add(dfl::add(Ai, df{b1.x, b1.y}), Pi));
-            sx = dfl::add(sx, dfl::mul(g, X));
-            sy = dfl::add(sy, dfl::mul(g, Y));
-            sz = dfl::add(sz, dfl::mul(g, Z));
-            const df mFv = dfl::mul(mF, vr);
-            sp = dfl::add(sp, mFv);
-            sv = dfl::add(sv, dfl::mul(mFv, Pi));
+        } else {
+            for (int e0 = sub; e0 < len; e0 += T * U) {
+                int j[U];
+                df tx[U], ty[U], tz[U], tp[U], tv[U], nmu[U];
+                bool use[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    j[u] = e0 + u * T < len ? __ldg(&ent[e0 + u * T]) : (int)i;
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const float4 J0 = __ldg(&xpk[3 * j[u]]), J1 = __ldg(&xpk[3 * j[u] + 1]);
+                    const float4 J2 = __ldg(&xpk[3 * j[u] + 2]);
+                    const float4 wa = __ldg(&vpa[j[u]]);
+                    const float2 wb = __ldg(&vpb[j[u]]);
+                    const float4 b0 = __ldg(&dpk[3 * j[u]]), b1 = __ldg(&dpk[3 * j[u] + 1]);
+                    const float4 b2 = __ldg(&dpk[3 * j[u] + 2]);
+                    float z2 = __fsub_rn(I0.z, J0.z), z1 = __fsub_rn(I1.z, J1.z), z0 = __fsub_rn(I2.z, J2.z);
+                    if (per) wrap_fx(z2, z1, z0, hlz, L2, L1, L0);
+                    const df X = dfl::fx_sum(__fsub_rn(I0.x, J0.x), __fsub_rn(I1.x, J1.x), __fsub_rn(I2.x, J2.x));
+                    const df Y = dfl::fx_sum(__fsub_rn(I0.y, J0.y), __fsub_rn(I1.y, J1.y), __fsub_rn(I2.y, J2.y));
+                    const df Z = dfl::fx_sum(z2, z1, z0);
+                    const df r2 = dfl::add(dfl::add_same(dfl::sqr(X), dfl::sqr(Y)), dfl::sqr(Z));
+                    const bool ok = e0 + u * T < len && r2.hi > 0.0f;  // (coincident: no force)
+                    const df rinv = dfl::rsqrt(r2);
+                    const df r = dfl::mul(r2, rinv);
+                    const df fa = dw_shape_k<KER>(dfl::mul(r, Hi), sn);
+                    const df fb = dw_shape_k<KER>(dfl::mul(r, df{b0.x, b0.y}), sn);
+                    const df Fb = dfl::mul(dfl::add(dfl::mul(Ki, fa), dfl::mul(df{b0.z, b0.w}, fb)), rinv);
+                    const df WX = dfl::sub(VXi, df{wa.x, wa.y}), WY = dfl::sub(VYi, df{wa.z, wa.w});
+                    const df WZ = dfl::sub(VZi, df{wb.x, wb.y});
+                    const df vr = dfl::add(dfl::add(dfl::mul(WX, X), dfl::mul(WY, Y)), dfl::mul(WZ, Z));
+                    const df hb = dfl::add(hhi, df{b1.z, b1.w});
+                    const df d1 = dfl::add(r2, dfl::mul(dfl::mul(eta2, hb), hb));
+                    const df rb = dfl::add(rhi, df{b2.x, b2.y});
+                    const df R = dfl::rcp(dfl::mul(d1, rb));
+                    const df mu = dfl::mul(dfl::mul(dfl::mul(hb, vr), rb), R);
+                    const df cb = dfl::add(cai, df{b2.z, b2.w});
+                    const df t = dfl::add(dfl::mul(betad, mu), dfl::neg(cb));
+                    const df Pv = dfl::mul(dfl::mul(mu, t), dfl::mul(d1, R));
+                    const bool visc = vr.hi < 0.0f;
+                    const df Pi = {visc ? Pv.hi : 0.f, visc ? Pv.lo : 0.f};
+                    nmu[u] = df{ok && visc ? -mu.hi : 0.f, ok && visc ? -mu.lo : 0.f};
+                    const df mF = dfl::mul(df{J0.w, J1.w}, Fb);
+                    const df g = dfl::mul(mF, dfl::add(dfl::add(Ai, df{b1.x, b1.y}), Pi));
+                    tx[u] = dfl::mul(g, X);
+                    ty[u] = dfl::mul(g, Y);
+                    tz[u] = dfl::mul(g, Z);
+                    tp[u] = dfl::mul(mF, vr);
+                    tv[u] = dfl::mul(tp[u], Pi);
+                    use[u] = ok;
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    if (!use[u]) continue;
+                    sx = dfl::add(sx, tx[u]);
+                    sy = dfl::add(sy, ty[u]);
+                    sz = dfl::add(sz, tz[u]);
+                    sp = dfl::add(sp, tp[u]);
+                    sv = dfl::add(sv, tv[u]);
+                    if (nmu[u].hi > mumx.hi) mumx = nmu[u];
+                }
+            }
         }
     }
     if (T > 1) {
@@ -421,12 +519,12 @@ k_forces_df(int64_t n, Batch B, const double4_32a* __restrict__ posh,
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) dtc = fmin(dtc, __shfl_xor_sync(0xffffffffu, dtc, o));
-    __shared__ double sh[kThreads / 32];
+    __shared__ double sh[kPairBlock<U> / 32];
     if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = dtc;
     __syncthreads();
     if (threadIdx.x == 0) {
         double m = sh[0];
-        for (int w = 1; w < kThreads / 32; ++w) m = fmin(m, sh[w]);
+        for (int w = 1; w < kPairBlock<U> / 32; ++w) m = fmin(m, sh[w]);
         dt_part[blockIdx.x] = m;
     }
 }
@@ -434,20 +532,17 @@ k_forces_df(int64_t n, Batch B, const double4_32a* __restrict__ posh,
 template <int T>
 static void forces_df_t(sph_ctx* c, cudaStream_t s) {
     const int64_t n = c->n;
-    const unsigned nb = (unsigned)((n * T + kThreads - 1) / kThreads);
     const int b = c->cur;
-    if (c->kern_kind == KER_WENDLAND)
-        k_forces_df<T, KER_WENDLAND><<<nb, kThreads, 0, s>>>(
+    auto go = [&](auto kernel_fn, int U) {
+        const unsigned tb = U > 1 ? kPairBlockMin : kThreads;
+        kernel_fn<<<(unsigned)((n * T + tb - 1) / tb), tb, 0, s>>>(
             n, batch_of(c), c->posh[b], c->vpa, c->vpb, c->dpk, c->xpk, c->cint, rows_of(c), c->acc,
             c->mumax, c->dt_part);
-    else if (c->kern_kind == KER_SINC)
-        k_forces_df<T, KER_SINC><<<nb, kThreads, 0, s>>>(
-            n, batch_of(c), c->posh[b], c->vpa, c->vpb, c->dpk, c->xpk, c->cint, rows_of(c), c->acc,
-            c->mumax, c->dt_part);
-    else
-        k_forces_df<T, KER_M4><<<nb, kThreads, 0, s>>>(
-            n, batch_of(c), c->posh[b], c->vpa, c->vpb, c->dpk, c->xpk, c->cint, rows_of(c), c->acc,
-            c->mumax, c->dt_part);
+        c->dt_block = (int)tb;
+    };
+    if (c->kern_kind == KER_WENDLAND) go(k_forces_df<T, KER_WENDLAND, 4>, 4);
+    else if (c->kern_kind == KER_SINC) go(k_forces_df<T, KER_SINC, 1>, 1);
+    else go(k_forces_df<T, KER_M4, 4>, 4);
 }
 
 void launch_forces_df(sph_ctx* c, cudaStream_t s) {
@@ -481,7 +576,7 @@ k_volume_df(int64_t n, Batch B, const double4_32a* __restrict__ velm,
 // in FP64 by the adjugate (C_i = 0 if singular) and stored as float pairs:
 //   cpk[3i] = (C00, C01), cpk[3i+1] = (C02, C11), cpk[3i+2] = (C12, C22).
 template <int T, int KER>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kPairBlockMin)
 k_iad_df(int64_t n, Batch B, const double4_32a* __restrict__ posh,
          const float4* __restrict__ xpk, const float2* __restrict__ vdf, Rows R,
          float4* __restrict__ cpk) {
@@ -504,11 +599,23 @@ k_iad_df(int64_t n, Batch B, const double4_32a* __restrict__ posh,
         const bool per = B.kp[inst].periodic_z != 0;
         const float hlz = g.hlzc, L2 = g.lzc[0], L1 = g.lzc[1], L0 = g.lzc[2];
         const float4 I0 = xpk[3 * i], I1 = xpk[3 * i + 1], I2 = xpk[3 * i + 2];
+        // (the next neighbour's loads go out before one is evaluated)
+        float4 N0 = I0, N1 = I1, N2 = I2;
+        float2 nv = make_float2(0.0f, 0.0f);
+        auto fetch = [&](int e) {
+            if (e < len) {
+                const int j = __ldg(&ent[e]);
+                N0 = __ldg(&xpk[3 * j]);
+                N1 = __ldg(&xpk[3 * j + 1]);
+                N2 = __ldg(&xpk[3 * j + 2]);
+                nv = __ldg(&vdf[j]);
+            }
+        };
+        fetch(sub);
         for (int e = sub; e < len; e += T) {
-            const int j = __ldg(&ent[e]);
-            const float4 J0 = __ldg(&xpk[3 * j]), J1 = __ldg(&xpk[3 * j + 1]);
-            const float4 J2 = __ldg(&xpk[3 * j + 2]);
-            const float2 vj = __ldg(&vdf[j]);
+            const float4 J0 = N0, J1 = N1, J2 = N2;
+            const float2 vj = nv;
+            fetch(e + T);
             float z2 = __fsub_rn(I0.z, J0.z), z1 = __fsub_rn(I1.z, J1.z), z0 = __fsub_rn(I2.z, J2.z);
             if (per) wrap_fx(z2, z1, z0, hlz, L2, L1, L0);
             const df X = dfl::fx_sum(__fsub_rn(I0.x, J0.x), __fsub_rn(I1.x, J1.x), __fsub_rn(I2.x, J2.x));
@@ -559,8 +666,10 @@ __device__ __forceinline__ void symv_df(const df* M, const df& x, const df& y, c
 
 // Forces with IAD gradients: as k_forces_df with F r_ij replaced by
 // G_ij = -(wnorm / 2) (h_i^-3 g(q_i) C_i + h_j^-3 g(q_j) C_j) r_ij.
-template <int T, int KER>
-__global__ void __launch_bounds__(kThreads, 2)
+// U: as in k_forces_df (125,000 particles, Wendland: 396 us at U = 1, 371 at 2,
+// 415 at 3; sinc at 216,000: 1,022 at 1, 1,195 at 2).
+template <int T, int KER, int U>
+__global__ void __launch_bounds__(kPairBlock<U>, U > 1 ? 1 : 2)
 k_forces_iad_df(int64_t n, Batch B, const double4_32a* __restrict__ posh,
                 const float4* __restrict__ vpa, const float2* __restrict__ vpb,
                 const float4* __restrict__ dpk,
@@ -596,63 +705,141 @@ k_forces_iad_df(int64_t n, Batch B, const double4_32a* __restrict__ posh,
         const df kg = dfl::from_double_fp64(-0.5 * (KER == KER_M4 ? kInvPi : kp.wnorm));
         const df eta2 = dfl::from_double_fp64(kp.eta2);
         const df betad = dfl::from_double_fp64(kp.beta);
-        for (int e = sub; e < len; e += T) {
-            const int j = __ldg(&ent[e]);
-            const float4 J0 = __ldg(&xpk[3 * j]), J1 = __ldg(&xpk[3 * j + 1]);
-            const float4 J2 = __ldg(&xpk[3 * j + 2]);
-            const float4 wa = __ldg(&vpa[j]);
-            const float2 wb = __ldg(&vpb[j]);
-            const float4 b0 = __ldg(&dpk[3 * j]), b1 = __ldg(&dpk[3 * j + 1]);
-            const float4 b2 = __ldg(&dpk[3 * j + 2]);
-            float z2 = __fsub_rn(I0.z, J0.z), z1 = __fsub_rn(I1.z, J1.z), z0 = __fsub_rn(I2.z, J2.z);
-            if (per) wrap_fx(z2, z1, z0, hlz, L2, L1, L0);
-            const df X = dfl::fx_sum(__fsub_rn(I0.x, J0.x), __fsub_rn(I1.x, J1.x), __fsub_rn(I2.x, J2.x));
-            const df Y = dfl::fx_sum(__fsub_rn(I0.y, J0.y), __fsub_rn(I1.y, J1.y), __fsub_rn(I2.y, J2.y));
-            const df Z = dfl::fx_sum(z2, z1, z0);
-            const df r2 = dfl::add(dfl::add_same(dfl::sqr(X), dfl::sqr(Y)), dfl::sqr(Z));
-            if (!(r2.hi > 0.0f)) continue;  // coincident particles exert no force
-            const df r = dfl::mul(r2, dfl::rsqrt(r2));
-            const df Hj = {b0.x, b0.y};
-            const df wi = dfl::mul(Hi3, w_shape_k<KER>(dfl::mul(r, Hi), sn));
-            const df wj = dfl::mul(dfl::mul(Hj, dfl::sqr(Hj)), w_shape_k<KER>(dfl::mul(r, Hj), sn));
-            df M[6];
-            {
-                const float4 d0 = __ldg(&cpk[3 * j]), d1 = __ldg(&cpk[3 * j + 1]);
-                const float4 d2 = __ldg(&cpk[3 * j + 2]);
-                const df Cj[6] = {{d0.x, d0.y}, {d0.z, d0.w}, {d1.x, d1.y},
-                                  {d1.z, d1.w}, {d2.x, d2.y}, {d2.z, d2.w}};
+        if constexpr (U == 1) {
+            for (int e = sub; e < len; e += T) {
+                const int j = __ldg(&ent[e]);
+                const float4 J0 = __ldg(&xpk[3 * j]), J1 = __ldg(&xpk[3 * j + 1]);
+                const float4 J2 = __ldg(&xpk[3 * j + 2]);
+                const float4 wa = __ldg(&vpa[j]);
+                const float2 wb = __ldg(&vpb[j]);
+                const float4 b0 = __ldg(&dpk[3 * j]), b1 = __ldg(&dpk[3 * j + 1]);
+                const float4 b2 = __ldg(&dpk[3 * j + 2]);
+                float z2 = __fsub_rn(I0.z, J0.z), z1 = __fsub_rn(I1.z, J1.z), z0 = __fsub_rn(I2.z, J2.z);
+                if (per) wrap_fx(z2, z1, z0, hlz, L2, L1, L0);
+                const df X = dfl::fx_sum(__fsub_rn(I0.x, J0.x), __fsub_rn(I1.x, J1.x), __fsub_rn(I2.x, J2.x));
+                const df Y = dfl::fx_sum(__fsub_rn(I0.y, J0.y), __fsub_rn(I1.y, J1.y), __fsub_rn(I2.y, J2.y));
+                const df Z = dfl::fx_sum(z2, z1, z0);
+                const df r2 = dfl::add(dfl::add_same(dfl::sqr(X), dfl::sqr(Y)), dfl::sqr(Z));
+                if (!(r2.hi > 0.0f)) continue;  // coincident particles exert no force
+                const df r = dfl::mul(r2, dfl::rsqrt(r2));
+                const df Hj = {b0.x, b0.y};
+                const df wi = dfl::mul(Hi3, w_shape_k<KER>(dfl::mul(r, Hi), sn));
+                const df wj = dfl::mul(dfl::mul(Hj, dfl::sqr(Hj)), w_shape_k<KER>(dfl::mul(r, Hj), sn));
+                df M[6];
+                {
+                    const float4 d0 = __ldg(&cpk[3 * j]), d1 = __ldg(&cpk[3 * j + 1]);
+                    const float4 d2 = __ldg(&cpk[3 * j + 2]);
+                    const df Cj[6] = {{d0.x, d0.y}, {d0.z, d0.w}, {d1.x, d1.y},
+                                      {d1.z, d1.w}, {d2.x, d2.y}, {d2.z, d2.w}};
+    #pragma unroll
+                    for (int k = 0; k < 6; ++k) M[k] = dfl::add(dfl::mul(wi, Ci[k]), dfl::mul(wj, Cj[k]));
+                }
+                df Gx, Gy, Gz;
+                symv_df(M, X, Y, Z, Gx, Gy, Gz);
+                Gx = dfl::mul(kg, Gx);
+                Gy = dfl::mul(kg, Gy);
+                Gz = dfl::mul(kg, Gz);
+                const df WX = dfl::sub(VXi, df{wa.x, wa.y}), WY = dfl::sub(VYi, df{wa.z, wa.w});
+                const df WZ = dfl::sub(VZi, df{wb.x, wb.y});
+                const df vr = dfl::add(dfl::add(dfl::mul(WX, X), dfl::mul(WY, Y)), dfl::mul(WZ, Z));
+                df Pi = {0.f, 0.f};
+                if (vr.hi < 0.0f) {
+                    const df hb = dfl::add(hhi, df{b1.z, b1.w});
+                    const df d1 = dfl::add(r2, dfl::mul(dfl::mul(eta2, hb), hb));
+                    const df rb = dfl::add(rhi, df{b2.x, b2.y});
+                    const df Rr = dfl::rcp(dfl::mul(d1, rb));
+                    const df mu = dfl::mul(dfl::mul(dfl::mul(hb, vr), rb), Rr);
+                    const df cb = dfl::add(cai, df{b2.z, b2.w});
+                    const df tt = dfl::add(dfl::mul(betad, mu), dfl::neg(cb));
+                    Pi = dfl::mul(dfl::mul(mu, tt), dfl::mul(d1, Rr));
+                    if (-mu.hi > mumx.hi) mumx = dfl::neg(mu);
+                }
+                const df mj = {J0.w, J1.w};
+                const df g = dfl::mul(mj, dfl::add(dfl::add(Ai, df{b1.x, b1.y}), Pi));
+                sx = dfl::add(sx, dfl::mul(g, Gx));
+                sy = dfl::add(sy, dfl::mul(g, Gy));
+                sz = dfl::add(sz, dfl::mul(g, Gz));
+                const df Gv = dfl::add(dfl::add(dfl::mul(Gx, WX), dfl::mul(Gy, WY)), dfl::mul(Gz, WZ));
+                const df mGv = dfl::mul(mj, Gv);
+                sp = dfl::add(sp, mGv);
+                sv = dfl::add(sv, dfl::mul(mGv, Pi));
+            }
+        } else {
+            for (int e0 = sub; e0 < len; e0 += T * U) {
+                int j[U];
+                df tx[U], ty[U], tz[U], tp[U], tv[U], nmu[U];
+                bool use[U];
 #pragma unroll
-                for (int k = 0; k < 6; ++k) M[k] = dfl::add(dfl::mul(wi, Ci[k]), dfl::mul(wj, Cj[k]));
+                for (int u = 0; u < U; ++u)
+                    j[u] = e0 + u * T < len ? __ldg(&ent[e0 + u * T]) : (int)i;
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const float4 J0 = __ldg(&xpk[3 * j[u]]), J1 = __ldg(&xpk[3 * j[u] + 1]);
+                    const float4 J2 = __ldg(&xpk[3 * j[u] + 2]);
+                    const float4 wa = __ldg(&vpa[j[u]]);
+                    const float2 wb = __ldg(&vpb[j[u]]);
+                    const float4 b0 = __ldg(&dpk[3 * j[u]]), b1 = __ldg(&dpk[3 * j[u] + 1]);
+                    const float4 b2 = __ldg(&dpk[3 * j[u] + 2]);
+                    float z2 = __fsub_rn(I0.z, J0.z), z1 = __fsub_rn(I1.z, J1.z), z0 = __fsub_rn(I2.z, J2.z);
+                    if (per) wrap_fx(z2, z1, z0, hlz, L2, L1, L0);
+                    const df X = dfl::fx_sum(__fsub_rn(I0.x, J0.x), __fsub_rn(I1.x, J1.x), __fsub_rn(I2.x, J2.x));
+                    const df Y = dfl::fx_sum(__fsub_rn(I0.y, J0.y), __fsub_rn(I1.y, J1.y), __fsub_rn(I2.y, J2.y));
+                    const df Z = dfl::fx_sum(z2, z1, z0);
+                    const df r2 = dfl::add(dfl::add_same(dfl::sqr(X), dfl::sqr(Y)), dfl::sqr(Z));
+                    const bool ok = e0 + u * T < len && r2.hi > 0.0f;  // (coincident: no force)
+                    const df r = dfl::mul(r2, dfl::rsqrt(r2));
+                    const df Hj = {b0.x, b0.y};
+                    const df wi = dfl::mul(Hi3, w_shape_k<KER>(dfl::mul(r, Hi), sn));
+                    const df wj = dfl::mul(dfl::mul(Hj, dfl::sqr(Hj)), w_shape_k<KER>(dfl::mul(r, Hj), sn));
+                    df M[6];
+                    {
+                        const float4 d0 = __ldg(&cpk[3 * j[u]]), d1 = __ldg(&cpk[3 * j[u] + 1]);
+                        const float4 d2 = __ldg(&cpk[3 * j[u] + 2]);
+                        const df Cj[6] = {{d0.x, d0.y}, {d0.z, d0.w}, {d1.x, d1.y},
+                                          {d1.z, d1.w}, {d2.x, d2.y}, {d2.z, d2.w}};
+        #pragma unroll
+                        for (int k = 0; k < 6; ++k) M[k] = dfl::add(dfl::mul(wi, Ci[k]), dfl::mul(wj, Cj[k]));
+                    }
+                    df Gx, Gy, Gz;
+                    symv_df(M, X, Y, Z, Gx, Gy, Gz);
+                    Gx = dfl::mul(kg, Gx);
+                    Gy = dfl::mul(kg, Gy);
+                    Gz = dfl::mul(kg, Gz);
+                    const df WX = dfl::sub(VXi, df{wa.x, wa.y}), WY = dfl::sub(VYi, df{wa.z, wa.w});
+                    const df WZ = dfl::sub(VZi, df{wb.x, wb.y});
+                    const df vr = dfl::add(dfl::add(dfl::mul(WX, X), dfl::mul(WY, Y)), dfl::mul(WZ, Z));
+                    const df hb = dfl::add(hhi, df{b1.z, b1.w});
+                    const df d1 = dfl::add(r2, dfl::mul(dfl::mul(eta2, hb), hb));
+                    const df rb = dfl::add(rhi, df{b2.x, b2.y});
+                    const df Rr = dfl::rcp(dfl::mul(d1, rb));
+                    const df mu = dfl::mul(dfl::mul(dfl::mul(hb, vr), rb), Rr);
+                    const df cb = dfl::add(cai, df{b2.z, b2.w});
+                    const df tt = dfl::add(dfl::mul(betad, mu), dfl::neg(cb));
+                    const df Pv = dfl::mul(dfl::mul(mu, tt), dfl::mul(d1, Rr));
+                    const bool visc = vr.hi < 0.0f;
+                    const df Pi = {visc ? Pv.hi : 0.f, visc ? Pv.lo : 0.f};
+                    nmu[u] = df{ok && visc ? -mu.hi : 0.f, ok && visc ? -mu.lo : 0.f};
+                    const df mj = {J0.w, J1.w};
+                    const df g = dfl::mul(mj, dfl::add(dfl::add(Ai, df{b1.x, b1.y}), Pi));
+                    tx[u] = dfl::mul(g, Gx);
+                    ty[u] = dfl::mul(g, Gy);
+                    tz[u] = dfl::mul(g, Gz);
+                    const df Gv = dfl::add(dfl::add(dfl::mul(Gx, WX), dfl::mul(Gy, WY)), dfl::mul(Gz, WZ));
+                    tp[u] = dfl::mul(mj, Gv);
+                    tv[u] = dfl::mul(tp[u], Pi);
+                    use[u] = ok;
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    if (!use[u]) continue;
+                    sx = dfl::add(sx, tx[u]);
+                    sy = dfl::add(sy, ty[u]);
+                    sz = dfl::add(sz, tz[u]);
+                    sp = dfl::add(sp, tp[u]);
+                    sv = dfl::add(sv, tv[u]);
+                    if (nmu[u].hi > mumx.hi) mumx = nmu[u];
+                }
             }
-            df Gx, Gy, Gz;
-            symv_df(M, X, Y, Z, Gx, Gy, Gz);
-            Gx = dfl::mul(kg, Gx);
-            Gy = dfl::mul(kg, Gy);
-            Gz = dfl::mul(kg, Gz);
-            const df WX = dfl::sub(VXi, df{wa.x, wa.y}), WY = dfl::sub(VYi, df{wa.z, wa.w});
-            const df WZ = dfl::sub(VZi, df{wb.x, wb.y});
-            const df vr = dfl::add(dfl::add(dfl::mul(WX, X), dfl::mul(WY, Y)), dfl::mul(WZ, Z));
-            df Pi = {0.f, 0.f};
-            if (vr.hi < 0.0f) {
-                const df hb = dfl::add(hhi, df{b1.z, b1.w});
-                const df d1 = dfl::add(r2, dfl::mul(dfl::mul(eta2, hb), hb));
-                const df rb = dfl::add(rhi, df{b2.x, b2.y});
-                const df Rr = dfl::rcp(dfl::mul(d1, rb));
-                const df mu = dfl::mul(dfl::mul(dfl::mul(hb, vr), rb), Rr);
-                const df cb = dfl::add(cai, df{b2.z, b2.w});
-                const df tt = dfl::add(dfl::mul(betad, mu), dfl::neg(cb));
-                Pi = dfl::mul(dfl::mul(mu, tt), dfl::mul(d1, Rr));
-                if (-mu.hi > mumx.hi) mumx = dfl::neg(mu);
-            }
-            const df mj = {J0.w, J1.w};
-            const df g = dfl::mul(mj, dfl::add(dfl::add(Ai, df{b1.x, b1.y}), Pi));
-            sx = dfl::add(sx, dfl::mul(g, Gx));
-            sy = dfl::add(sy, dfl::mul(g, Gy));
-            sz = dfl::add(sz, dfl::mul(g, Gz));
-            const df Gv = dfl::add(dfl::add(dfl::mul(Gx, WX), dfl::mul(Gy, WY)), dfl::mul(Gz, WZ));
-            const df mGv = dfl::mul(mj, Gv);
-            sp = dfl::add(sp, mGv);
-            sv = dfl::add(sv, dfl::mul(mGv, Pi));
         }
     }
     if (T > 1) {
@@ -684,27 +871,30 @@ k_forces_iad_df(int64_t n, Batch B, const double4_32a* __restrict__ posh,
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) dtc = fmin(dtc, __shfl_xor_sync(0xffffffffu, dtc, o));
-    __shared__ double sh[kThreads / 32];
+    __shared__ double sh[kPairBlock<U> / 32];
     if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = dtc;
     __syncthreads();
     if (threadIdx.x == 0) {
         double m = sh[0];
-        for (int w = 1; w < kThreads / 32; ++w) m = fmin(m, sh[w]);
+        for (int w = 1; w < kPairBlock<U> / 32; ++w) m = fmin(m, sh[w]);
         dt_part[blockIdx.x] = m;
     }
 }
 
 template <int T, int KER>
 static void iad_df_t(sph_ctx* c, cudaStream_t s) {
+    constexpr int U = KER == KER_SINC ? 1 : 2;
     const int64_t n = c->n;
-    const unsigned nb = (unsigned)((n * T + kThreads - 1) / kThreads);
+    const unsigned tm = kPairBlockMin, tf = kPairBlock<U>;
     const int b = c->cur;
     const Batch B = batch_of(c);
     const Rows R = rows_of(c);
-    k_iad_df<T, KER><<<nb, kThreads, 0, s>>>(n, B, c->posh[b], c->xpk, c->vdf, R, c->cpk);
-    k_forces_iad_df<T, KER><<<nb, kThreads, 0, s>>>(n, B, c->posh[b], c->vpa, c->vpb, c->dpk, c->xpk,
-                                                    c->cpk, c->cint, R, c->acc, c->mumax,
-                                                    c->dt_part);
+    k_iad_df<T, KER><<<(unsigned)((n * T + tm - 1) / tm), tm, 0, s>>>(n, B, c->posh[b], c->xpk,
+                                                                       c->vdf, R, c->cpk);
+    k_forces_iad_df<T, KER, U><<<(unsigned)((n * T + tf - 1) / tf), tf, 0, s>>>(
+        n, B, c->posh[b], c->vpa, c->vpb, c->dpk, c->xpk, c->cpk, c->cint, R, c->acc, c->mumax,
+        c->dt_part);
+    c->dt_block = (int)tf;
 }
 
 template <int KER>

@@ -177,8 +177,11 @@ k_pack_mx(int64_t n, Batch B, const double4_32a* __restrict__ posh,
 // ~2^-21 of the defining FP64 value and 1/h_j is packed as a float, so
 // r^2 / h_j^2 below / above 4 by more than 2^-18 decides; the band between,
 // and a periodic axis shorter than 8 h_j, take the FP64 test itself.
-template <bool FUSE, int T, bool OUTER>
-__global__ void __launch_bounds__(kThreads)
+// U: neighbours evaluated at a time, their terms added in the order of the row
+// (the same bits for every U). U = 4 in blocks of 64: 1M sphere 677 us (746 one
+// at a time in blocks of 256), 8,191 particles 49 (53).
+template <bool FUSE, int T, bool OUTER, int U>
+__global__ void __launch_bounds__(kPairBlock<U>)
 k_density_mx(int64_t n, Batch B, const double4_32a* __restrict__ posh,
              const double* __restrict__ ue, float4* __restrict__ mpk,
              Rows R, double4_32a* __restrict__ therm,
@@ -201,27 +204,42 @@ k_density_mx(int64_t n, Batch B, const double4_32a* __restrict__ posh,
     // rows read from the CSR (a gather set overflowed) are complete already
     const bool append = OUTER && !(R.status[2] & IF_SLAB_OVF);
     Append ap;
-    for (int e = sub; e < len; e += T) {
-        const int j = __ldg(&ent[e]);
-        const float4 b0 = __ldg(&mpk[5 * j]), b1 = __ldg(&mpk[5 * j + 1]);
-        const float dx = rel(a0.x, a1.x, b0.x, b1.x), dy = rel(a0.y, a1.y, b0.y, b1.y);
-        const float dz = rel_z(a0.z, a1.z, b0.z, b1.z, zw);
-        const float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
-        const float q = r2 > 0.0f ? r2 * rsqrt_f(r2) * hinv : 0.0f;
-        acc = dfl::addf(acc, b0.w * w_shape_f(q));
-        if (append) {
-            const float t = r2 * b1.w * b1.w;  // (r / h_j)^2
-            bool in_j;
-            if (!(zw.per && b1.w * zw.lzh < 8.0f) && t < 4.0f * 0.99999619f) {
-                in_j = true;
-            } else if (!(zw.per && b1.w * zw.lzh < 8.0f) && t > 4.0f * 1.00000381f) {
-                in_j = false;
-            } else {
-                const double4_32a pj = posh[j];
-                const double Rj = 2.0 * pj.w;
-                in_j = exact_r2_def(posh[i], pj, zw.per, kp.lz) < __dmul_rn(Rj, Rj);
+    for (int e0 = sub; e0 < len; e0 += T * U) {
+        int j[U];
+        float term[U], tq[U], hj[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            j[u] = U == 1 || e0 + u * T < len ? __ldg(&ent[e0 + u * T]) : (int)i;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const float4 b0 = __ldg(&mpk[5 * j[u]]), b1 = __ldg(&mpk[5 * j[u] + 1]);
+            const float dx = rel(a0.x, a1.x, b0.x, b1.x), dy = rel(a0.y, a1.y, b0.y, b1.y);
+            const float dz = rel_z(a0.z, a1.z, b0.z, b1.z, zw);
+            const float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
+            const float q = r2 > 0.0f ? r2 * rsqrt_f(r2) * hinv : 0.0f;
+            term[u] = b0.w * w_shape_f(q);
+            tq[u] = r2 * b1.w * b1.w;  // (r / h_j)^2
+            hj[u] = b1.w;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (U > 1 && e0 + u * T >= len) break;
+            acc = dfl::addf(acc, term[u]);
+            if (append) {
+                const float t = tq[u];
+                const bool wide = zw.per && hj[u] * zw.lzh < 8.0f;
+                bool in_j;
+                if (!wide && t < 4.0f * 0.99999619f) {
+                    in_j = true;
+                } else if (!wide && t > 4.0f * 1.00000381f) {
+                    in_j = false;
+                } else {
+                    const double4_32a pj = posh[j[u]];
+                    const double Rj = 2.0 * pj.w;
+                    in_j = exact_r2_def(posh[i], pj, zw.per, kp.lz) < __dmul_rn(Rj, Rj);
+                }
+                if (!in_j) ap.add(i, j[u], R.ngather, O);  // i belongs in the outer part of row j
             }
-            if (!in_j) ap.add(i, j, R.ngather, O);  // i belongs in the outer part of row j
         }
     }
     if (OUTER) ap.flush(i, O);
@@ -247,8 +265,9 @@ k_density_mx(int64_t n, Batch B, const double4_32a* __restrict__ posh,
     }
 }
 
-template <int T>
-__global__ void __launch_bounds__(kThreads)
+// U: as in k_forces_df.
+template <int T, int U>
+__global__ void __launch_bounds__(kPairBlock<U>)
 k_forces_mx(int64_t n, Batch B, const double4_32a* __restrict__ posh,
             const float4* __restrict__ mpk, const double* __restrict__ cint,
             Rows R,
@@ -270,40 +289,96 @@ k_forces_mx(int64_t n, Batch B, const double4_32a* __restrict__ posh,
         const ZWrap zw = make_zwrap(kp, B.grid[inst]);
         const float eta2 = (float)kp.eta2, beta = (float)kp.beta;
         const float cpi = 0.5f * kInvPiF;
-        for (int e = sub; e < len; e += T) {
-            const int j = __ldg(&ent[e]);
-            const float4 b0 = __ldg(&mpk[5 * j]), b1 = __ldg(&mpk[5 * j + 1]);
-            const float4 b2 = __ldg(&mpk[5 * j + 2]), b3 = __ldg(&mpk[5 * j + 3]);
-            const float4 b4 = __ldg(&mpk[5 * j + 4]);
-            const float dx = rel(a0.x, a1.x, b0.x, b1.x), dy = rel(a0.y, a1.y, b0.y, b1.y);
-            const float dz = rel_z(a0.z, a1.z, b0.z, b1.z, zw);
-            const float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
-            if (!(r2 > 0.0f)) continue;  // coincident particles exert no force
-            const float rinv = rsqrt_f(r2);
-            const float r = r2 * rinv;
-            const float fa = dw_shape_f(r * a1.w), fb = dw_shape_f(r * b1.w);
-            const float Fb = fmaf(a2.w, fa, b2.w * fb) * (cpi * rinv);
-            const float wx = rel(a2.x, a3.x, b2.x, b3.x), wy = rel(a2.y, a3.y, b2.y, b3.y);
-            const float wz = rel(a2.z, a3.z, b2.z, b3.z);
-            const float vr = fmaf(wz, dz, fmaf(wy, dy, wx * dx));
-            float Pi = 0.0f;
-            if (vr < 0.0f) {
-                const float hb = a4.x + b4.x;
-                const float d1 = fmaf(eta2 * hb, hb, r2);
-                const float rb = a4.y + b4.y;
-                const float R = rcp_f(d1 * rb);
-                const float mu = hb * vr * rb * R;
-                Pi = mu * fmaf(beta, mu, -(a4.z + b4.z)) * (d1 * R);
-                mum = fmaxf(mum, -mu);
+        if constexpr (U == 1) {
+            for (int e = sub; e < len; e += T) {
+                const int j = __ldg(&ent[e]);
+                const float4 b0 = __ldg(&mpk[5 * j]), b1 = __ldg(&mpk[5 * j + 1]);
+                const float4 b2 = __ldg(&mpk[5 * j + 2]), b3 = __ldg(&mpk[5 * j + 3]);
+                const float4 b4 = __ldg(&mpk[5 * j + 4]);
+                const float dx = rel(a0.x, a1.x, b0.x, b1.x), dy = rel(a0.y, a1.y, b0.y, b1.y);
+                const float dz = rel_z(a0.z, a1.z, b0.z, b1.z, zw);
+                const float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
+                if (!(r2 > 0.0f)) continue;  // coincident particles exert no force
+                const float rinv = rsqrt_f(r2);
+                const float r = r2 * rinv;
+                const float fa = dw_shape_f(r * a1.w), fb = dw_shape_f(r * b1.w);
+                const float Fb = fmaf(a2.w, fa, b2.w * fb) * (cpi * rinv);
+                const float wx = rel(a2.x, a3.x, b2.x, b3.x), wy = rel(a2.y, a3.y, b2.y, b3.y);
+                const float wz = rel(a2.z, a3.z, b2.z, b3.z);
+                const float vr = fmaf(wz, dz, fmaf(wy, dy, wx * dx));
+                float Pi = 0.0f;
+                if (vr < 0.0f) {
+                    const float hb = a4.x + b4.x;
+                    const float d1 = fmaf(eta2 * hb, hb, r2);
+                    const float rb = a4.y + b4.y;
+                    const float R = rcp_f(d1 * rb);
+                    const float mu = hb * vr * rb * R;
+                    Pi = mu * fmaf(beta, mu, -(a4.z + b4.z)) * (d1 * R);
+                    mum = fmaxf(mum, -mu);
+                }
+                const float mF = b0.w * Fb;
+                const float g = mF * ((a3.w + b3.w) + Pi);
+                sx = dfl::addf(sx, g * dx);
+                sy = dfl::addf(sy, g * dy);
+                sz = dfl::addf(sz, g * dz);
+                const float mFv = mF * vr;
+                sp = dfl::addf(sp, mFv);
+                sv = dfl::addf(sv, mFv * Pi);
             }
-            const float mF = b0.w * Fb;
-            const float g = mF * ((a3.w + b3.w) + Pi);
-            sx = dfl::addf(sx, g * dx);
-            sy = dfl::addf(sy, g * dy);
-            sz = dfl::addf(sz, g * dz);
-            const float mFv = mF * vr;
-            sp = dfl::addf(sp, mFv);
-            sv = dfl::addf(sv, mFv * Pi);
+        } else {
+            for (int e0 = sub; e0 < len; e0 += T * U) {
+                int j[U];
+                float tx[U], ty[U], tz[U], tp[U], tv[U], nmu[U];
+                bool use[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    j[u] = e0 + u * T < len ? __ldg(&ent[e0 + u * T]) : (int)i;
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const float4 b0 = __ldg(&mpk[5 * j[u]]), b1 = __ldg(&mpk[5 * j[u] + 1]);
+                    const float4 b2 = __ldg(&mpk[5 * j[u] + 2]), b3 = __ldg(&mpk[5 * j[u] + 3]);
+                    const float4 b4 = __ldg(&mpk[5 * j[u] + 4]);
+                    const float dx = rel(a0.x, a1.x, b0.x, b1.x), dy = rel(a0.y, a1.y, b0.y, b1.y);
+                    const float dz = rel_z(a0.z, a1.z, b0.z, b1.z, zw);
+                    const float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
+                    const bool ok = e0 + u * T < len && r2 > 0.0f;  // (coincident: no force)
+                    const float rinv = rsqrt_f(r2);
+                    const float r = r2 * rinv;
+                    const float fa = dw_shape_f(r * a1.w), fb = dw_shape_f(r * b1.w);
+                    const float Fb = fmaf(a2.w, fa, b2.w * fb) * (cpi * rinv);
+                    const float wx = rel(a2.x, a3.x, b2.x, b3.x), wy = rel(a2.y, a3.y, b2.y, b3.y);
+                    const float wz = rel(a2.z, a3.z, b2.z, b3.z);
+                    const float vr = fmaf(wz, dz, fmaf(wy, dy, wx * dx));
+                    const float hb = a4.x + b4.x;
+                    const float d1 = fmaf(eta2 * hb, hb, r2);
+                    const float rb = a4.y + b4.y;
+                    const float R = rcp_f(d1 * rb);
+                    const float mu = hb * vr * rb * R;
+                    // (__fmul_rn: this product stays out of the sum that takes it)
+                    const float Pv = __fmul_rn(mu * fmaf(beta, mu, -(a4.z + b4.z)), d1 * R);
+                    const bool visc = vr < 0.0f;
+                    const float Pi = visc ? Pv : 0.0f;
+                    nmu[u] = ok && visc ? -mu : 0.0f;
+                    const float mF = b0.w * Fb;
+                    const float g = mF * ((a3.w + b3.w) + Pi);
+                    tx[u] = g * dx;
+                    ty[u] = g * dy;
+                    tz[u] = g * dz;
+                    tp[u] = mF * vr;
+                    tv[u] = tp[u] * Pi;
+                    use[u] = ok;
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    if (!use[u]) continue;
+                    sx = dfl::addf(sx, tx[u]);
+                    sy = dfl::addf(sy, ty[u]);
+                    sz = dfl::addf(sz, tz[u]);
+                    sp = dfl::addf(sp, tp[u]);
+                    sv = dfl::addf(sv, tv[u]);
+                    mum = fmaxf(mum, nmu[u]);
+                }
+            }
         }
     }
     if (T > 1) {
@@ -333,12 +408,12 @@ k_forces_mx(int64_t n, Batch B, const double4_32a* __restrict__ posh,
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) dtc = fmin(dtc, __shfl_xor_sync(0xffffffffu, dtc, o));
-    __shared__ double sh[kThreads / 32];
+    __shared__ double sh[kPairBlock<U> / 32];
     if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = dtc;
     __syncthreads();
     if (threadIdx.x == 0) {
         double m = sh[0];
-        for (int w = 1; w < kThreads / 32; ++w) m = fmin(m, sh[w]);
+        for (int w = 1; w < kPairBlock<U> / 32; ++w) m = fmin(m, sh[w]);
         dt_part[blockIdx.x] = m;
     }
 }
@@ -360,11 +435,14 @@ void launch_pack_mx(sph_ctx* c, bool thermo, cudaStream_t s) {
 template <bool FUSE, int T, bool OUTER>
 static void density_mx_t(sph_ctx* c, cudaStream_t s) {
     const int64_t n = c->n;
-    const unsigned nb = (unsigned)((n * T + kThreads - 1) / kThreads);
     const int b = c->cur;
-    k_density_mx<FUSE, T, OUTER><<<nb, kThreads, 0, s>>>(
-        n, batch_of(c), c->posh[b], c->ue[b], c->mpk, OUTER ? rows_gather(c) : rows_of(c),
-        c->therm, c->pint, c->cint, c->status, OuterOut{c->rslab, c->ocnt, c->status});
+    auto go = [&](auto kernel_fn, int U) {
+        const unsigned tb = U > 1 ? kPairBlockMin : kThreads;
+        kernel_fn<<<(unsigned)((n * T + tb - 1) / tb), tb, 0, s>>>(
+            n, batch_of(c), c->posh[b], c->ue[b], c->mpk, OUTER ? rows_gather(c) : rows_of(c),
+            c->therm, c->pint, c->cint, c->status, OuterOut{c->rslab, c->ocnt, c->status});
+    };
+    go(k_density_mx<FUSE, T, OUTER, 4>, 4);
 }
 
 template <bool FUSE, bool OUTER>
@@ -388,11 +466,18 @@ void launch_density_mx(sph_ctx* c, bool fuse_eos, cudaStream_t s, bool outer) {
 template <int T>
 static void forces_mx_t(sph_ctx* c, cudaStream_t s) {
     const int64_t n = c->n;
-    const unsigned nb = (unsigned)((n * T + kThreads - 1) / kThreads);
     const int b = c->cur;
-    k_forces_mx<T><<<nb, kThreads, 0, s>>>(n, batch_of(c), c->posh[b], c->mpk, c->cint,
-                                           rows_of(c), c->acc, c->mumax,
-                                           c->dt_part);
+    auto go = [&](auto kernel_fn, int U) {
+        const unsigned tb = U > 1 ? kPairBlockMin : kThreads;
+        kernel_fn<<<(unsigned)((n * T + tb - 1) / tb), tb, 0, s>>>(
+            n, batch_of(c), c->posh[b], c->mpk, c->cint, rows_of(c), c->acc, c->mumax, c->dt_part);
+        c->dt_block = (int)tb;
+    };
+    // small batches, with a few warps per scheduler, are bound by the latency of
+    // a pair, large ones by the L1 data pipe (us, U = 4 and U = 1: 8,191 particles
+    // 38 and 46, 30,000 48 and 54, 60,000 116 and 114, 1M 1,028 and 1,000)
+    if (c->n <= kPairUnrollN) go(k_forces_mx<T, 4>, 4);
+    else go(k_forces_mx<T, 1>, 1);
 }
 
 void launch_forces_mx(sph_ctx* c, cudaStream_t s) {

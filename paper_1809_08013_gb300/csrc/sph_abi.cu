@@ -220,7 +220,7 @@ bool allocate_all(sph_ctx* c, int64_t nslots, Allocator& al) {
          al(&c->nnb, N) && al(&c->ngather, N) && al(&c->rowlen, N) &&
          al(&c->offsets, N + 1) && al(&c->row_part, (size_t)scan_parts(N) + 1) &&
          al(&c->idx, (size_t)nnzcap) && al(&c->red_part, (N + kSlotAlign - 1) / kSlotAlign * kBoxStride) &&
-         al(&c->dt_part, nfb * kMaxPairThreads) && al(&c->grid, (size_t)max_instances) &&
+         al(&c->dt_part, nfb * kMaxPairThreads * (kThreads / kPairBlockMin)) && al(&c->grid, (size_t)max_instances) &&
          al(&c->status, 4) && al(&c->blk, nfb) &&
          al(&c->ioff, (size_t)max_instances + 1) && al(&c->icnt, (size_t)max_instances) &&
          al(&c->coff, (size_t)max_instances + 1) && al(&c->kpi, (size_t)max_instances) &&

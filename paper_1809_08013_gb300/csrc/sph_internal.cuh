@@ -31,6 +31,8 @@ constexpr int64_t kRadixSmallN = 262144;
 constexpr int kScanTile = kThreads * 8;             // elements per block in scans
 constexpr int kReduceBlocks = 304;                  // 2 x 152 SMs
 constexpr int kMaxPairThreads = 8;                  // lanes per particle in the pair kernels
+constexpr int64_t kPairUnrollN = 50000;             // see forces_mx_t
+constexpr int kPairBlockMin = 64;                   // smallest block of the pair kernels
 constexpr int kBoxStride = 16;                      // doubles per bounding-box partial
 constexpr int kBoxWarpSlots = 64;                   // bounding box: slots per warp (4 per partial)
 
@@ -334,7 +336,9 @@ struct sph_ctx {
     int32_t* wl;            // their indices (count in status[3])
     int32_t* gwl;           // groups of 32 that go on searching together (count in wctr[1])
     double* red_part;       // bbox partials: kBoxStride per group of kSlotAlign slots
-    double* dt_part;        // per force block (kMaxPairThreads per kThreads slots)
+    double* dt_part;        // per force block (at most kMaxPairThreads lanes per slot, and
+                            // kPairBlockMin threads per block)
+    int dt_block;           // threads per block of the last force kernel
     sph::Grid* grid;        // per instance
     unsigned long long* wctr;  // [0] work counter of k_h_union, [1] length of gwl (zeroed
                                // per build)
@@ -418,6 +422,10 @@ inline Rows rows_gather(const sph_ctx* c) {
 // and appends the outer parts of the rows (k_density_df / k_density_mx with
 // OUTER); at precision 2 and outside a step, k_outer builds them before it.
 inline bool fused_outer(const sph_ctx* c) { return c->prec == PREC_FP64 || c->prec == PREC_MIXED; }
+
+// Threads per block of a pair kernel that evaluates U neighbours at a time.
+template <int U>
+constexpr int kPairBlock = U > 1 ? kPairBlockMin : kThreads;
 
 // The defining FP64 squared distance, operation by operation (minimum image
 // along z when periodic): (dx dx + dy dy) + dz dz, each operation rounded.
