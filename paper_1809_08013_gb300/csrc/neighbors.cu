@@ -25,6 +25,8 @@
 // iteration count never stalls other particles.
 #include <math_constants.h>
 
+#include <cooperative_groups.h>
+
 #include <algorithm>
 #include <type_traits>
 
@@ -212,8 +214,8 @@ struct FlatCells {
 template <int PRUNE, class Chunk>
 __device__ __forceinline__ void particle_pass(const Grid* __restrict__ g,
                                               const int2* __restrict__ cells,
-                                              const unsigned long long* __restrict__ cell_hmax,
-                                              const float4* __restrict__ fpos, const float4& q,
+                                              const unsigned long long* cell_hmax,
+                                              const float4* fpos, const float4& q,
                                               float R, long long hib, int* delta, Chunk&& chunk) {
     const int lane = threadIdx.x & 31;
     int x0, x1, y0, y1, z0, z1;
@@ -241,7 +243,7 @@ __device__ __forceinline__ void particle_pass(const Grid* __restrict__ g,
             if (PRUNE && cnt > 0) {
                 float reach = R;
                 if (PRUNE == 2) {
-                    const long long hcb = (long long)__ldg(&cell_hmax[lin]);
+                    const long long hcb = (long long)cell_hmax[lin];
                     reach = reach_f32(__longlong_as_double(hcb > hib ? hcb : hib));
                 }
                 const float gx = axis_gap(q.x, kx, g, 0), gy = axis_gap(q.y, ky, g, 1);
@@ -250,14 +252,16 @@ __device__ __forceinline__ void particle_pass(const Grid* __restrict__ g,
             }
         }
         const FlatCells F(cnt, start, delta);
+        // (PRUNE = 2: cell_hmax and fpos.w were written by this same kernel)
+        auto load = [&](int j) { return PRUNE == 2 ? fpos[j] : __ldg(&fpos[j]); };
         int jn = F.total > 0 ? F.slot(0, F.total, delta) : -1;
-        float4 fn = jn >= 0 ? __ldg(&fpos[jn]) : make_float4(0.f, 0.f, 0.f, 0.f);
+        float4 fn = jn >= 0 ? load(jn) : make_float4(0.f, 0.f, 0.f, 0.f);
         for (int t0 = 0; t0 < F.total; t0 += 32) {
             const int j = jn;
             const float4 f = fn;
             if (t0 + 32 < F.total) {
                 jn = F.slot(t0 + 32, F.total, delta);
-                if (jn >= 0) fn = __ldg(&fpos[jn]);
+                if (jn >= 0) fn = load(jn);
             }
             chunk(j >= 0, j, f);
         }
@@ -392,6 +396,27 @@ __device__ __forceinline__ void cluster_walk(const Cluster& K, const Grid* __res
         seen += cl.total;
         __syncwarp();
     }
+}
+
+// (2 h)^2 in the length unit of the double-float pair kernels, as a float within
+// 2^-22 (integer and FP32 operations only), for the spare float of the position
+// pack; NaN (the exact test alone decides) where the periodic wrap could decide
+// differently, or for an h whose exponent cannot be moved.
+__device__ __forceinline__ float pair_reach2(double h, const Grid* __restrict__ g) {
+    const long long b = __double_as_longlong(h);
+    if (b == 0) return 0.0f;
+    if (b < (64ll << 52) || b > kHMaxBits) return CUDART_NAN_F;
+    float lo, hi;
+    f32_bounds(h, lo, hi);
+    if (g->periodic_z && 2.0f * hi > 0.2499f * g->lzf) return CUDART_NAN_F;
+    f32_bounds(__longlong_as_double(b + ((long long)(1 - g->uL) << 52)), lo, hi);
+    return lo * lo;
+}
+
+// What a finished search leaves in the pack of particle i (precision 0).
+__device__ __forceinline__ void write_reach2(float4* __restrict__ xpk, int64_t i, double h,
+                                             const Grid* __restrict__ g, const KParams& kp) {
+    if (kp.precision == PREC_FP64) xpk[3 * i + 2].w = pair_reach2(h, g);
 }
 
 // ------------------------------------------------------------ h search
@@ -569,7 +594,7 @@ __device__ __forceinline__ void union_group(
     int32_t* __restrict__ rslab, double* __restrict__ hs_lo, double* __restrict__ hs_hi,
     int32_t* __restrict__ hs_it, int32_t* __restrict__ wl, unsigned* __restrict__ status,
     float4* st, int* sidx, int2* recb, const int32_t* __restrict__ order,
-    int32_t* __restrict__ lst, LMeta* __restrict__ lmeta) {
+    int32_t* __restrict__ lst, LMeta* __restrict__ lmeta, float4* __restrict__ xpk) {
     const int lane = threadIdx.x & 31;
     const int64_t i = i0 + lane;
     const int inst = slot_inst(B, i0);
@@ -834,6 +859,7 @@ __device__ __forceinline__ void union_group(
     }
     if (deferred || listed) return;
     posh[i].w = h;
+    write_reach2(xpk, i, h, g, kp);
     nnb[i] = cnt;
     ngather[i] = cnt;
     if (cnt > kGSlab) atomicOr(&status[2], (unsigned)IF_SLAB_OVF);
@@ -857,7 +883,7 @@ k_h_lists(int64_t n, Batch B, double4_32a* posh, const float4* __restrict__ fpos
           double* __restrict__ hs_lo, double* __restrict__ hs_hi, int32_t* __restrict__ hs_it,
           int32_t* __restrict__ wl, unsigned* __restrict__ status,
           const int32_t* __restrict__ order, const int32_t* __restrict__ lst,
-          const LMeta* __restrict__ lmeta) {
+          const LMeta* __restrict__ lmeta, float4* __restrict__ xpk) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const int inst = slot_inst(B, i);
@@ -906,6 +932,7 @@ k_h_lists(int64_t n, Batch B, double4_32a* posh, const float4* __restrict__ fpos
         return;
     }
     posh[i].w = h;
+    write_reach2(xpk, i, h, g, kp);
     nnb[i] = cnt;
     ngather[i] = cnt;
     if (cnt > kGSlab) atomicOr(&status[2], (unsigned)IF_SLAB_OVF);
@@ -977,7 +1004,8 @@ k_h_count(int64_t n, Batch B, double4_32a* posh, const float4* __restrict__ fpos
           const int2* __restrict__ cells, int32_t* __restrict__ nnb, int32_t* __restrict__ ngather,
           int32_t* __restrict__ rslab, double* __restrict__ hs_lo, double* __restrict__ hs_hi,
           int32_t* __restrict__ hs_it, int32_t* __restrict__ wl, int32_t* __restrict__ gwl,
-          unsigned* __restrict__ status, unsigned long long* __restrict__ wctr) {
+          unsigned* __restrict__ status, unsigned long long* __restrict__ wctr,
+          float4* __restrict__ xpk) {
     constexpr int kCh = kCountChunks<W>, kCap = kCountCap<W>;
     __shared__ CountSmem<W> s_w[W];
     __shared__ int s_cnt[W][32];
@@ -1256,6 +1284,7 @@ k_h_count(int64_t n, Batch B, double4_32a* posh, const float4* __restrict__ fpos
     nnb[i] = cnt;
     ngather[i] = cnt;
     if (!valid) return;
+    write_reach2(xpk, i, h, g, kp);
     if (cnt > kGSlab) atomicOr(&status[2], (unsigned)IF_SLAB_OVF);
     if (!conv) {
         atomicOr(&status[0], (unsigned)ST_HNOCONV);
@@ -1275,7 +1304,7 @@ k_h_union(int64_t n, Batch B, double4_32a* posh, const float4* __restrict__ fpos
           int32_t* __restrict__ wl, unsigned* __restrict__ status,
           unsigned long long* __restrict__ wctr, int2* __restrict__ recs,
           const int32_t* __restrict__ order, int32_t* __restrict__ lst,
-          LMeta* __restrict__ lmeta, const int32_t* __restrict__ gwl) {
+          LMeta* __restrict__ lmeta, const int32_t* __restrict__ gwl, float4* __restrict__ xpk) {
     __shared__ float4 s_f[kThreads / 32][32];
     __shared__ int s_i[kThreads / 32][32];
     const int warp = threadIdx.x >> 5;
@@ -1290,7 +1319,7 @@ k_h_union(int64_t n, Batch B, double4_32a* posh, const float4* __restrict__ fpos
         union_group<LISTS>(gi * 32, n, B, posh, fpos, cells, nnb, ngather, rslab, hs_lo, hs_hi, hs_it,
                     wl, status, s_f[warp], s_i[warp],
                     recs + ((int64_t)(blockIdx.x * (kThreads / 32) + warp) * 32 + lane) * kRec,
-                    order, lst, lmeta);
+                    order, lst, lmeta, xpk);
     }
 }
 
@@ -1351,7 +1380,7 @@ k_h_iterate(Batch B, double4_32a* posh, const float4* __restrict__ fpos,
             const double* __restrict__ hs_hi, const int32_t* __restrict__ hs_it,
             const int32_t* __restrict__ wl, unsigned* __restrict__ status,
             const int32_t* __restrict__ order, const int32_t* __restrict__ lst,
-            const LMeta* __restrict__ lmeta) {
+            const LMeta* __restrict__ lmeta, float4* __restrict__ xpk) {
     __shared__ int s_delta[kThreads / 32][32];
     __shared__ int2 s_rec[kThreads / 32][kRecW];  // (FP32 r^2 bits, j)
     const int warp = threadIdx.x >> 5;
@@ -1494,6 +1523,7 @@ k_h_iterate(Batch B, double4_32a* posh, const float4* __restrict__ fpos,
         __syncwarp();  // the records are reused by this warp's next particle
         if (lane == 0) {
             posh[i].w = h;
+            write_reach2(xpk, i, h, g, kp);
             nnb[i] = cnt;
             ngather[i] = cnt;
             if (cnt > kGSlab) atomicOr(&status[2], (unsigned)IF_SLAB_OVF);
@@ -1505,61 +1535,23 @@ k_h_iterate(Batch B, double4_32a* posh, const float4* __restrict__ fpos,
     }
 }
 
-// Per-particle FP32 thresholds at the final h, and (2h)^2 in the length unit
-// of the double-float pair kernels in the spare float of the position pack
-// (NaN where the periodic wrap could decide differently: exact test only).
-__global__ void __launch_bounds__(kThreads)
-k_finalize_h(int64_t n, Batch B, const double4_32a* __restrict__ posh,
-             float4* __restrict__ fpos, float* __restrict__ tin, int32_t* __restrict__ ocnt,
-             float4* __restrict__ xpk) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    ocnt[i] = 0;
+// FP32 thresholds of particle i at its final h, for the kernels that look at
+// pairs from both sides (k_outer, the CSR fallback).
+__device__ __forceinline__ void write_thresholds(int64_t i, const Batch& B,
+                                                 const double4_32a* __restrict__ posh,
+                                                 float4* __restrict__ fpos, float* __restrict__ tin) {
     const int inst = slot_inst(B, i);
     if (!slot_real(B, inst, i)) return;
-    const Grid* g = B.grid + inst;
-    const double h = posh[i].w;
-    const Thr t = thresholds(2.0 * h, g);
+    const Thr t = thresholds(2.0 * posh[i].w, B.grid + inst);
     fpos[i].w = t.tout;
     tin[i] = t.tin;
-    const double R = 2.0 * h * p2d(-g->uL);
-    xpk[3 * i + 2].w = (g->periodic_z && 2.0 * h > 0.25 * g->lz) ? CUDART_NAN_F : (float)(R * R);
 }
 
-// Per-cell max h, and the instance's max (one atomic per block); blockIdx.y
-// is the instance.
 __global__ void __launch_bounds__(kThreads)
-k_cell_hmax(Batch B, Grid* gw, const int2* __restrict__ cells,
-            const double4_32a* __restrict__ posh, unsigned long long* __restrict__ cell_hmax) {
-    const int inst = blockIdx.y;
-    const long long nc = B.grid[inst].ncells, cb = B.grid[inst].cbase;
-    cells += cb;
-    cell_hmax += cb;
-    long long bmax = 0;  // bits of positive doubles order like their values
-    for (long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x; c < nc;
-         c += (long long)gridDim.x * blockDim.x) {
-        const int2 se = cells[c];
-        long long m = 0;
-        for (int k = se.x; k < se.y; ++k) {
-            const long long b = __double_as_longlong(posh[k].w);
-            m = (b > m && b <= kHMaxBits) ? b : m;  // h outside the geometry range: not counted
-        }
-        cell_hmax[c] = (unsigned long long)m;
-        bmax = m > bmax ? m : bmax;
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const long long v = __shfl_xor_sync(kFull, bmax, o);
-        bmax = v > bmax ? v : bmax;
-    }
-    __shared__ long long sh[kThreads / 32];
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = bmax;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        long long m = sh[0];
-        for (int w = 1; w < kThreads / 32; ++w) m = sh[w] > m ? sh[w] : m;
-        atomicMax(&gw[inst].hmax_bits, (unsigned long long)m);
-    }
+k_thresholds(int64_t n, Batch B, const double4_32a* __restrict__ posh, float4* __restrict__ fpos,
+             float* __restrict__ tin) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) write_thresholds(i, B, posh, fpos, tin);
 }
 
 // ------------------------------------------------------------ CSR
@@ -1687,26 +1679,16 @@ k_compose(int64_t n, const int32_t* __restrict__ rowlen, const int32_t* __restri
 // Fallback (a row overflowed a slab): the full two-pass build below.
 // FILL = false: rowlen[i] = |S_i|, ngather[i] = |N_i|.
 // FILL = true : write row i at offsets[i] (N_i first) with ballot-compacted,
-//               coalesced stores; nothing is written when the total exceeds
-//               the capacity (status bit raised).
+//               coalesced stores.
 // A cell is visited when its box lies within 2 max(h_i, max h of the cell).
 template <bool FILL>
-__global__ void __launch_bounds__(kThreads)
-k_csr(int64_t n, Batch B, const double4_32a* __restrict__ posh,
-      const float4* __restrict__ fpos, const float* __restrict__ tin,
-      const int2* __restrict__ cells, const unsigned long long* __restrict__ cell_hmax,
-      int32_t* __restrict__ rowlen, int32_t* __restrict__ ngather,
-      const int64_t* __restrict__ offsets, int32_t* __restrict__ idx, int64_t nnzcap,
-      unsigned* __restrict__ status, unsigned mask) {
-    __shared__ int s_delta[kThreads / 32][32];
-    const int warp = threadIdx.x >> 5;
+__device__ __forceinline__ void csr_rows(
+    int64_t n, const Batch& B, const double4_32a* __restrict__ posh, const float4* fpos,
+    const float* tin, const int2* __restrict__ cells, const unsigned long long* cell_hmax,
+    int32_t* rowlen, int32_t* ngather, const int64_t* offsets, int32_t* __restrict__ idx,
+    int* delta) {
     const int lane = threadIdx.x & 31;
-    if (!(status[2] & mask)) return;  // the slab path built the list
     const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (FILL && offsets[n] > nnzcap) {
-        if (gw == 0 && lane == 0) atomicOr(&status[0], (unsigned)ST_CAPACITY);
-        return;
-    }
     const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
     for (int64_t i = gw; i < n; i += nwarps) {  // persistent: one warp per particle in turn
     const int inst = slot_inst(B, i);
@@ -1724,7 +1706,7 @@ k_csr(int64_t n, Batch B, const double4_32a* __restrict__ posh,
     const float4 fi = fpos[i];
     const float tin_i = tin[i];
     const long long hib = __double_as_longlong(pi.w);
-    const long long hgb = (long long)g->hmax_bits;
+    const long long hgb = (long long)*(volatile const unsigned long long*)&g->hmax_bits;
     const float Rbig = reach_f32(__longlong_as_double(hgb > hib ? hgb : hib));
     double R2i = -1.0;
     const unsigned lt = (1u << lane) - 1u;
@@ -1735,7 +1717,7 @@ k_csr(int64_t n, Batch B, const double4_32a* __restrict__ posh,
         po_end = offsets[i + 1];
     }
     int cg = 0, co = 0;
-    particle_pass<2>(g, cl, chm, fpos, fi, Rbig, hib, s_delta[warp],
+    particle_pass<2>(g, cl, chm, fpos, fi, Rbig, hib, delta,
                         [&](bool valid, int j, const float4& fj) {
         bool in_i = false, in_j = false;
         if (valid && j != i) {
@@ -1750,7 +1732,7 @@ k_csr(int64_t n, Batch B, const double4_32a* __restrict__ posh,
                 in_i = er2 < R2i;
             }
             if (!in_i && r2f <= fj.w) {
-                if (r2f < __ldg(&tin[j])) {
+                if (r2f < tin[j]) {
                     in_j = true;
                 } else {
                     const double4_32a pj = posh[j];
@@ -1781,33 +1763,133 @@ k_csr(int64_t n, Batch B, const double4_32a* __restrict__ posh,
     }
 }
 
+// The whole fallback in one cooperative kernel: thresholds and the cells' max
+// h, row lengths, their scan, rows, with grid barriers between. Without the
+// flag every block returns at once: a step launches this twice, where the
+// passes and the scan as kernels of their own made ten launches that did
+// nothing (and two more kernels prepared in every step what only they read).
+__global__ void __launch_bounds__(kThreads)
+k_csr_fallback(int64_t n, int ninst, Batch B, Grid* gw_, const double4_32a* __restrict__ posh,
+               float4* fpos, float* tin, const int2* __restrict__ cells,
+               unsigned long long* cell_hmax, int32_t* rowlen, int32_t* ngather, int64_t* offsets,
+               int64_t* part, int32_t* __restrict__ idx, int64_t nnzcap, unsigned* status,
+               unsigned mask) {
+    if (!(*(volatile unsigned*)&status[2] & mask)) return;  // the slab path built the list
+    __shared__ int s_delta[kThreads / 32][32];
+    __shared__ int64_t s_sum[kThreads / 32];
+    const cooperative_groups::grid_group grid = cooperative_groups::this_grid();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t nt = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = t0; i < n; i += nt) write_thresholds(i, B, posh, fpos, tin);
+    for (int k = 0; k < ninst; ++k) {
+        const long long nc = B.grid[k].ncells, cb = B.grid[k].cbase;
+        long long most = 0;  // bits of positive doubles order like their values
+        for (long long c = t0; c < nc; c += nt) {
+            const int2 se = cells[cb + c];
+            long long m = 0;
+            for (int q = se.x; q < se.y; ++q) {
+                const long long hb = __double_as_longlong(posh[q].w);
+                m = (hb > m && hb <= kHMaxBits) ? hb : m;  // (h outside the geometry range: not counted)
+            }
+            cell_hmax[cb + c] = (unsigned long long)m;
+            most = m > most ? m : most;
+        }
+        if (most > 0) atomicMax(&gw_[k].hmax_bits, (unsigned long long)most);
+    }
+    grid.sync();
+    csr_rows<false>(n, B, posh, fpos, tin, cells, cell_hmax, rowlen, ngather, offsets, idx,
+                    s_delta[warp]);
+    grid.sync();
+    // exclusive scan of the row lengths: a contiguous range of rows per block
+    const int64_t per = (n + gridDim.x - 1) / gridDim.x;
+    const int64_t r0 = min(per * blockIdx.x, n), r1 = min(r0 + per, n);
+    auto block_sum = [&](int64_t v) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
+        __syncthreads();
+        if (lane == 0) s_sum[warp] = v;
+        __syncthreads();
+        int64_t a = 0;
+        for (int w = 0; w < kThreads / 32; ++w) a += s_sum[w];
+        return a;
+    };
+    int64_t mine = 0;
+    for (int64_t i = r0 + threadIdx.x; i < r1; i += blockDim.x) mine += rowlen[i];
+    mine = block_sum(mine);
+    if (threadIdx.x == 0) part[blockIdx.x] = mine;
+    grid.sync();
+    int64_t before = 0;
+    for (int q = threadIdx.x; q < (int)blockIdx.x; q += blockDim.x) before += part[q];
+    before = block_sum(before);
+    for (int64_t i0 = r0; i0 < r1; i0 += blockDim.x) {
+        const int64_t i = i0 + threadIdx.x;
+        const int64_t len = i < r1 ? rowlen[i] : 0;
+        int64_t inc = len;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int64_t v = __shfl_up_sync(kFull, inc, o);
+            if (lane >= o) inc += v;
+        }
+        __syncthreads();
+        if (lane == 31) s_sum[warp] = inc;
+        __syncthreads();
+        int64_t off = before;
+        for (int w = 0; w < warp; ++w) off += s_sum[w];
+        if (i < r1) {
+            offsets[i] = off + inc - len;
+            if (i == n - 1) offsets[n] = off + inc;
+        }
+        for (int w = warp; w < kThreads / 32; ++w) off += s_sum[w];
+        before = off;
+    }
+    grid.sync();
+    if (*(volatile int64_t*)&offsets[n] > nnzcap) {
+        if (t0 == 0) atomicOr(&status[0], (unsigned)ST_CAPACITY);
+        return;
+    }
+    csr_rows<true>(n, B, posh, fpos, tin, cells, cell_hmax, rowlen, ngather, offsets, idx,
+                   s_delta[warp]);
+}
+
+// Blocks of k_csr_fallback resident at once on this device (0: none).
+int csr_fallback_blocks(int nsm) {
+    int per = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_csr_fallback, kThreads, 0) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    return std::min(per, 4) * nsm;
+}
+
 void launch_h_search(sph_ctx* c, cudaStream_t s) {
     const int64_t n = c->n;
     if (n == 0) return;
     const unsigned nb = (unsigned)((n + kThreads - 1) / kThreads);
     double4_32a* posh = c->posh[c->cur];
     const Batch B = batch_of(c);
-    c->launches += 4;  // the first count, k_h_iterate, k_finalize_h, k_cell_hmax
+    c->launches += 2;  // the first count, k_h_iterate
     if (c->any_lists) {
         c->launches += 1;
         k_h_lists<<<nb, kThreads, 0, s>>>(n, B, posh, c->fpos, c->nnb, c->ngather, c->rslab,
                                           c->hs_lo, c->hs_hi, c->hs_it, c->wl, c->status,
-                                          c->order[c->cur], c->lst, c->lmeta);
+                                          c->order[c->cur], c->lst, c->lmeta, c->xpk);
     }
     const int64_t nbu = std::min<int64_t>((int64_t)c->nsm * kUnionBlocksPerSM, ((n + 31) / 32 + 7) / 8);
     if (c->any_lists) {
         k_h_union<true><<<(unsigned)nbu, kThreads, 0, s>>>(
             n, B, posh, c->fpos, c->cells, c->nnb, c->ngather, c->rslab, c->hs_lo, c->hs_hi,
-            c->hs_it, c->wl, c->status, c->wctr, c->recs, c->order[c->cur], c->lst, c->lmeta, c->gwl);
+            c->hs_it, c->wl, c->status, c->wctr, c->recs, c->order[c->cur], c->lst, c->lmeta, c->gwl, c->xpk);
         k_h_iterate<true><<<kReduceBlocks * 4, kThreads, 0, s>>>(
             B, posh, c->fpos, c->cells, c->nnb, c->ngather, c->rslab, c->hs_lo, c->hs_hi,
-            c->hs_it, c->wl, c->status, c->order[c->cur], c->lst, c->lmeta);
+            c->hs_it, c->wl, c->status, c->order[c->cur], c->lst, c->lmeta, c->xpk);
     } else {
         const int64_t groups = (n + 31) / 32;
         auto count = [&](auto fn, int warps) {
             fn<<<(unsigned)groups, 32 * warps, 0, s>>>(n, B, posh, c->fpos, c->cells, c->nnb,
                                                        c->ngather, c->rslab, c->hs_lo, c->hs_hi,
-                                                       c->hs_it, c->wl, c->gwl, c->status, c->wctr);
+                                                       c->hs_it, c->wl, c->gwl, c->status, c->wctr,
+                                                       c->xpk);
         };
         // Warps per group: as many as fill the chip once. Measured (first count,
         // us, with 8 / 4 / 2 / 1 warps): 4,096 particles 24 / 31 / 48 / 86, the
@@ -1823,34 +1905,27 @@ void launch_h_search(sph_ctx* c, cudaStream_t s) {
             k_h_union<false><<<(unsigned)nbu, kThreads, 0, s>>>(
                 n, B, posh, c->fpos, c->cells, c->nnb, c->ngather, c->rslab, c->hs_lo, c->hs_hi,
                 c->hs_it, c->wl, c->status, c->wctr, c->recs, c->order[c->cur], c->lst, c->lmeta,
-                c->gwl);
+                c->gwl, c->xpk);
         }
         k_h_iterate<false><<<kReduceBlocks * 4, kThreads, 0, s>>>(
             B, posh, c->fpos, c->cells, c->nnb, c->ngather, c->rslab, c->hs_lo, c->hs_hi,
-            c->hs_it, c->wl, c->status, c->order[c->cur], c->lst, c->lmeta);
+            c->hs_it, c->wl, c->status, c->order[c->cur], c->lst, c->lmeta, c->xpk);
     }
-    k_finalize_h<<<nb, kThreads, 0, s>>>(n, B, posh, c->fpos, c->tin, c->ocnt, c->xpk);
-    const unsigned gx = (unsigned)std::max(2, kReduceBlocks / c->ninst);
-    k_cell_hmax<<<dim3(gx, (unsigned)c->ninst), kThreads, 0, s>>>(B, c->grid, c->cells, posh,
-                                                                  c->cell_hmax);
 }
 
 // The two-pass CSR build, for the rows flagged in status[2] & mask (launched
-// every step; without the flag its kernels return at once).
+// every step; without the flag it returns at once).
 static void csr_fallback(sph_ctx* c, cudaStream_t s, unsigned mask) {
-    const int64_t n = c->n;
-    double4_32a* posh = c->posh[c->cur];
-    const Batch B = batch_of(c);
-    c->launches += 5;  // two build passes and the three kernels of the scan
-    k_csr<false><<<kReduceBlocks * 4, kThreads, 0, s>>>(n, B, posh, c->fpos, c->tin, c->cells,
-                                                        c->cell_hmax, c->rowlen, c->ngather,
-                                                        nullptr, nullptr, c->nnzcap, c->status,
-                                                        mask);
-    launch_scan_i32_i64(c->rowlen, n, c->offsets, c->row_part, s, c->status + 2, mask);
-    k_csr<true><<<kReduceBlocks * 4, kThreads, 0, s>>>(n, B, posh, c->fpos, c->tin, c->cells,
-                                                       c->cell_hmax, c->rowlen, c->ngather,
-                                                       c->offsets, c->idx, c->nnzcap, c->status,
-                                                       mask);
+    int64_t n = c->n, cap = c->nnzcap;
+    int ninst = c->ninst;
+    const double4_32a* posh = c->posh[c->cur];
+    Batch B = batch_of(c);
+    c->launches += 1;
+    void* args[] = {&n, &ninst, &B, &c->grid, &posh, &c->fpos, &c->tin, &c->cells, &c->cell_hmax,
+                    &c->rowlen, &c->ngather, &c->offsets, &c->row_part, &c->idx, &cap, &c->status,
+                    &mask};
+    cudaLaunchCooperativeKernel((const void*)k_csr_fallback, dim3((unsigned)c->csr_blocks),
+                                dim3(kThreads), args, 0, s);
 }
 
 static void rowlen_sort(sph_ctx* c, cudaStream_t s, unsigned mask) {
@@ -1878,7 +1953,9 @@ void launch_csr(sph_ctx* c, cudaStream_t s, bool outer_later) {
     double4_32a* posh = c->posh[c->cur];
     const Batch B = batch_of(c);
     if (!outer_later) {
-        c->launches += 2;
+        c->launches += 3;
+        k_thresholds<<<(unsigned)((n + kThreads - 1) / kThreads), kThreads, 0, s>>>(
+            n, B, posh, c->fpos, c->tin);
         k_outer<<<nbw, kThreads, 0, s>>>(n, B, posh, c->fpos, c->tin, c->ngather, c->rslab,
                                          c->ocnt, c->status);
         rowlen_sort(c, s, (unsigned)IF_SLAB_OVF);

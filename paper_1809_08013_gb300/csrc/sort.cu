@@ -29,7 +29,8 @@ k_load_state(int64_t n, Batch B, const int64_t* __restrict__ coff, const double*
              const double* __restrict__ m, const double* __restrict__ u,
              double4_32a* __restrict__ posh, double4_32a* __restrict__ velm,
              double* __restrict__ ue, int32_t* __restrict__ order, double4_32a* __restrict__ posh2,
-             double4_32a* __restrict__ velm2, double* __restrict__ ue2, int32_t* __restrict__ order2) {
+             double4_32a* __restrict__ velm2, double* __restrict__ ue2, int32_t* __restrict__ order2,
+             int32_t* __restrict__ ocnt) {
     const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= n) return;
     const int inst = slot_inst(B, k);
@@ -39,6 +40,7 @@ k_load_state(int64_t n, Batch B, const int64_t* __restrict__ coff, const double*
         velm[k] = velm2[k] = make_double4_32a(0.0, 0.0, 0.0, 0.0);
         ue[k] = ue2[k] = 0.0;
         order[k] = order2[k] = -1;
+        ocnt[k] = 0;
         return;
     }
     const int64_t c = __ldg(&coff[inst]) + r;
@@ -56,7 +58,7 @@ void launch_load_state(sph_ctx* c, const sph_particles* P, cudaStream_t s) {
     k_load_state<<<(unsigned)((n + kThreads - 1) / kThreads), kThreads, 0, s>>>(
         n, batch_of(c), c->coff, P->x, P->y, P->z, P->h, P->vx, P->vy, P->vz, P->m, P->u,
         c->posh[b], c->velm[b], c->ue[b], c->order[b], c->posh[1 - b], c->velm[1 - b],
-        c->ue[1 - b], c->order[1 - b]);
+        c->ue[1 - b], c->order[1 - b], c->ocnt);
 }
 
 // Pack of the double-float pair kernels for particle k: the fixed-point chunks
@@ -721,7 +723,8 @@ k_permute(int64_t ntot, Batch B, const int64_t* __restrict__ roff,
           const int32_t* __restrict__ order_in, double4_32a* __restrict__ posh_out,
           double4_32a* __restrict__ velm_out, double* __restrict__ u_out,
           int32_t* __restrict__ order_out, float4* __restrict__ fpos, float4* __restrict__ xpk,
-          float4* __restrict__ vpa, float2* __restrict__ vpb, int2* __restrict__ cells) {
+          float4* __restrict__ vpa, float2* __restrict__ vpb, int2* __restrict__ cells,
+          int32_t* __restrict__ ocnt) {
     const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= ntot) return;
     const int64_t o = perm[r];
@@ -748,6 +751,7 @@ k_permute(int64_t ntot, Batch B, const int64_t* __restrict__ roff,
     u_out[k] = u_in[o];
     order_out[k] = order_in[o];
     fpos[k] = make_float4((float)p.x, (float)p.y, (float)p.z, 0.0f);
+    ocnt[k] = 0;  // outer entries of the row, to be appended
 }
 
 // Tiles of the sort for nt keys. Up to kRadixSmallN a chained sort with tiles
@@ -834,7 +838,7 @@ void launch_build_cells(sph_ctx* c, cudaStream_t s) {
     k_permute<<<nbt, kThreads, 0, s>>>(nt, B, c->roff, c->keys[src], c->vals[src], c->posh[a],
                                         c->velm[a], c->ue[a], c->order[a], c->posh[b], c->velm[b],
                                         c->ue[b], c->order[b], c->fpos, c->xpk, c->vpa, c->vpb,
-                                        c->cells);
+                                        c->cells, c->ocnt);
     c->cur = b;
 }
 

@@ -218,7 +218,7 @@ bool allocate_all(sph_ctx* c, int64_t nslots, Allocator& al) {
          al(&c->hist, 4 * (size_t)radix_counts((int64_t)N)) &&
          al(&c->cells, (size_t)c->cellcap) && al(&c->cell_hmax, (size_t)c->cellcap) &&
          al(&c->nnb, N) && al(&c->ngather, N) && al(&c->rowlen, N) &&
-         al(&c->offsets, N + 1) && al(&c->row_part, (size_t)scan_parts(N) + 1) &&
+         al(&c->offsets, N + 1) && al(&c->row_part, std::max<size_t>((size_t)scan_parts(N) + 1, 4 * (size_t)c->nsm)) &&
          al(&c->idx, (size_t)nnzcap) && al(&c->red_part, (N + kSlotAlign - 1) / kSlotAlign * kBoxStride) &&
          al(&c->dt_part, nfb * kMaxPairThreads * (kThreads / kPairBlockMin)) && al(&c->grid, (size_t)max_instances) &&
          al(&c->status, 4) && al(&c->blk, nfb) &&
@@ -685,8 +685,9 @@ sph_status sph_ctx_create_batch(sph_ctx** out, int64_t ncap, int64_t nnzcap, int
         cudaGetLastError();
         c->nsm = 1;
     }
+    c->csr_blocks = csr_fallback_blocks(c->nsm);
     Allocator A{false, 0};
-    bool ok = allocate_all(c, nslots, A);
+    bool ok = c->csr_blocks > 0 && allocate_all(c, nslots, A);
     ok = ok && cudaMallocHost((void**)&c->status_host, 2 * sizeof(unsigned)) == cudaSuccess;
     ok = ok && cudaMemset(c->status, 0, 4 * sizeof(unsigned)) == cudaSuccess &&
          cudaMemset(c->offsets, 0, sizeof(int64_t)) == cudaSuccess &&

@@ -351,6 +351,7 @@ struct sph_ctx {
     bool group_search;      // some instance has kGroupSearchN particles or more
     int lay_n;              // instances of the last batch layout (first, count) ...
     int64_t lay_first[sph::kMaxInstances], lay_cnt[sph::kMaxInstances];  // ... and theirs
+    int csr_blocks;         // blocks of the cooperative CSR fallback
     int nsm;                // streaming multiprocessors of the device
     unsigned* status;       // [0] bits, [1] non-converged count, [2] internal flags,
                             // [3] h-search worklist length
@@ -511,6 +512,7 @@ void launch_h_search(sph_ctx* c, cudaStream_t s);
 // launch_rows_finish completes the rows after it
 void launch_csr(sph_ctx* c, cudaStream_t s, bool outer_later = false);
 void launch_rows_finish(sph_ctx* c, cudaStream_t s);
+int csr_fallback_blocks(int nsm);
 // the rows as a CSR in offsets / idx (a copy in slab form; nothing after a fallback)
 void launch_compose(sph_ctx* c, cudaStream_t s);
 
@@ -538,10 +540,9 @@ enum : unsigned {
 };
 
 // ---- scan.cu
-// exclusive scan of n int32 into n+1 int64 (out[n] = total); with gate, only
-// when *gate & mask is set on the device when the kernels run
+// exclusive scan of n int32 into n+1 int64 (out[n] = total)
 void launch_scan_i32_i64(const int32_t* in, int64_t n, int64_t* out, int64_t* part,
-                         cudaStream_t s, const unsigned* gate = nullptr, unsigned mask = 0u);
+                         cudaStream_t s);
 int64_t scan_parts(int64_t n);
 
 }  // namespace sph
