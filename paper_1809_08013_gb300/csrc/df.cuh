@@ -46,6 +46,16 @@ __device__ __forceinline__ df add(df x, df y) {
 
 __device__ __forceinline__ df sub(df x, df y) { return add(x, neg(y)); }
 
+// x + y + z with one renormalisation (19 operations; two sums take 22): the high
+// parts by two TwoSums, all low parts folded in once, within ~2^-47 (|x| + |y| +
+// |z|) like two sums.
+__device__ __forceinline__ df add3(df x, df y, df z) {
+    const df a = two_sum(x.hi, y.hi);
+    const df b = two_sum(a.hi, z.hi);
+    const float e = __fadd_rn(__fadd_rn(a.lo, b.lo), __fadd_rn(__fadd_rn(x.lo, y.lo), z.lo));
+    return fast_two_sum(b.hi, e);
+}
+
 // x + y for operands of the same sign (no cancellation), left unnormalised:
 // the low part may reach ~1.5 ulp of the high one. Only for a sum whose
 // consumer is a normalising add: a product of an unnormalised value rounds

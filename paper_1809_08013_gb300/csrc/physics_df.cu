@@ -331,7 +331,7 @@ void launch_density_df(sph_ctx* c, bool fuse_eos, cudaStream_t s, bool outer) {
 // ------------------------------------------------------------ forces + dt
 // Definitions as in physics.cu; algebra: Fbar = (0.5/pi)(f(q_i)/h_i^4 +
 // f(q_j)/h_j^4)/r, one shared reciprocal R = 1/((r^2 + eta2 hb^2) rhob) for the
-// viscosity, mu = hb v.r rhob R, 1/rhob = (r^2 + eta2 hb^2) R. Every sum is
+// viscosity: with a = hb v.r R, mu = a rhob and Pi = a (beta mu - alpha cb). Every sum is
 // linear in Fbar, so its constant factor (0.5/pi, or dnorm/2) is applied once
 // per particle, in FP64, when the sums are written out.
 // U: neighbours evaluated at a time, their terms added in the order of the row
@@ -344,6 +344,9 @@ void launch_density_df(sph_ctx* c, bool fuse_eos, cudaStream_t s, bool outer) {
 // 70 (108), 104k 216 (247), 1M 1,795 (1,893); the Wendland kernel at 216,000
 // 427 (457). U = 3: 1,860 at 1M; 5 or 6: 2,330. The sinc shapes, with a loop
 // over terms, are faster one at a time (1,076 against 1,410 at 216,000).
+// Three-term sums (add3), Pi = a t (one product less) and the next neighbours'
+// indices loaded while these are evaluated: then 4,096 particles 41 us, 104k 205,
+// 1M 1,704 (2,062 with the sums alone: the index loads are what hides the gathers).
 template <int T, int KER, int U>
 __global__ void __launch_bounds__(kPairBlock<U>, U > 1 ? 1 : (KER == KER_SINC ? 2 : 3))
 k_forces_df(int64_t n, Batch B, const double4_32a* __restrict__ posh,
@@ -400,21 +403,22 @@ k_forces_df(int64_t n, Batch B, const double4_32a* __restrict__ posh,
                 const df Fb = dfl::mul(dfl::add(dfl::mul(Ki, fa), dfl::mul(df{b0.z, b0.w}, fb)), rinv);
                 const df WX = dfl::sub(VXi, df{wa.x, wa.y}), WY = dfl::sub(VYi, df{wa.z, wa.w});
                 const df WZ = dfl::sub(VZi, df{wb.x, wb.y});
-                const df vr = dfl::add(dfl::add(dfl::mul(WX, X), dfl::mul(WY, Y)), dfl::mul(WZ, Z));
+                const df vr = dfl::add3(dfl::mul(WX, X), dfl::mul(WY, Y), dfl::mul(WZ, Z));
                 df Pi = {0.f, 0.f};
                 if (vr.hi < 0.0f) {
                     const df hb = dfl::add(hhi, df{b1.z, b1.w});
                     const df d1 = dfl::add(r2, dfl::mul(dfl::mul(eta2, hb), hb));
                     const df rb = dfl::add(rhi, df{b2.x, b2.y});
                     const df R = dfl::rcp(dfl::mul(d1, rb));
-                    const df mu = dfl::mul(dfl::mul(dfl::mul(hb, vr), rb), R);
+                    const df av = dfl::mul(dfl::mul(hb, vr), R);  // mu / rho_b
+                    const df mu = dfl::mul(av, rb);
                     const df cb = dfl::add(cai, df{b2.z, b2.w});
                     const df t = dfl::add(dfl::mul(betad, mu), dfl::neg(cb));
-                    Pi = dfl::mul(dfl::mul(mu, t), dfl::mul(d1, R));
+                    Pi = dfl::mul(av, t);
                     if (-mu.hi > mumx.hi) mumx = dfl::neg(mu);
                 }
                 const df mF = dfl::mul(df{J0.w, J1.w}, Fb);
-                const df g = dfl::mul(mF, dfl::add(dfl::add(Ai, df{b1.x, b1.y}), Pi));
+                const df g = dfl::mul(mF, dfl::add3(Ai, df{b1.x, b1.y}, Pi));
                 sx = dfl::add(sx, dfl::mul(g, X));
                 sy = dfl::add(sy, dfl::mul(g, Y));
                 sz = dfl::add(sz, dfl::mul(g, Z));
@@ -423,13 +427,19 @@ k_forces_df(int64_t n, Batch B, const double4_32a* __restrict__ posh,
                 sv = dfl::add(sv, dfl::mul(mFv, Pi));
             }
         } else {
+            int jn[U];  // the next neighbours' indices
+#pragma unroll
+            for (int u = 0; u < U; ++u) jn[u] = sub + u * T < len ? __ldg(&ent[sub + u * T]) : (int)i;
             for (int e0 = sub; e0 < len; e0 += T * U) {
                 int j[U];
                 df tx[U], ty[U], tz[U], tp[U], tv[U], nmu[U];
                 bool use[U];
 #pragma unroll
-                for (int u = 0; u < U; ++u)
-                    j[u] = e0 + u * T < len ? __ldg(&ent[e0 + u * T]) : (int)i;
+                for (int u = 0; u < U; ++u) {
+                    const int e = e0 + (U + u) * T;
+                    j[u] = jn[u];
+                    jn[u] = e < len ? __ldg(&ent[e]) : (int)i;
+                }
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
                     const float4 J0 = __ldg(&xpk[3 * j[u]]), J1 = __ldg(&xpk[3 * j[u] + 1]);
@@ -452,20 +462,21 @@ k_forces_df(int64_t n, Batch B, const double4_32a* __restrict__ posh,
                     const df Fb = dfl::mul(dfl::add(dfl::mul(Ki, fa), dfl::mul(df{b0.z, b0.w}, fb)), rinv);
                     const df WX = dfl::sub(VXi, df{wa.x, wa.y}), WY = dfl::sub(VYi, df{wa.z, wa.w});
                     const df WZ = dfl::sub(VZi, df{wb.x, wb.y});
-                    const df vr = dfl::add(dfl::add(dfl::mul(WX, X), dfl::mul(WY, Y)), dfl::mul(WZ, Z));
+                    const df vr = dfl::add3(dfl::mul(WX, X), dfl::mul(WY, Y), dfl::mul(WZ, Z));
                     const df hb = dfl::add(hhi, df{b1.z, b1.w});
                     const df d1 = dfl::add(r2, dfl::mul(dfl::mul(eta2, hb), hb));
                     const df rb = dfl::add(rhi, df{b2.x, b2.y});
                     const df R = dfl::rcp(dfl::mul(d1, rb));
-                    const df mu = dfl::mul(dfl::mul(dfl::mul(hb, vr), rb), R);
+                    const df av = dfl::mul(dfl::mul(hb, vr), R);  // mu / rho_b
+                    const df mu = dfl::mul(av, rb);
                     const df cb = dfl::add(cai, df{b2.z, b2.w});
                     const df t = dfl::add(dfl::mul(betad, mu), dfl::neg(cb));
-                    const df Pv = dfl::mul(dfl::mul(mu, t), dfl::mul(d1, R));
+                    const df Pv = dfl::mul(av, t);
                     const bool visc = vr.hi < 0.0f;
                     const df Pi = {visc ? Pv.hi : 0.f, visc ? Pv.lo : 0.f};
                     nmu[u] = df{ok && visc ? -mu.hi : 0.f, ok && visc ? -mu.lo : 0.f};
                     const df mF = dfl::mul(df{J0.w, J1.w}, Fb);
-                    const df g = dfl::mul(mF, dfl::add(dfl::add(Ai, df{b1.x, b1.y}), Pi));
+                    const df g = dfl::mul(mF, dfl::add3(Ai, df{b1.x, b1.y}, Pi));
                     tx[u] = dfl::mul(g, X);
                     ty[u] = dfl::mul(g, Y);
                     tz[u] = dfl::mul(g, Z);
@@ -659,15 +670,16 @@ k_iad_df(int64_t n, Batch B, const double4_32a* __restrict__ posh,
 // symmetric 3x3 (in the cpk order) times a vector, in double-float
 __device__ __forceinline__ void symv_df(const df* M, const df& x, const df& y, const df& z, df& ox,
                                         df& oy, df& oz) {
-    ox = dfl::add(dfl::add(dfl::mul(M[0], x), dfl::mul(M[1], y)), dfl::mul(M[2], z));
-    oy = dfl::add(dfl::add(dfl::mul(M[1], x), dfl::mul(M[3], y)), dfl::mul(M[4], z));
-    oz = dfl::add(dfl::add(dfl::mul(M[2], x), dfl::mul(M[4], y)), dfl::mul(M[5], z));
+    ox = dfl::add3(dfl::mul(M[0], x), dfl::mul(M[1], y), dfl::mul(M[2], z));
+    oy = dfl::add3(dfl::mul(M[1], x), dfl::mul(M[3], y), dfl::mul(M[4], z));
+    oz = dfl::add3(dfl::mul(M[2], x), dfl::mul(M[4], y), dfl::mul(M[5], z));
 }
 
 // Forces with IAD gradients: as k_forces_df with F r_ij replaced by
 // G_ij = -(wnorm / 2) (h_i^-3 g(q_i) C_i + h_j^-3 g(q_j) C_j) r_ij.
 // U: as in k_forces_df (125,000 particles, Wendland: 396 us at U = 1, 371 at 2,
-// 415 at 3; sinc at 216,000: 1,022 at 1, 1,195 at 2).
+// 415 at 3; 351 at 2 since the sums and index loads of k_forces_df are used here
+// too; sinc at 216,000: 1,022 at 1, 1,195 at 2).
 template <int T, int KER, int U>
 __global__ void __launch_bounds__(kPairBlock<U>, U > 1 ? 1 : 2)
 k_forces_iad_df(int64_t n, Batch B, const double4_32a* __restrict__ posh,
@@ -741,37 +753,44 @@ k_forces_iad_df(int64_t n, Batch B, const double4_32a* __restrict__ posh,
                 Gz = dfl::mul(kg, Gz);
                 const df WX = dfl::sub(VXi, df{wa.x, wa.y}), WY = dfl::sub(VYi, df{wa.z, wa.w});
                 const df WZ = dfl::sub(VZi, df{wb.x, wb.y});
-                const df vr = dfl::add(dfl::add(dfl::mul(WX, X), dfl::mul(WY, Y)), dfl::mul(WZ, Z));
+                const df vr = dfl::add3(dfl::mul(WX, X), dfl::mul(WY, Y), dfl::mul(WZ, Z));
                 df Pi = {0.f, 0.f};
                 if (vr.hi < 0.0f) {
                     const df hb = dfl::add(hhi, df{b1.z, b1.w});
                     const df d1 = dfl::add(r2, dfl::mul(dfl::mul(eta2, hb), hb));
                     const df rb = dfl::add(rhi, df{b2.x, b2.y});
                     const df Rr = dfl::rcp(dfl::mul(d1, rb));
-                    const df mu = dfl::mul(dfl::mul(dfl::mul(hb, vr), rb), Rr);
+                    const df av = dfl::mul(dfl::mul(hb, vr), Rr);  // mu / rho_b
+                    const df mu = dfl::mul(av, rb);
                     const df cb = dfl::add(cai, df{b2.z, b2.w});
                     const df tt = dfl::add(dfl::mul(betad, mu), dfl::neg(cb));
-                    Pi = dfl::mul(dfl::mul(mu, tt), dfl::mul(d1, Rr));
+                    Pi = dfl::mul(av, tt);
                     if (-mu.hi > mumx.hi) mumx = dfl::neg(mu);
                 }
                 const df mj = {J0.w, J1.w};
-                const df g = dfl::mul(mj, dfl::add(dfl::add(Ai, df{b1.x, b1.y}), Pi));
+                const df g = dfl::mul(mj, dfl::add3(Ai, df{b1.x, b1.y}, Pi));
                 sx = dfl::add(sx, dfl::mul(g, Gx));
                 sy = dfl::add(sy, dfl::mul(g, Gy));
                 sz = dfl::add(sz, dfl::mul(g, Gz));
-                const df Gv = dfl::add(dfl::add(dfl::mul(Gx, WX), dfl::mul(Gy, WY)), dfl::mul(Gz, WZ));
+                const df Gv = dfl::add3(dfl::mul(Gx, WX), dfl::mul(Gy, WY), dfl::mul(Gz, WZ));
                 const df mGv = dfl::mul(mj, Gv);
                 sp = dfl::add(sp, mGv);
                 sv = dfl::add(sv, dfl::mul(mGv, Pi));
             }
         } else {
+            int jn[U];  // the next neighbours' indices
+#pragma unroll
+            for (int u = 0; u < U; ++u) jn[u] = sub + u * T < len ? __ldg(&ent[sub + u * T]) : (int)i;
             for (int e0 = sub; e0 < len; e0 += T * U) {
                 int j[U];
                 df tx[U], ty[U], tz[U], tp[U], tv[U], nmu[U];
                 bool use[U];
 #pragma unroll
-                for (int u = 0; u < U; ++u)
-                    j[u] = e0 + u * T < len ? __ldg(&ent[e0 + u * T]) : (int)i;
+                for (int u = 0; u < U; ++u) {
+                    const int e = e0 + (U + u) * T;
+                    j[u] = jn[u];
+                    jn[u] = e < len ? __ldg(&ent[e]) : (int)i;
+                }
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
                     const float4 J0 = __ldg(&xpk[3 * j[u]]), J1 = __ldg(&xpk[3 * j[u] + 1]);
@@ -807,24 +826,25 @@ k_forces_iad_df(int64_t n, Batch B, const double4_32a* __restrict__ posh,
                     Gz = dfl::mul(kg, Gz);
                     const df WX = dfl::sub(VXi, df{wa.x, wa.y}), WY = dfl::sub(VYi, df{wa.z, wa.w});
                     const df WZ = dfl::sub(VZi, df{wb.x, wb.y});
-                    const df vr = dfl::add(dfl::add(dfl::mul(WX, X), dfl::mul(WY, Y)), dfl::mul(WZ, Z));
+                    const df vr = dfl::add3(dfl::mul(WX, X), dfl::mul(WY, Y), dfl::mul(WZ, Z));
                     const df hb = dfl::add(hhi, df{b1.z, b1.w});
                     const df d1 = dfl::add(r2, dfl::mul(dfl::mul(eta2, hb), hb));
                     const df rb = dfl::add(rhi, df{b2.x, b2.y});
                     const df Rr = dfl::rcp(dfl::mul(d1, rb));
-                    const df mu = dfl::mul(dfl::mul(dfl::mul(hb, vr), rb), Rr);
+                    const df av = dfl::mul(dfl::mul(hb, vr), Rr);  // mu / rho_b
+                    const df mu = dfl::mul(av, rb);
                     const df cb = dfl::add(cai, df{b2.z, b2.w});
                     const df tt = dfl::add(dfl::mul(betad, mu), dfl::neg(cb));
-                    const df Pv = dfl::mul(dfl::mul(mu, tt), dfl::mul(d1, Rr));
+                    const df Pv = dfl::mul(av, tt);
                     const bool visc = vr.hi < 0.0f;
                     const df Pi = {visc ? Pv.hi : 0.f, visc ? Pv.lo : 0.f};
                     nmu[u] = df{ok && visc ? -mu.hi : 0.f, ok && visc ? -mu.lo : 0.f};
                     const df mj = {J0.w, J1.w};
-                    const df g = dfl::mul(mj, dfl::add(dfl::add(Ai, df{b1.x, b1.y}), Pi));
+                    const df g = dfl::mul(mj, dfl::add3(Ai, df{b1.x, b1.y}, Pi));
                     tx[u] = dfl::mul(g, Gx);
                     ty[u] = dfl::mul(g, Gy);
                     tz[u] = dfl::mul(g, Gz);
-                    const df Gv = dfl::add(dfl::add(dfl::mul(Gx, WX), dfl::mul(Gy, WY)), dfl::mul(Gz, WZ));
+                    const df Gv = dfl::add3(dfl::mul(Gx, WX), dfl::mul(Gy, WY), dfl::mul(Gz, WZ));
                     tp[u] = dfl::mul(mj, Gv);
                     tv[u] = dfl::mul(tp[u], Pi);
                     use[u] = ok;
