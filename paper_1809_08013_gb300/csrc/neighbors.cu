@@ -19,10 +19,13 @@
 // Symmetric set S_i = { j != i : r_ij < 2h_i or r_ij < 2h_j } as CSR: row i
 // holds N_i (r_ij < 2h_i) first, then the rest.
 //
-// Work decomposition: one warp per particle. The lanes take 32 candidates of
-// a cell at a time (coalesced loads), counts come from ballots and row
-// entries are compacted with ballot prefix counts, so the particle's own
-// iteration count never stalls other particles.
+// Work decomposition: a first count at the h a particle comes with, 32
+// consecutive particles at a time, one lane each (k_h_count; ~98% of them need
+// no more in a running simulation); those that go on, one warp per particle
+// (k_h_iterate), which takes 32 candidates at a time with ballots and ballot
+// prefix counts, so that a particle's own iteration count never stalls the
+// others. A large instance of which much goes on (a first step) first takes
+// further counts 32 particles at a time (k_h_union).
 #include <math_constants.h>
 
 #include <cooperative_groups.h>
@@ -420,12 +423,15 @@ __device__ __forceinline__ void write_reach2(float4* __restrict__ xpk, int64_t i
 }
 
 // ------------------------------------------------------------ h search
-// Phase 1: one warp per 32 consecutive (Morton-sorted) particles, one lane
-// per particle. Each pass counts N_i(h) for every still-searching lane over
-// the union of their query boxes (candidates staged once for the warp) and
-// records the gather set in the slab. While more than defer_lanes lanes are
-// still searching the warp keeps going; the stragglers are then handed, with
-// their bisection state, to the per-particle kernel below through a worklist.
+// Groups (union_group, k_h_union): one warp per 32 consecutive (Morton-sorted)
+// particles, one lane per particle, for the groups left with more than
+// defer_lanes searching lanes by the first count (k_h_count; with candidate
+// lists the search starts here). Each pass counts N_i(h) for every
+// still-searching lane over the union of their query boxes (candidates staged
+// once for the warp) and records the gather set in the slab. While more than
+// defer_lanes lanes are still searching the warp keeps going; the stragglers
+// are then handed, with their bisection state, to the per-particle kernel
+// below through a worklist.
 
 // Cell index of a (float) coordinate along axis d, clamped to the grid; only
 // used to cluster the lanes of a warp, so FP32 rounding is harmless.

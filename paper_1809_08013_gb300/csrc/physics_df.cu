@@ -192,7 +192,14 @@ __device__ __forceinline__ void eos_d(const KParams& kp, double rho, double u, d
 // The next neighbour's loads go out before one is evaluated, in blocks of 64
 // threads: 1M patch 681 us (732 without, in blocks of 256; the branch-free shape
 // gave 38 us of that).
-template <bool FUSE, int T, int KER, bool OUTER>
+// U: neighbours evaluated at a time, their terms added in the order of the row
+// (the same bits for every U). A lane's append waits for the slot its last one
+// got, and in a warp some lane has one at almost every neighbour: while there
+// are too few warps to hide that (up to kPairUnrollN particles) four at a time,
+// each with an append of its own in flight: 4,096 particles 44 us (54), 27,000 43
+// (57). Beyond, one at a time: 104k 107 us (116), 1M 681 (807); two appends in
+// flight without the unrolling 721 at 1M.
+template <bool FUSE, int T, int KER, bool OUTER, int U>
 __global__ void __launch_bounds__(kPairBlockMin)
 k_density_df(int64_t n, Batch B, const double4_32a* __restrict__ posh,
              const float4* __restrict__ xpk, const double* __restrict__ ue,
@@ -221,55 +228,122 @@ k_density_df(int64_t n, Batch B, const double4_32a* __restrict__ posh,
     if (sub == 0) acc = df{I0.w, I1.w};  // self term m_i W(0, h_i): shape 1
     // rows read from the CSR (a gather set overflowed) are complete already
     const bool append = OUTER && !(R.status[2] & IF_SLAB_OVF);
-    Append ap;
-    int jn = (int)i;
-    float4 N0 = I0, N1 = I1, N2 = I2;
-    auto fetch = [&](int e) {
-        if (e < len) {
-            jn = __ldg(&ent[e]);
-            N0 = __ldg(&xpk[3 * jn]);
-            N1 = __ldg(&xpk[3 * jn + 1]);
-            N2 = __ldg(&xpk[3 * jn + 2]);
-        }
-    };
-    fetch(sub);
-    for (int e = sub; e < len; e += T) {
-        const int j = jn;
-        const float4 J0 = N0, J1 = N1, J2 = N2;
-        fetch(e + T);
-        const df mj = {J0.w, J1.w};
-        float z2 = __fsub_rn(I0.z, J0.z), z1 = __fsub_rn(I1.z, J1.z), z0 = __fsub_rn(I2.z, J2.z);
-        if (per) wrap_fx(z2, z1, z0, hlz, L2, L1, L0);
-        const df X = dfl::fx_sum(__fsub_rn(I0.x, J0.x), __fsub_rn(I1.x, J1.x), __fsub_rn(I2.x, J2.x));
-        const df Y = dfl::fx_sum(__fsub_rn(I0.y, J0.y), __fsub_rn(I1.y, J1.y), __fsub_rn(I2.y, J2.y));
-        const df Z = dfl::fx_sum(z2, z1, z0);
-        const df r2 = dfl::add(dfl::add_same(dfl::sqr(X), dfl::sqr(Y)), dfl::sqr(Z));
-        df w = {1.0f, 0.0f};  // coincident particles: q = 0
-        if (KER == KER_M4) {
-            const df v = w_shape(dfl::mul(dfl::mul(r2, dfl::rsqrt(r2)), Hi));
-            w.hi = r2.hi > 0.0f ? v.hi : w.hi;
-            w.lo = r2.hi > 0.0f ? v.lo : w.lo;
-        } else if (r2.hi > 0.0f) {
-            const df q = dfl::mul(dfl::mul(r2, dfl::rsqrt(r2)), Hi);
-            w = w_shape_k<KER>(q, sn);
-        }
-        acc = dfl::add(acc, dfl::mul(mj, w));
-        if (append) {
-            const float tj = J2.w;  // (2 h_j)^2 in the length unit (NaN: exact test only)
-            bool in_j;
-            if (r2.hi < tj * 0.99999905f) {
-                in_j = true;
-            } else if (r2.hi > tj * 1.00000095f) {
-                in_j = false;
-            } else {
-                const double4_32a pj = posh[j];
-                const double Rj = 2.0 * pj.w;
-                in_j = exact_r2_def(pi, pj, per, kp.lz) < __dmul_rn(Rj, Rj);
+    Append ap[U];
+    if constexpr (U == 1) {
+        int jn = (int)i;
+        float4 N0 = I0, N1 = I1, N2 = I2;
+        auto fetch = [&](int e) {
+            if (e < len) {
+                jn = __ldg(&ent[e]);
+                N0 = __ldg(&xpk[3 * jn]);
+                N1 = __ldg(&xpk[3 * jn + 1]);
+                N2 = __ldg(&xpk[3 * jn + 2]);
             }
-            if (!in_j) ap.add(i, j, R.ngather, O);  // i belongs in the outer part of row j
+        };
+        fetch(sub);
+        for (int e = sub; e < len; e += T) {
+            const int j = jn;
+            const float4 J0 = N0, J1 = N1, J2 = N2;
+            fetch(e + T);
+            const df mj = {J0.w, J1.w};
+            float z2 = __fsub_rn(I0.z, J0.z), z1 = __fsub_rn(I1.z, J1.z), z0 = __fsub_rn(I2.z, J2.z);
+            if (per) wrap_fx(z2, z1, z0, hlz, L2, L1, L0);
+            const df X = dfl::fx_sum(__fsub_rn(I0.x, J0.x), __fsub_rn(I1.x, J1.x), __fsub_rn(I2.x, J2.x));
+            const df Y = dfl::fx_sum(__fsub_rn(I0.y, J0.y), __fsub_rn(I1.y, J1.y), __fsub_rn(I2.y, J2.y));
+            const df Z = dfl::fx_sum(z2, z1, z0);
+            const df r2 = dfl::add(dfl::add_same(dfl::sqr(X), dfl::sqr(Y)), dfl::sqr(Z));
+            df w = {1.0f, 0.0f};  // coincident particles: q = 0
+            if (KER == KER_M4) {
+                const df v = w_shape(dfl::mul(dfl::mul(r2, dfl::rsqrt(r2)), Hi));
+                w.hi = r2.hi > 0.0f ? v.hi : w.hi;
+                w.lo = r2.hi > 0.0f ? v.lo : w.lo;
+            } else if (r2.hi > 0.0f) {
+                const df q = dfl::mul(dfl::mul(r2, dfl::rsqrt(r2)), Hi);
+                w = w_shape_k<KER>(q, sn);
+            }
+            acc = dfl::add(acc, dfl::mul(mj, w));
+            if (append) {
+                const float tj = J2.w;  // (2 h_j)^2 in the length unit (NaN: exact test only)
+                bool in_j;
+                if (r2.hi < tj * 0.99999905f) {
+                    in_j = true;
+                } else if (r2.hi > tj * 1.00000095f) {
+                    in_j = false;
+                } else {
+                    const double4_32a pj = posh[j];
+                    const double Rj = 2.0 * pj.w;
+                    in_j = exact_r2_def(pi, pj, per, kp.lz) < __dmul_rn(Rj, Rj);
+                }
+                if (!in_j) ap[0].add(i, j, R.ngather, O);  // i belongs in the outer part of row j
+            }
+        }
+    } else {
+        int jn[U];  // the next neighbours' indices
+#pragma unroll
+        for (int u = 0; u < U; ++u) jn[u] = sub + u * T < len ? __ldg(&ent[sub + u * T]) : (int)i;
+        for (int e0 = sub; e0 < len; e0 += T * U) {
+            int j[U];
+            df term[U];
+            float rr[U], tj[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int e = e0 + (U + u) * T;
+                j[u] = jn[u];
+                jn[u] = e < len ? __ldg(&ent[e]) : (int)i;
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const float4 J0 = __ldg(&xpk[3 * j[u]]), J1 = __ldg(&xpk[3 * j[u] + 1]);
+                const float4 J2 = __ldg(&xpk[3 * j[u] + 2]);
+                const df mj = {J0.w, J1.w};
+                float z2 = __fsub_rn(I0.z, J0.z), z1 = __fsub_rn(I1.z, J1.z), z0 = __fsub_rn(I2.z, J2.z);
+                if (per) wrap_fx(z2, z1, z0, hlz, L2, L1, L0);
+                const df X = dfl::fx_sum(__fsub_rn(I0.x, J0.x), __fsub_rn(I1.x, J1.x), __fsub_rn(I2.x, J2.x));
+                const df Y = dfl::fx_sum(__fsub_rn(I0.y, J0.y), __fsub_rn(I1.y, J1.y), __fsub_rn(I2.y, J2.y));
+                const df Z = dfl::fx_sum(z2, z1, z0);
+                const df r2 = dfl::add(dfl::add_same(dfl::sqr(X), dfl::sqr(Y)), dfl::sqr(Z));
+                const df q = dfl::mul(dfl::mul(r2, dfl::rsqrt(r2)), Hi);
+                df w = KER == KER_M4 ? w_shape(q) : w_shape_k<KER>(q, sn);
+                w.hi = r2.hi > 0.0f ? w.hi : 1.0f;
+                w.lo = r2.hi > 0.0f ? w.lo : 0.0f;
+                term[u] = dfl::mul(mj, w);
+                rr[u] = r2.hi;
+                tj[u] = J2.w;  // as above
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const df s1 = dfl::add(acc, term[u]);
+                const bool ok = e0 + u * T < len;
+                acc.hi = ok ? s1.hi : acc.hi;
+                acc.lo = ok ? s1.lo : acc.lo;
+            }
+            if (append) {
+                bool out[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    out[u] = false;
+                    if (e0 + u * T >= len || rr[u] < tj[u] * 0.99999905f) continue;
+                    bool in_j = false;
+                    if (!(rr[u] > tj[u] * 1.00000095f)) {
+                        const double4_32a pj = posh[j[u]];
+                        const double Rj = 2.0 * pj.w;
+                        in_j = exact_r2_def(pi, pj, per, kp.lz) < __dmul_rn(Rj, Rj);
+                    }
+                    out[u] = !in_j;
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    if (out[u]) ap[u].flush(i, O);
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    if (out[u]) ap[u].add(i, j[u], R.ngather, O);
+            }
         }
     }
-    if (OUTER) ap.flush(i, O);
+    if (OUTER) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) ap[u].flush(i, O);
+    }
     }
     if (T > 1) {
         acc = dfl::lane_sum<T>(acc);
@@ -305,9 +379,19 @@ static void density_df_t(sph_ctx* c, cudaStream_t s) {
             n, batch_of(c), c->posh[b], c->xpk, c->ue[b], R, c->therm, c->kern, c->dpk, c->pint,
             c->cint, c->status, OuterOut{c->rslab, c->ocnt, c->status});
     };
-    if (c->kern_kind == KER_WENDLAND) go(k_density_df<FUSE, T, KER_WENDLAND, OUTER>);
-    else if (c->kern_kind == KER_SINC) go(k_density_df<FUSE, T, KER_SINC, OUTER>);
-    else go(k_density_df<FUSE, T, KER_M4, OUTER>);
+    if (c->kern_kind == KER_SINC) {
+        go(k_density_df<FUSE, T, KER_SINC, OUTER, 1>);
+        return;
+    }
+    if constexpr (OUTER) {
+        if (n <= kPairUnrollN) {
+            if (c->kern_kind == KER_WENDLAND) go(k_density_df<FUSE, T, KER_WENDLAND, OUTER, 4>);
+            else go(k_density_df<FUSE, T, KER_M4, OUTER, 4>);
+            return;
+        }
+    }
+    if (c->kern_kind == KER_WENDLAND) go(k_density_df<FUSE, T, KER_WENDLAND, OUTER, 1>);
+    else go(k_density_df<FUSE, T, KER_M4, OUTER, 1>);
 }
 
 template <bool FUSE, bool OUTER>

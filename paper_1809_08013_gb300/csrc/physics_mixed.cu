@@ -180,7 +180,9 @@ k_pack_mx(int64_t n, Batch B, const double4_32a* __restrict__ posh,
 // U: neighbours evaluated at a time, their terms added in the order of the row
 // (the same bits for every U). U = 4 in blocks of 64: 1M sphere 677 us (746 one
 // at a time in blocks of 256), 8,191 particles 49 (53).
-template <bool FUSE, int T, bool OUTER, int U>
+// A: appends in flight per lane, 1 or U (as in k_density_df, U while there are
+// few warps: 8,191 particles 42 us; the 1M sphere takes 715 us with U).
+template <bool FUSE, int T, bool OUTER, int U, int A>
 __global__ void __launch_bounds__(kPairBlock<U>)
 k_density_mx(int64_t n, Batch B, const double4_32a* __restrict__ posh,
              const double* __restrict__ ue, float4* __restrict__ mpk,
@@ -203,7 +205,7 @@ k_density_mx(int64_t n, Batch B, const double4_32a* __restrict__ posh,
     if (sub == 0) acc = df{a0.w, 0.0f};  // self term m_i W(0, h_i): shape 1
     // rows read from the CSR (a gather set overflowed) are complete already
     const bool append = OUTER && !(R.status[2] & IF_SLAB_OVF);
-    Append ap;
+    Append ap[A];
     for (int e0 = sub; e0 < len; e0 += T * U) {
         int j[U];
         float term[U], tq[U], hj[U];
@@ -221,28 +223,38 @@ k_density_mx(int64_t n, Batch B, const double4_32a* __restrict__ posh,
             tq[u] = r2 * b1.w * b1.w;  // (r / h_j)^2
             hj[u] = b1.w;
         }
+        // is i in N_j?
+        auto in_row = [&](int u) {
+            const float t = tq[u];
+            const bool wide = zw.per && hj[u] * zw.lzh < 8.0f;
+            if (!wide && t < 4.0f * 0.99999619f) return true;
+            if (!wide && t > 4.0f * 1.00000381f) return false;
+            const double4_32a pj = posh[j[u]];
+            const double Rj = 2.0 * pj.w;
+            return exact_r2_def(posh[i], pj, zw.per, kp.lz) < __dmul_rn(Rj, Rj);
+        };
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             if (U > 1 && e0 + u * T >= len) break;
             acc = dfl::addf(acc, term[u]);
-            if (append) {
-                const float t = tq[u];
-                const bool wide = zw.per && hj[u] * zw.lzh < 8.0f;
-                bool in_j;
-                if (!wide && t < 4.0f * 0.99999619f) {
-                    in_j = true;
-                } else if (!wide && t > 4.0f * 1.00000381f) {
-                    in_j = false;
-                } else {
-                    const double4_32a pj = posh[j[u]];
-                    const double Rj = 2.0 * pj.w;
-                    in_j = exact_r2_def(posh[i], pj, zw.per, kp.lz) < __dmul_rn(Rj, Rj);
-                }
-                if (!in_j) ap.add(i, j[u], R.ngather, O);  // i belongs in the outer part of row j
-            }
+            if (A == 1 && append && !in_row(u)) ap[0].add(i, j[u], R.ngather, O);
+        }
+        if (A > 1 && append) {
+            bool out[U];  // i belongs in the outer part of row j
+#pragma unroll
+            for (int u = 0; u < U; ++u) out[u] = e0 + u * T < len && !in_row(u);
+#pragma unroll
+            for (int u = 0; u < A; ++u)
+                if (out[u]) ap[u].flush(i, O);
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (out[u]) ap[u % A].add(i, j[u], R.ngather, O);
         }
     }
-    if (OUTER) ap.flush(i, O);
+    if (OUTER) {
+#pragma unroll
+        for (int u = 0; u < A; ++u) ap[u].flush(i, O);
+    }
     }
     if (T > 1) {
         acc = dfl::lane_sum<T>(acc);
@@ -436,13 +448,14 @@ template <bool FUSE, int T, bool OUTER>
 static void density_mx_t(sph_ctx* c, cudaStream_t s) {
     const int64_t n = c->n;
     const int b = c->cur;
-    auto go = [&](auto kernel_fn, int U) {
-        const unsigned tb = U > 1 ? kPairBlockMin : kThreads;
+    auto go = [&](auto kernel_fn) {
+        const unsigned tb = kPairBlockMin;
         kernel_fn<<<(unsigned)((n * T + tb - 1) / tb), tb, 0, s>>>(
             n, batch_of(c), c->posh[b], c->ue[b], c->mpk, OUTER ? rows_gather(c) : rows_of(c),
             c->therm, c->pint, c->cint, c->status, OuterOut{c->rslab, c->ocnt, c->status});
     };
-    go(k_density_mx<FUSE, T, OUTER, 4>, 4);
+    if (OUTER && n <= kPairUnrollN) go(k_density_mx<FUSE, T, OUTER, 4, OUTER ? 4 : 1>);
+    else go(k_density_mx<FUSE, T, OUTER, 4, 1>);
 }
 
 template <bool FUSE, bool OUTER>
