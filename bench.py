@@ -88,19 +88,19 @@ FLOPS_PAIR_TABLE = 75
 # used only while the kernel's sources hash to the captured version (sha1 of
 # the files listed, in order); otherwise the bench reports null.
 NCU_EVIDENCE = {
-    # k_forces_df<2, M4>, the 1M patch, second step of the timed call
-    "df": {"sources": ("physics_df.cu", "df.cuh"), "sha1": "f8d02101d48d3d37cc808df61a0e0cc2ec302d17",
-           "dram_bytes": (697.33 + 44.48) * 1e6, "warp_inst": 1708627293,
-           "issue_active": 73.42, "pairs": 100727656,
+    # k_forces_df<2, M4, 4>, the 1M patch, second step of the timed call
+    "df": {"sources": ("physics_df.cu", "df.cuh"), "sha1": "6b34b61419cb667bdd22b4617dfddfc08bd76086",
+           "dram_bytes": (697.69 + 38.97) * 1e6, "warp_inst": 1617169777,
+           "issue_active": 76.46, "pairs": 100727656,
            "profile": "profiles/forces_patch1m_evrard1m.md"},
     # k_forces_mx<2>, the 1M Evrard sphere, mixed precision
-    "mixed": {"sources": ("physics_mixed.cu", "df.cuh"), "sha1": "342c531574d34f46723d3a8d907325d05aed3aee",
-              "dram_bytes": (650.91 + 37.92) * 1e6, "warp_inst": 583622306,
-              "issue_active": 47.63, "pairs": 105700202,
+    "mixed": {"sources": ("physics_mixed.cu", "df.cuh"), "sha1": "f3c32d039da8447eefa0c3ba066a1764a8952a78",
+              "dram_bytes": (650.85 + 37.97) * 1e6, "warp_inst": 583622378,
+              "issue_active": 47.60, "pairs": 105700202,
               "profile": "profiles/forces_patch1m_evrard1m.md"},
     # k_forces<M4>, the 1M patch, native FP64 pair sums
-    "fp64": {"sources": ("physics.cu",), "sha1": "6247f00dbf82cc04d06456dd9af9a433de9cf7fe",
-             "dram_bytes": (654.77 + 37.64) * 1e6, "warp_inst": 1248076044,
+    "fp64": {"sources": ("physics.cu",), "sha1": "12b17fe0c829156a517c097abcffbd823c552bce",
+             "dram_bytes": (655.07 + 37.67) * 1e6, "warp_inst": 1248069518,
              "issue_active": 7.48, "pairs": 100727656,
              "profile": "profiles/forces_patch1m_evrard1m.md"},
 }
