@@ -642,7 +642,7 @@ k_radix_scatter(const uint32_t* __restrict__ kin, const int32_t* __restrict__ vi
     // thread d: keys of digit d in all tiles, and in the tiles before this one
     uint32_t total = 0, before = 0;
     {
-        static_assert(kThreads == 256, "one digit per thread");
+        static_assert(kThreads == 256 && kRadixThreads == kThreads, "one digit per thread");
         const int d = threadIdx.x;
         const int tile = (int)blockIdx.x;
         if (R.groups == 1) {
@@ -752,35 +752,6 @@ k_permute(int64_t ntot, Batch B, const int64_t* __restrict__ roff,
     order_out[k] = order_in[o];
     fpos[k] = make_float4((float)p.x, (float)p.y, (float)p.z, 0.0f);
     ocnt[k] = 0;  // outer entries of the row, to be appended
-}
-
-// Tiles of the sort for nt keys. Up to kRadixSmallN a chained sort with tiles
-// of 512 keys, so that there are blocks enough for the chip: keys and passes
-// take 39 us at 104k keys and 45 us at 200k against 50 and 58 us with a
-// histogram kernel per pass and tiles of 2048; at 1M the additions contend
-// and it is 147 us against 73.
-static RadixGeom radix_geom(int64_t nt) {
-    RadixGeom R;
-    R.chained = nt <= kRadixSmallN;
-    R.items = R.chained ? kRadixItemsSmall : kRadixItems;
-    const int64_t tile = (int64_t)kThreads * R.items;
-    R.tile_shift = 0;
-    while ((int64_t)1 << R.tile_shift < tile) R.tile_shift += 1;
-    R.tiles = (int)((nt + tile - 1) / tile);
-    // up to 64 tiles: a block reads the counts of every tile; more: groups of
-    // about sqrt(tiles), one count per group and one per earlier tile of its own
-    R.group_shift = 4;
-    while (((int64_t)4 << (2 * R.group_shift)) < R.tiles) R.group_shift += 1;
-    if (R.tiles <= 64) R.group_shift = 6;
-    R.groups = ((R.tiles - 1) >> R.group_shift) + 1;
-    return R;
-}
-
-// Counts of one pass for at most n keys.
-int64_t radix_counts(int64_t n) {
-    const int64_t a = radix_geom(n).counts();
-    const int64_t b = radix_geom(n < kRadixSmallN ? n : kRadixSmallN).counts();
-    return a > b ? a : b;
 }
 
 void launch_build_cells(sph_ctx* c, cudaStream_t s) {

@@ -19,15 +19,13 @@
 #include <stdint.h>
 
 #include "../../include/sph.h"
+#include "radix_geom.cuh"
 
 namespace sph {
 
 constexpr int kMortonBits = 8;                      // bits per axis -> 24-bit keys
 constexpr int kMaxCellsPerAxis = 1 << kMortonBits;  // 256
 constexpr int kThreads = 256;
-constexpr int kRadixItems = 8;                      // keys per thread in the sort
-constexpr int kRadixItemsSmall = 2;                 // ... of at most kRadixSmallN keys
-constexpr int64_t kRadixSmallN = 262144;
 constexpr int kScanTile = kThreads * 8;             // elements per block in scans
 constexpr int kReduceBlocks = 304;                  // 2 x 152 SMs
 constexpr int kMaxPairThreads = 8;                  // lanes per particle in the pair kernels
@@ -259,23 +257,6 @@ inline KParams kparams(const sph_params* p) {
     }
     return k;
 }
-
-// Tiling of the radix sort, and the digit counts of one of its passes: per
-// tile [tiles][256], then per group of 2^group_shift tiles [groups][256].
-struct RadixGeom {
-    bool chained;  // each pass counts for the next (else a histogram kernel does)
-    int items, tiles, groups, tile_shift, group_shift;
-    __host__ __device__ int64_t counts() const { return (int64_t)(tiles + groups) * 256; }
-    // c keys of tile t have `digit`
-    __device__ __forceinline__ void count(uint32_t* hist, int64_t t, uint32_t digit,
-                                          uint32_t c) const {
-        if (c == 0) return;
-        atomicAdd(&hist[t * 256 + digit], c);
-        if (groups > 1)
-            atomicAdd(&hist[((int64_t)tiles + (t >> group_shift)) * 256 + digit], c);
-    }
-};
-int64_t radix_counts(int64_t n);  // counts of one pass for at most n keys
 
 }  // namespace sph
 
