@@ -1129,11 +1129,11 @@ k_h_count(int64_t n, Batch B, double4_32a* posh, const float4* __restrict__ fpos
                         if (sizeof(CountPlace<W>) == 2)
                             asm volatile("{.reg .pred p; setp.lt.f32 p, %1, 0f00000000;\n\t"
                                          "@p st.shared.u16 [%0], %2;\n\t@p add.u32 %0, %0, %3;}"
-                                         : "+r"(at) : "f"(d[k]), "r"(id + k0 + k), "n"(kRow));
+                                         : "+r"(at) : "f"(d[k]), "r"(id + k0 + k), "n"(kRow) : "memory");
                         else
                             asm volatile("{.reg .pred p; setp.lt.f32 p, %1, 0f00000000;\n\t"
                                          "@p st.shared.u8 [%0], %2;\n\t@p add.u32 %0, %0, %3;}"
-                                         : "+r"(at) : "f"(d[k]), "r"(id + k0 + k), "n"(kRow));
+                                         : "+r"(at) : "f"(d[k]), "r"(id + k0 + k), "n"(kRow) : "memory");
                     }
                 }
                 again = __any_sync(kFull, !(mn > w));  // a candidate in some lane's band
