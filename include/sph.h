@@ -47,7 +47,8 @@ typedef enum {
                             affected step are not valid; recreate with more capacity */
     SPH_E_HNOCONV = 5,   /* some particle's h search ended outside n_target +- n_tol;
                             results are still computed with its last h */
-    SPH_E_TIMEOUT = 6,   /* reserved for bounded device waits */
+    SPH_E_TIMEOUT = 6,   /* a bounded wait on the device saw no progress for some 15 s and
+                            gave up: outputs of the affected step are not valid */
     SPH_E_RANGE = 7,     /* precision 0 or 1: some per-particle quantity of the pair
                             kernels lies outside the range they hold (see below); the
                             density and force outputs of the affected step are not

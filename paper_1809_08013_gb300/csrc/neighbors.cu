@@ -28,8 +28,6 @@
 // further counts 32 particles at a time (k_h_union).
 #include <math_constants.h>
 
-#include <cooperative_groups.h>
-
 #include <algorithm>
 #include <type_traits>
 
@@ -1682,32 +1680,31 @@ k_compose(int64_t n, const int32_t* __restrict__ rowlen, const int32_t* __restri
     for (int s = lane; s < len; s += 32) idx[off + s] = __ldg(&rslab[i * kRSlab + s]);
 }
 
-// Fallback (a row overflowed a slab): the full two-pass build below.
-// FILL = false: rowlen[i] = |S_i|, ngather[i] = |N_i|.
-// FILL = true : write row i at offsets[i] (N_i first) with ballot-compacted,
-//               coalesced stores.
+// Fallback (a row overflowed a slab): the full two-pass build below. One warp,
+// row i of an instance with grid g:
+// FILL = false: rowlen[i] = |S_i|, ngather[i] = |N_i|; returns |S_i|.
+// FILL = true : write the row (of rowlen[i] entries) at idx + first, N_i first,
+//               with ballot-compacted, coalesced stores.
 // A cell is visited when its box lies within 2 max(h_i, max h of the cell).
 template <bool FILL>
-__device__ __forceinline__ void csr_rows(
-    int64_t n, const Batch& B, const double4_32a* __restrict__ posh, const float4* fpos,
-    const float* tin, const int2* __restrict__ cells, const unsigned long long* cell_hmax,
-    int32_t* rowlen, int32_t* ngather, const int64_t* offsets, int32_t* __restrict__ idx,
-    int* delta) {
+__device__ __forceinline__ int csr_row(int64_t i, const Batch& B,
+                                       const double4_32a* __restrict__ posh, const float4* fpos,
+                                       const float* tin, const int2* __restrict__ cells,
+                                       const unsigned long long* cell_hmax, int32_t* rowlen,
+                                       int32_t* ngather, int64_t first, int32_t* __restrict__ idx,
+                                       int* delta) {
     const int lane = threadIdx.x & 31;
-    const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t i = gw; i < n; i += nwarps) {  // persistent: one warp per particle in turn
     const int inst = slot_inst(B, i);
     if (!slot_real(B, inst, i)) {
         if (!FILL && lane == 0) {
             rowlen[i] = 0;
             ngather[i] = 0;
         }
-        continue;
+        return 0;
     }
     const Grid* __restrict__ g = B.grid + inst;
     const int2* __restrict__ cl = cells + g->cbase;
-    const unsigned long long* __restrict__ chm = cell_hmax + g->cbase;
+    const unsigned long long* chm = cell_hmax + g->cbase;
     const double4_32a pi = posh[i];
     const float4 fi = fpos[i];
     const float tin_i = tin[i];
@@ -1716,11 +1713,11 @@ __device__ __forceinline__ void csr_rows(
     const float Rbig = reach_f32(__longlong_as_double(hgb > hib ? hgb : hib));
     double R2i = -1.0;
     const unsigned lt = (1u << lane) - 1u;
-    int64_t pg = 0, po = 0, pg_end = 0, po_end = 0;
+    int64_t pg = 0, po = 0, po_end = 0;
     if (FILL) {
-        pg = offsets[i];
-        pg_end = po = pg + ngather[i];
-        po_end = offsets[i + 1];
+        pg = first;
+        po = pg + ngather[i];
+        po_end = pg + rowlen[i];
     }
     int cg = 0, co = 0;
     particle_pass<2>(g, cl, chm, fpos, fi, Rbig, hib, delta,
@@ -1753,7 +1750,7 @@ __device__ __forceinline__ void csr_rows(
         if (FILL) {
             if (in_i) {
                 const int64_t q = pg + cg + __popc(gm & lt);
-                if (q < pg_end) idx[q] = j;
+                if (q < po) idx[q] = j;
             } else if (in_j) {
                 const int64_t q = po + co + __popc(om & lt);
                 if (q < po_end) idx[q] = j;
@@ -1766,106 +1763,194 @@ __device__ __forceinline__ void csr_rows(
         rowlen[i] = cg + co;
         ngather[i] = cg;
     }
-    }
+    return cg + co;
 }
 
-// The whole fallback in one cooperative kernel: thresholds and the cells' max
-// h, row lengths, their scan, rows, with grid barriers between. Without the
-// flag every block returns at once: a step launches this twice, where the
-// passes and the scan as kernels of their own made ten launches that did
-// nothing (and two more kernels prepared in every step what only they read).
+// Wait, all threads of the block together, until *done items are done. False
+// when kCsrIdle looks in a row (half a microsecond apart on average, so some 15 s)
+// found no progress: reported (SPH_E_TIMEOUT), and the rows count as over
+// capacity, so that nothing reads them.
+constexpr int kCsrIdle = 1 << 25;
+__device__ __forceinline__ bool csr_wait(const unsigned* done, unsigned target, int64_t* total,
+                                         int64_t nnzcap, unsigned* status) {
+    __shared__ bool s_ok;
+    if (threadIdx.x == 0) {
+        unsigned seen = 0u;
+        bool ok = false;
+        for (int idle = 0; idle < kCsrIdle; ++idle) {
+            const unsigned v = *(volatile const unsigned*)done;
+            ok = v >= target;
+            if (ok) break;
+            if (v != seen) idle = 0;
+            seen = v;
+            __nanosleep(500);
+        }
+        if (!ok) {
+            atomicOr(&status[0], (unsigned)ST_TIMEOUT);
+            *(volatile int64_t*)total = nnzcap + 1;
+        }
+        __threadfence();
+        s_ok = ok;
+    }
+    __syncthreads();
+    return s_ok;
+}
+
+// An item of a phase is done (all threads together); the number done before it,
+// valid in every thread.
+__device__ __forceinline__ unsigned csr_done(unsigned* done) {
+    __shared__ unsigned s_before;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        s_before = atomicAdd(done, 1u);
+        __threadfence();
+    }
+    __syncthreads();
+    return s_before;
+}
+
+// Rows of an item, of the 8 warps of a block in turn: the most while that leaves
+// kCsrItems items for every block, else fewer, down to one a warp. A step of
+// 90,003 particles with rows of 140 entries takes 1,988 us at two items a block
+// (the last ones leave blocks idle), 1,886 at four, 1,915 at eight.
+constexpr int kCsrWarps = kThreads / 32;
+constexpr int kCsrRowsMax = 8, kCsrItems = 4;
+__device__ __forceinline__ int csr_rows_per_item(int64_t n, int blocks) {
+    const int64_t r = n / (kCsrItems * (int64_t)kCsrWarps * blocks);
+    return kCsrWarps * (r < 1 ? 1 : (r > kCsrRowsMax ? kCsrRowsMax : (int)r));
+}
+
+// The whole fallback in one kernel. Without the flag every block returns at
+// once: a step launches this twice, where the passes and the scan as kernels of
+// their own made ten launches that did nothing (and two more kernels prepared in
+// every step what only they read). Three phases of items: thresholds and the
+// cells' max h; row lengths, summed per item, the sums scanned by whoever counts
+// the last; offsets and rows. Blocks draw their items from one counter, in the
+// order of the phases, and an item waits only for earlier phases, whose items all
+// belong to blocks that run already: it ends for any number of resident blocks. (A
+// cooperative launch with grid barriers, which needs all its blocks resident
+// together, held back the work of other contexts: two contexts of 4,096
+// particles on two streams took 251 us a step of both, now 186; eight of 27,000
+// 1,303 and 1,070.)
 __global__ void __launch_bounds__(kThreads)
-k_csr_fallback(int64_t n, int ninst, Batch B, Grid* gw_, const double4_32a* __restrict__ posh,
-               float4* fpos, float* tin, const int2* __restrict__ cells,
-               unsigned long long* cell_hmax, int32_t* rowlen, int32_t* ngather, int64_t* offsets,
-               int64_t* part, int32_t* __restrict__ idx, int64_t nnzcap, unsigned* status,
-               unsigned mask) {
+k_csr_fallback(int64_t n, Batch B, Grid* gw_, const double4_32a* __restrict__ posh, float4* fpos,
+               float* tin, const int2* __restrict__ cells, unsigned long long* cell_hmax,
+               int32_t* rowlen, int32_t* ngather, int64_t* offsets, int64_t* part,
+               int32_t* __restrict__ idx, int64_t nnzcap, unsigned* status, unsigned mask,
+               CsrSync* Y) {
     if (!(*(volatile unsigned*)&status[2] & mask)) return;  // the slab path built the list
-    __shared__ int s_delta[kThreads / 32][32];
-    __shared__ int64_t s_sum[kThreads / 32];
-    const cooperative_groups::grid_group grid = cooperative_groups::this_grid();
+    __shared__ int s_delta[kCsrWarps][32];
+    __shared__ int64_t s_sum[kCsrWarps];
+    __shared__ int64_t s_off[kCsrWarps * kCsrRowsMax];
+    __shared__ unsigned s_item;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t nt = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = t0; i < n; i += nt) write_thresholds(i, B, posh, fpos, tin);
-    for (int k = 0; k < ninst; ++k) {
-        const long long nc = B.grid[k].ncells, cb = B.grid[k].cbase;
-        long long most = 0;  // bits of positive doubles order like their values
-        for (long long c = t0; c < nc; c += nt) {
-            const int2 se = cells[cb + c];
-            long long m = 0;
-            for (int q = se.x; q < se.y; ++q) {
-                const long long hb = __double_as_longlong(posh[q].w);
-                m = (hb > m && hb <= kHMaxBits) ? hb : m;  // (h outside the geometry range: not counted)
+    const int rows = csr_rows_per_item(n, (int)gridDim.x);
+    const unsigned nprep = (unsigned)((n + kThreads - 1) / kThreads);
+    const unsigned nrow = (unsigned)((n + rows - 1) / rows);
+    for (;;) {
+        __syncthreads();
+        if (threadIdx.x == 0) s_item = atomicAdd(&Y->next, 1u);
+        __syncthreads();
+        unsigned t = s_item;
+        if (t < nprep) {  // 256 slots, of one instance, and their share of its cells
+            const int64_t i = (int64_t)t * kThreads + threadIdx.x;
+            const int inst = slot_inst(B, (int64_t)t * kThreads);
+            if (i < n) write_thresholds(i, B, posh, fpos, tin);
+            const int64_t all = (__ldg(&B.icnt[inst]) + kThreads - 1) / kThreads * kThreads;
+            const long long nc = B.grid[inst].ncells, cb = B.grid[inst].cbase;
+            long long most = 0;  // bits of positive doubles order like their values
+            for (long long c = i - __ldg(&B.ioff[inst]); c < nc; c += all) {
+                const int2 se = cells[cb + c];
+                long long m = 0;
+                for (int q = se.x; q < se.y; ++q) {
+                    const long long hb = __double_as_longlong(posh[q].w);
+                    m = (hb > m && hb <= kHMaxBits) ? hb : m;  // (h outside the geometry range: not counted)
+                }
+                cell_hmax[cb + c] = (unsigned long long)m;
+                most = m > most ? m : most;
             }
-            cell_hmax[cb + c] = (unsigned long long)m;
-            most = m > most ? m : most;
+            if (most > 0) atomicMax(&gw_[inst].hmax_bits, (unsigned long long)most);
+            csr_done(&Y->prepared);
+            continue;
         }
-        if (most > 0) atomicMax(&gw_[k].hmax_bits, (unsigned long long)most);
-    }
-    grid.sync();
-    csr_rows<false>(n, B, posh, fpos, tin, cells, cell_hmax, rowlen, ngather, offsets, idx,
-                    s_delta[warp]);
-    grid.sync();
-    // exclusive scan of the row lengths: a contiguous range of rows per block
-    const int64_t per = (n + gridDim.x - 1) / gridDim.x;
-    const int64_t r0 = min(per * blockIdx.x, n), r1 = min(r0 + per, n);
-    auto block_sum = [&](int64_t v) {
+        t -= nprep;
+        if (t < nrow) {
+            if (!csr_wait(&Y->prepared, nprep, offsets + n, nnzcap, status)) return;
+            const int64_t i0 = (int64_t)t * rows;
+            int64_t sum = 0;
+            for (int r = warp; r < rows && i0 + r < n; r += kCsrWarps)
+                sum += csr_row<false>(i0 + r, B, posh, fpos, tin, cells, cell_hmax, rowlen, ngather,
+                                      0, idx, s_delta[warp]);
+            if (lane == 0) s_sum[warp] = sum;
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                int64_t a = 0;
+                for (int w = 0; w < kCsrWarps; ++w) a += s_sum[w];
+                part[t] = a;
+            }
+            if (csr_done(&Y->counted) + 1 != nrow) continue;
+            // the last item counted: exclusive scan of the items' sums
+            int64_t before = 0;
+            for (unsigned q0 = 0; q0 < nrow; q0 += kThreads) {
+                const unsigned q = q0 + threadIdx.x;
+                const int64_t v = q < nrow ? part[q] : 0;
+                int64_t inc = v;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
-        __syncthreads();
-        if (lane == 0) s_sum[warp] = v;
-        __syncthreads();
-        int64_t a = 0;
-        for (int w = 0; w < kThreads / 32; ++w) a += s_sum[w];
-        return a;
-    };
-    int64_t mine = 0;
-    for (int64_t i = r0 + threadIdx.x; i < r1; i += blockDim.x) mine += rowlen[i];
-    mine = block_sum(mine);
-    if (threadIdx.x == 0) part[blockIdx.x] = mine;
-    grid.sync();
-    int64_t before = 0;
-    for (int q = threadIdx.x; q < (int)blockIdx.x; q += blockDim.x) before += part[q];
-    before = block_sum(before);
-    for (int64_t i0 = r0; i0 < r1; i0 += blockDim.x) {
-        const int64_t i = i0 + threadIdx.x;
-        const int64_t len = i < r1 ? rowlen[i] : 0;
-        int64_t inc = len;
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int64_t u = __shfl_up_sync(kFull, inc, o);
+                    if (lane >= o) inc += u;
+                }
+                __syncthreads();
+                if (lane == 31) s_sum[warp] = inc;
+                __syncthreads();
+                int64_t off = before;
+                for (int w = 0; w < kCsrWarps; ++w) {
+                    off += w < warp ? s_sum[w] : 0;
+                    before += s_sum[w];
+                }
+                if (q < nrow) part[q] = off + inc - v;
+            }
+            if (threadIdx.x == 0) {
+                *(volatile int64_t*)&offsets[n] = before;
+                if (before > nnzcap) atomicOr(&status[0], (unsigned)ST_CAPACITY);
+            }
+            csr_done(&Y->scanned);
+            continue;
+        }
+        t -= nrow;
+        if (t >= nrow || !csr_wait(&Y->scanned, 1u, offsets + n, nnzcap, status)) return;
+        const int64_t i0 = (int64_t)t * rows;
+        if (warp == 0) {  // offsets of the item's rows (at most two a lane)
+            static_assert(kCsrWarps * kCsrRowsMax == 64, "two rows a lane");
+            const int64_t ia = i0 + 2 * lane;
+            const int64_t a = 2 * lane < rows && ia < n ? rowlen[ia] : 0;
+            const int64_t b = 2 * lane + 1 < rows && ia + 1 < n ? rowlen[ia + 1] : 0;
+            int64_t inc = a + b;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int64_t v = __shfl_up_sync(kFull, inc, o);
-            if (lane >= o) inc += v;
+            for (int o = 1; o < 32; o <<= 1) {
+                const int64_t u = __shfl_up_sync(kFull, inc, o);
+                if (lane >= o) inc += u;
+            }
+            const int64_t off = part[t] + inc - (a + b);
+            s_off[2 * lane] = off;
+            s_off[2 * lane + 1] = off + a;
+            if (2 * lane < rows && ia < n) offsets[ia] = off;
+            if (2 * lane + 1 < rows && ia + 1 < n) offsets[ia + 1] = off + a;
         }
         __syncthreads();
-        if (lane == 31) s_sum[warp] = inc;
-        __syncthreads();
-        int64_t off = before;
-        for (int w = 0; w < warp; ++w) off += s_sum[w];
-        if (i < r1) {
-            offsets[i] = off + inc - len;
-            if (i == n - 1) offsets[n] = off + inc;
-        }
-        for (int w = warp; w < kThreads / 32; ++w) off += s_sum[w];
-        before = off;
+        if (*(volatile int64_t*)&offsets[n] > nnzcap) continue;
+        for (int r = warp; r < rows && i0 + r < n; r += kCsrWarps)
+            csr_row<true>(i0 + r, B, posh, fpos, tin, cells, cell_hmax, rowlen, ngather, s_off[r],
+                          idx, s_delta[warp]);
     }
-    grid.sync();
-    if (*(volatile int64_t*)&offsets[n] > nnzcap) {
-        if (t0 == 0) atomicOr(&status[0], (unsigned)ST_CAPACITY);
-        return;
-    }
-    csr_rows<true>(n, B, posh, fpos, tin, cells, cell_hmax, rowlen, ngather, offsets, idx,
-                   s_delta[warp]);
 }
 
-// Blocks of k_csr_fallback resident at once on this device (0: none).
-int csr_fallback_blocks(int nsm) {
-    int per = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_csr_fallback, kThreads, 0) != cudaSuccess) {
-        cudaGetLastError();
-        return 0;
-    }
-    return std::min(per, 4) * nsm;
+// Blocks of the fallback, and the items of at most n rows: of kCsrRowsMax rows a
+// warp, or of r < kCsrRowsMax, and then n < (r + 1) kCsrItems kCsrWarps blocks.
+int csr_fallback_blocks(int nsm) { return 4 * nsm; }
+int64_t csr_fallback_parts(int64_t n, int nsm) {
+    return n / (kCsrWarps * kCsrRowsMax) + 2 * kCsrItems * (int64_t)csr_fallback_blocks(nsm) + 2;
 }
 
 void launch_h_search(sph_ctx* c, cudaStream_t s) {
@@ -1920,18 +2005,14 @@ void launch_h_search(sph_ctx* c, cudaStream_t s) {
 }
 
 // The two-pass CSR build, for the rows flagged in status[2] & mask (launched
-// every step; without the flag it returns at once).
+// every step; without the flag it returns at once). The step's two launches
+// have their own counters (CsrSync, cleared with every build).
 static void csr_fallback(sph_ctx* c, cudaStream_t s, unsigned mask) {
-    int64_t n = c->n, cap = c->nnzcap;
-    int ninst = c->ninst;
-    const double4_32a* posh = c->posh[c->cur];
-    Batch B = batch_of(c);
     c->launches += 1;
-    void* args[] = {&n, &ninst, &B, &c->grid, &posh, &c->fpos, &c->tin, &c->cells, &c->cell_hmax,
-                    &c->rowlen, &c->ngather, &c->offsets, &c->row_part, &c->idx, &cap, &c->status,
-                    &mask};
-    cudaLaunchCooperativeKernel((const void*)k_csr_fallback, dim3((unsigned)c->csr_blocks),
-                                dim3(kThreads), args, 0, s);
+    k_csr_fallback<<<(unsigned)csr_fallback_blocks(c->nsm), kThreads, 0, s>>>(
+        c->n, batch_of(c), c->grid, c->posh[c->cur], c->fpos, c->tin, c->cells, c->cell_hmax,
+        c->rowlen, c->ngather, c->offsets, c->row_part, c->idx, c->nnzcap, c->status, mask,
+        c->csync + (mask == (unsigned)IF_OUTER_OVF ? 1 : 0));
 }
 
 static void rowlen_sort(sph_ctx* c, cudaStream_t s, unsigned mask) {

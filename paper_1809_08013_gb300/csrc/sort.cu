@@ -319,7 +319,7 @@ constexpr int kGridThreads = 1024;
 __global__ void __launch_bounds__(kGridThreads)
 k_grid_setup(const double* __restrict__ part, Batch B, Grid* __restrict__ grid,
              unsigned* __restrict__ status, unsigned long long* __restrict__ wctr,
-             unsigned* __restrict__ lctr) {
+             unsigned* __restrict__ lctr, CsrSync* __restrict__ csync) {
     const int inst = blockIdx.x;
     const int64_t n = B.icnt[inst];
     const int64_t b0 = B.ioff[inst] / kSlotAlign;
@@ -393,6 +393,7 @@ k_grid_setup(const double* __restrict__ part, Batch B, Grid* __restrict__ grid,
         status[3] = 0u;
         wctr[0] = 0ull;
         wctr[1] = 0ull;
+        csync[0] = csync[1] = CsrSync{0u, 0u, 0u, 0u};
     }
     const double hmean = n > 0 ? hs / (double)n : 1.0;
     double w = 2.0 * hmean * kp.cell_scale;
@@ -777,7 +778,7 @@ void launch_build_cells(sph_ctx* c, cudaStream_t s) {
                                                   passes * R.counts());
     }
     k_grid_setup<<<c->ninst, kGridThreads, 0, s>>>(c->red_part, B, c->grid, c->status, c->wctr,
-                                                    c->lctr);
+                                                    c->lctr, c->csync);
     if (n == 0) return;
     if (nt == 0) return;
     const unsigned nbt = (unsigned)((nt + kThreads - 1) / kThreads);

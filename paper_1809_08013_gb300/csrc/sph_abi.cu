@@ -145,7 +145,7 @@ void free_all(sph_ctx* c) {
     void* ptrs[] = {c->posh[0], c->posh[1], c->velm[0], c->velm[1], c->ue[0], c->ue[1],
                     c->therm, c->kern, c->acc, c->pint, c->cint, c->dpk, c->mpk, c->mumax, c->fpos, c->tin, c->order[0],
                     c->order[1], c->keys[0], c->keys[1], c->vals[0], c->vals[1], c->hist, c->cells, c->cell_hmax, c->nnb, c->ngather, c->rowlen,
-                    c->offsets, c->row_part, c->idx, c->rslab, c->ocnt, c->hs_lo, c->hs_hi, c->hs_it, c->wl, c->gwl, c->red_part, c->dt_part, c->grid,
+                    c->offsets, c->row_part, c->csync, c->idx, c->rslab, c->ocnt, c->hs_lo, c->hs_hi, c->hs_it, c->wl, c->gwl, c->red_part, c->dt_part, c->grid,
                     c->status, c->scratch_scalar, c->blk, c->ioff, c->icnt, c->coff, c->kpi,
                     c->tune_dt, c->roff, c->wctr, c->recs, c->iad_a, c->iad_b, c->vol, c->xpk, c->vpa, c->vpb,
                     c->stage, c->stage_nnb, c->vdf, c->cpk, c->lst, c->lmeta, c->lctr};
@@ -218,7 +218,8 @@ bool allocate_all(sph_ctx* c, int64_t nslots, Allocator& al) {
          al(&c->hist, 4 * (size_t)radix_counts((int64_t)N)) &&
          al(&c->cells, (size_t)c->cellcap) && al(&c->cell_hmax, (size_t)c->cellcap) &&
          al(&c->nnb, N) && al(&c->ngather, N) && al(&c->rowlen, N) &&
-         al(&c->offsets, N + 1) && al(&c->row_part, std::max<size_t>((size_t)scan_parts(N) + 1, 4 * (size_t)c->nsm)) &&
+         al(&c->offsets, N + 1) && al(&c->row_part, std::max<size_t>((size_t)scan_parts(N) + 1, (size_t)csr_fallback_parts((int64_t)N, c->nsm))) &&
+         al(&c->csync, 2) &&
          al(&c->idx, (size_t)nnzcap) && al(&c->red_part, (N + kSlotAlign - 1) / kSlotAlign * kBoxStride) &&
          al(&c->dt_part, nfb * kMaxPairThreads * (kThreads / kPairBlockMin)) && al(&c->grid, (size_t)max_instances) &&
          al(&c->status, 4) && al(&c->blk, nfb) &&
@@ -685,9 +686,8 @@ sph_status sph_ctx_create_batch(sph_ctx** out, int64_t ncap, int64_t nnzcap, int
         cudaGetLastError();
         c->nsm = 1;
     }
-    c->csr_blocks = csr_fallback_blocks(c->nsm);
     Allocator A{false, 0};
-    bool ok = c->csr_blocks > 0 && allocate_all(c, nslots, A);
+    bool ok = allocate_all(c, nslots, A);
     ok = ok && cudaMallocHost((void**)&c->status_host, 2 * sizeof(unsigned)) == cudaSuccess;
     ok = ok && cudaMemset(c->status, 0, 4 * sizeof(unsigned)) == cudaSuccess &&
          cudaMemset(c->offsets, 0, sizeof(int64_t)) == cudaSuccess &&
@@ -1213,6 +1213,10 @@ sph_status sph_sync(sph_ctx* c, void* stream) {
         set_err(c, "a particle's state was non-finite or outside the geometry range "
                    "(|x|, |y|, |z| <= FLT_MAX, 0 <= h <= 2^100)");
         return SPH_E_NONFINITE;
+    }
+    if (bits & ST_TIMEOUT) {
+        set_err(c, "the neighbour list build made no progress and was given up");
+        return SPH_E_TIMEOUT;
     }
     if (bits & ST_CAPACITY) {
         set_err(c, "neighbour list exceeded nnz capacity %lld", (long long)c->nnzcap);

@@ -40,6 +40,7 @@ enum : unsigned {
     ST_HNOCONV = 2u,    // some h search did not converge
     ST_RANGE = 4u,      // a float-pair quantity left the range of the pair kernels
     ST_NONFINITE = 8u,  // a particle's state was non-finite or outside the geometry range
+    ST_TIMEOUT = 16u,   // a wait of the CSR fallback saw no progress and gave up
 };
 
 // Geometry range of a particle (integer tests on the bits, no FP64 pipe): the
@@ -168,6 +169,12 @@ struct Grid {
     int lbuild, lstamp;
     float dm2;
     int gvalid;  // the geometry above is that of a list build (kept while the lists are)
+};
+
+// Counters of one launch of the CSR fallback (neighbors.cu): the next item, and
+// the items done of its phases.
+struct CsrSync {
+    unsigned next, prepared, counted, scanned;
 };
 
 // 2^e as a double, exactly (e in [-1022, 1023]); integer operations only.
@@ -305,7 +312,7 @@ struct sph_ctx {
     unsigned long long* cell_hmax;  // per cell, bits of max h (h > 0)
     int32_t *nnb, *ngather, *rowlen;
     int64_t* offsets;
-    int64_t* row_part;      // scan partials of the row lengths
+    int64_t* row_part;      // scan partials of the row lengths, sums of the CSR fallback's items
     int32_t* idx;
     int32_t* rslab;         // kRSlab per particle: row i of S_i = the gather set of the last
                             // h-search count (ngather[i]), then the outer set (ocnt[i],
@@ -332,7 +339,7 @@ struct sph_ctx {
     bool group_search;      // some instance has kGroupSearchN particles or more
     int lay_n;              // instances of the last batch layout (first, count) ...
     int64_t lay_first[sph::kMaxInstances], lay_cnt[sph::kMaxInstances];  // ... and theirs
-    int csr_blocks;         // blocks of the cooperative CSR fallback
+    sph::CsrSync* csync;    // counters of the step's two launches of the CSR fallback
     int nsm;                // streaming multiprocessors of the device
     unsigned* status;       // [0] bits, [1] non-converged count, [2] internal flags,
                             // [3] h-search worklist length
@@ -494,6 +501,7 @@ void launch_h_search(sph_ctx* c, cudaStream_t s);
 void launch_csr(sph_ctx* c, cudaStream_t s, bool outer_later = false);
 void launch_rows_finish(sph_ctx* c, cudaStream_t s);
 int csr_fallback_blocks(int nsm);
+int64_t csr_fallback_parts(int64_t n, int nsm);
 // the rows as a CSR in offsets / idx (a copy in slab form; nothing after a fallback)
 void launch_compose(sph_ctx* c, cudaStream_t s);
 

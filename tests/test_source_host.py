@@ -33,3 +33,10 @@ def test_asm_that_writes_memory_says_so():
                 seen += 1
                 assert '"memory"' in s, (name, s)
     assert seen > 0
+
+
+def test_no_launch_needs_the_whole_gpu():
+    # a cooperative launch starts only when all its blocks fit at once: contexts
+    # that step on streams of their own then wait for one another
+    for name, text in _sources().items():
+        assert "LaunchCooperative" not in text and "cooperative_groups" not in text, name
