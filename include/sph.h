@@ -333,7 +333,9 @@ typedef struct {
  * trials go to context scratch); the context keeps the chosen knobs for
  * sph_batch_step until the next sph_batch_set, and a single-problem call
  * takes them from its sph_params. space = NULL uses cell_scale {0.875, 1,
- * 1.25}, pair_threads {1, 2, 4}, defer_lanes {8, 16}. Synchronises the
+ * 1.25}, pair_threads {1, 2, 4}, defer_lanes {8, 16}. defer_lanes is tried
+ * where the batch's h search reads it: with candidate lists, or an instance of
+ * 100,000 particles or more; else it stays as it is. Synchronises the
  * stream (not capturable). SPH_E_INVAL for nsteps < 1, P->n too short for
  * the batch, invalid candidates or more than SPH_TUNE_MAX_TRIALS of them.
  * Device conditions of the trial runs (h non-convergence) stay in the

@@ -7,7 +7,8 @@
 // row a warp waits for and coalesce the row reads, at the price of a
 // cross-lane reduction), and the h-search hand-over threshold (how few
 // particles of a warp may still be searching before each gets a warp of its
-// own). The tuner times trial runs of the current batch from the caller's
+// own; read with candidate lists or an instance of kGroupSearchN particles, and
+// only then tried). The tuner times trial runs of the current batch from the caller's
 // state and keeps, knob by knob, the fastest value (one coordinate-descent
 // pass, in the order lanes, cell width, hand-over).
 #include <string.h>
@@ -137,7 +138,10 @@ extern "C" sph_status sph_autotune(sph_ctx* c, sph_particles* P, int nsteps,
         const Knobs b = best;
         if (sp.cell_scales[q] != b.cs) run(Knobs{sp.cell_scales[q], b.tpp, b.defer});
     }
-    for (int q = 0; q < sp.n_defer_lanes; ++q) {
+    // (a search that reads no defer_lanes runs the same with every value: k_h_count
+    // hands over all that goes on)
+    const bool deferring = c->any_lists || c->group_search;
+    for (int q = 0; deferring && q < sp.n_defer_lanes; ++q) {
         const Knobs b = best;
         if (sp.defer_lanes[q] != b.defer) run(Knobs{b.cs, b.tpp, sp.defer_lanes[q]});
     }
