@@ -41,3 +41,15 @@ def test_order_within_each_instance(capacity, counts):
         assert np.array_equal(order[a:a + counts[k]], want), k
         a += counts[k]
     ctx.close()
+
+
+def test_one_context_for_problems_of_other_sizes():
+    from paper_1809_08013_gb300 import binding as B
+    ctx = B.Context(300000, nnz_capacity=48 * 300000)
+    for n in (300000, 262145, 262144, 5000, 262145):  # with and without a histogram kernel
+        s, p = ics.evrard(n, seed=n)
+        s["h"][:] = 0.75 * n ** (-1.0 / 3.0)
+        p.n_target = p.n_tol = 8
+        ctx.build_neighbors(p, B.alloc_arrays(s))
+        assert np.array_equal(ctx.neighbors_to_host()[3], expected_order(s, max(2 * n, 4096))), n
+    ctx.close()
