@@ -47,8 +47,13 @@ __device__ __forceinline__ df add(df x, df y) {
 __device__ __forceinline__ df sub(df x, df y) { return add(x, neg(y)); }
 
 // x + y + z with one renormalisation (19 operations; two sums take 22): the high
-// parts by two TwoSums, all low parts folded in once, within ~2^-47 (|x| + |y| +
-// |z|) like two sums.
+// parts by two TwoSums, all low parts folded in once. The low parts meet in one
+// float sum, so its own error is 1.2 to 1.3 times that of two sums (r.m.s. and
+// worst case, random operands with low parts as products leave them). The outputs
+// do not show it: against 64 bits, patches and spheres of 4,096 to 150,000
+// particles, M4, Wendland and sinc, kernel derivatives and IAD, the r.m.s. errors
+// of a and du are within 0.1% of those with two sums in its place; that of mumax
+// is up to 0.7% larger.
 __device__ __forceinline__ df add3(df x, df y, df z) {
     const df a = two_sum(x.hi, y.hi);
     const df b = two_sum(a.hi, z.hi);

@@ -970,7 +970,7 @@ k_h_lists(int64_t n, Batch B, double4_32a* posh, const float4* __restrict__ fpos
 // Bound: instruction issue. Against testing, collecting bits and appending bit
 // by bit in one loop (the record passes of k_h_union), a candidate costs ~10
 // instead of ~16 instructions, the appends do not diverge chunk by chunk, and
-// a row takes a quarter of the stores. Measured (ncu, a steady step): 17.6k
+// a row takes a quarter of the stores. Measured (ncu, a steady step): 17.1k
 // warp instructions a group on the 70^3 patch (24.7k before); 1M patch 641 us
 // (940), 1M sphere 848 us (1,227), 8,191-particle sphere 46 us (232). Tried:
 // sign bits of a chunk shifted into a word and walked bit by bit at the end

@@ -185,26 +185,28 @@ __device__ __forceinline__ void eos_d(const KParams& kp, double rho, double u, d
 // KER: the M4 spline, the Wendland C2 or the sinc kernel.
 // OUTER: the kernel also decides, for each j of N_i, whether i is in N_j --
 // r_ij^2 < (2 h_j)^2 by the defining FP64 test -- and appends i to the outer
-// part of every row j where it is not (Append). The pair's double-float r^2 is within ~2^-45 of the defining FP64 value and
-// (2 h_j)^2 is packed as a float (within 2^-24), so r^2 below / above it by
-// more than 2^-20 decides; the band between takes the FP64 test itself. The
-// sets are the exact ones, as built by k_outer.
-// The next neighbour's loads go out before one is evaluated, in blocks of 64
-// threads: 1M patch 681 us (732 without, in blocks of 256; the branch-free shape
-// gave 38 us of that).
+// part of every row j where it is not (Append). The pair's double-float r^2 is
+// within ~2^-45 of the defining FP64 value and (2 h_j)^2 is packed as a float, up
+// to 2^-22 below its value (pair_reach2); with the roundings of the comparison
+// that is under 2^-21, so r^2 below / above it by more than 2^-20 decides; the
+// band between takes the FP64 test itself. The sets are the exact ones, as built
+// by k_outer.
 // U: neighbours evaluated at a time, their terms added in the order of the row
 // (the same bits for every U). A lane's append waits for the slot its last one
 // got, and in a warp some lane has one at almost every neighbour: while there
 // are too few warps to hide that (up to kPairUnrollN particles) four at a time,
-// each with an append of its own in flight: 4,096 particles 44 us (54), 27,000 43
-// (57). Beyond, one at a time: 104k 107 us (116), 1M 681 (807); two appends in
-// flight without the unrolling 721 at 1M.
+// each with an append of its own in flight; beyond, one at a time, the next
+// neighbour's loads ahead of it. In blocks of 64 threads. Density phase in us, four /
+// one at a time, patch: 8,000 particles 38 / 47, 27,000 43 / 52, 42,875 53 / 56,
+// 50,653 74 / 67, 104k 114 / 106, 1M 802 / 675 (732 without the loads ahead, in
+// blocks of 256); sphere: 8,000 39 / 49, 42,875 55 / 60, 50,653 83 / 68, 1M 920 /
+// 795. Two appends in flight without the unrolling: 721 at 1M.
 template <bool FUSE, int T, int KER, bool OUTER, int U>
 __global__ void __launch_bounds__(kPairBlockMin)
 k_density_df(int64_t n, Batch B, const double4_32a* __restrict__ posh,
              const float4* __restrict__ xpk, const double* __restrict__ ue,
              Rows R, double4_32a* __restrict__ therm,
-             double2* __restrict__ kern, float4* __restrict__ dpk, double* __restrict__ pint,
+             float4* __restrict__ dpk, double* __restrict__ pint,
              double* __restrict__ cint, unsigned* status, OuterOut O) {
     const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / T;
     const int sub = (int)(threadIdx.x % T);
@@ -376,7 +378,7 @@ static void density_df_t(sph_ctx* c, cudaStream_t s) {
     auto go = [&](auto kernel_fn) {
         const unsigned tb = kPairBlockMin;
         kernel_fn<<<(unsigned)((n * T + tb - 1) / tb), tb, 0, s>>>(
-            n, batch_of(c), c->posh[b], c->xpk, c->ue[b], R, c->therm, c->kern, c->dpk, c->pint,
+            n, batch_of(c), c->posh[b], c->xpk, c->ue[b], R, c->therm, c->dpk, c->pint,
             c->cint, c->status, OuterOut{c->rslab, c->ocnt, c->status});
     };
     if (c->kern_kind == KER_SINC) {

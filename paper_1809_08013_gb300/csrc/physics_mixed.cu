@@ -211,7 +211,7 @@ k_density_mx(int64_t n, Batch B, const double4_32a* __restrict__ posh,
         float term[U], tq[U], hj[U];
 #pragma unroll
         for (int u = 0; u < U; ++u)
-            j[u] = U == 1 || e0 + u * T < len ? __ldg(&ent[e0 + u * T]) : (int)i;
+            j[u] = e0 + u * T < len ? __ldg(&ent[e0 + u * T]) : (int)i;
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             const float4 b0 = __ldg(&mpk[5 * j[u]]), b1 = __ldg(&mpk[5 * j[u] + 1]);
@@ -235,7 +235,7 @@ k_density_mx(int64_t n, Batch B, const double4_32a* __restrict__ posh,
         };
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            if (U > 1 && e0 + u * T >= len) break;
+            if (e0 + u * T >= len) break;
             acc = dfl::addf(acc, term[u]);
             if (A == 1 && append && !in_row(u)) ap[0].add(i, j[u], R.ngather, O);
         }
@@ -267,9 +267,9 @@ k_density_mx(int64_t n, Batch B, const double4_32a* __restrict__ posh,
     if (FUSE) {
         double p, c;
         eos_m(kp, rho, ue[i], p, c);
-        const double A = p / (rho * rho);
-        therm[i] = make_double4_32a(0.5 * rho, A, 0.5 * kp.alpha * c, 0.5 * hd);
-        pack_thermo(mpk, i, hd, rho, A, kp.alpha, c, dfl::pair_units(g.uL, g.uM, g.uV), status);
+        const double prho2 = p / (rho * rho);
+        therm[i] = make_double4_32a(0.5 * rho, prho2, 0.5 * kp.alpha * c, 0.5 * hd);
+        pack_thermo(mpk, i, hd, rho, prho2, kp.alpha, c, dfl::pair_units(g.uL, g.uM, g.uV), status);
         pint[i] = p;
         cint[i] = c;
     } else {
@@ -488,7 +488,8 @@ static void forces_mx_t(sph_ctx* c, cudaStream_t s) {
     };
     // small batches, with a few warps per scheduler, are bound by the latency of
     // a pair, large ones by the L1 data pipe (us, U = 4 and U = 1: 8,191 particles
-    // 38 and 46, 30,000 48 and 54, 60,000 116 and 114, 1M 1,028 and 1,000)
+    // 38 and 46, 30,000 48 and 54, 42,875 69 and 74, 50,653 96 and 76, 104k 167 and
+    // 134, 1M 1,028 and 1,000)
     if (c->n <= kPairUnrollN) go(k_forces_mx<T, 4>, 4);
     else go(k_forces_mx<T, 1>, 1);
 }

@@ -36,10 +36,12 @@ struct RadixGeom {
 };
 
 // Tiles of the sort for nt keys. Up to kRadixSmallN a chained sort with tiles
-// of 512 keys, so that there are blocks enough for the chip: keys and passes
-// take 39 us at 104k keys and 45 us at 200k against 50 and 58 us with a
-// histogram kernel per pass and tiles of 2048; at 1M the additions contend
-// and it is 147 us against 73.
+// of 512 keys, so that there are blocks enough for the chip; beyond, where its
+// additions contend, a histogram kernel per pass and tiles of 2048. The line is
+// where the two cross. Cells phase (bounding box to permute) of a patch in us,
+// chained / with histograms: 4,096 keys 42 / 56, 27,000 52 / 66, 104k 73 / 85,
+// 195k 92 / 100, 262k 101 / 100, 301k 111 / 108, 405k 136 / 125, 1M 269 / 210; of
+// a sphere 200k 96 / 105, 262k 106 / 105, 300k 117 / 114.
 inline RadixGeom radix_geom(int64_t nt) {
     RadixGeom R;
     R.chained = nt <= kRadixSmallN;

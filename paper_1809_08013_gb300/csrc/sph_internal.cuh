@@ -29,7 +29,7 @@ constexpr int kThreads = 256;
 constexpr int kScanTile = kThreads * 8;             // elements per block in scans
 constexpr int kReduceBlocks = 304;                  // 2 x 152 SMs
 constexpr int kMaxPairThreads = 8;                  // lanes per particle in the pair kernels
-constexpr int64_t kPairUnrollN = 50000;             // see forces_mx_t
+constexpr int64_t kPairUnrollN = 50000;             // see k_density_df, forces_mx_t
 constexpr int kPairBlockMin = 64;                   // smallest block of the pair kernels
 constexpr int kBoxStride = 16;                      // doubles per bounding-box partial
 constexpr int kBoxWarpSlots = 64;                   // bounding box: slots per warp (4 per partial)
@@ -105,10 +105,16 @@ constexpr int kRec = 256;    // h search: candidates recorded per lane in flight
 // Instances of at least this many particles go on with a search that many
 // lanes of a warp have not finished in groups of 32 (k_h_union), the others one
 // warp per particle (k_h_iterate): a small problem has too few groups to hide
-// the latency of one. Measured for the first step of a patch (us): 104k
-// particles 641 in groups, 645 one by one; 1M 3,934 and 6,100; below that a
-// group has the chip to itself (27,000: 172 one by one). By the instance, not the batch: the two leave a row in another order,
-// and an instance gives the same bits alone and in a batch.
+// the latency of one. By the instance, not the batch: the two leave a row in
+// another order, and an instance gives the same bits alone and in a batch. First
+// step from the analytic h, whole call in us, in groups / one by one: patches of
+// 64,000 particles 974 / 790, 79,507 1,076 / 947, 97,336 1,153 / 1,113 (the
+// search alone at 104k 641 / 645, at 1M 3,934 / 6,100); spheres of 30,000 774 /
+// 408, 60,000 1,015 / 686, 90,000 1,196 / 910. Ten instances in one batch fill
+// the chip either way and cross lower: ten patches of 42,875 4,083 / 4,053,
+// 64,000 5,226 / 5,950, 91,125 6,793 / 8,674; ten spheres of 60,000 4,420 /
+// 4,285, of 90,000 6,298 / 6,258. The line is that of instances alone: such
+// batches of patches pay for it in their first step.
 constexpr int64_t kGroupSearchN = 100000;
 constexpr int kUnionBlocksPerSM = 4;  // resident blocks of the persistent h search
 // Candidate lists of the h search, kept across steps (neighbors.cu). While an
@@ -360,7 +366,7 @@ struct sph_ctx {
     int64_t timed_steps;
     // One step of the current batch as a CUDA graph, per parity of the
     // double-buffered state (cur at the start of the step), replayed by
-    // sph_step / sph_batch_step instead of its ~35 separate launches.
+    // sph_step / sph_batch_step instead of its 16 to 25 separate launches.
     struct StepGraph {
         bool valid;
         int64_t key[11];         // what the launches bake in (sizes, kinds, dt/time pointers,
@@ -408,8 +414,8 @@ inline Rows rows_gather(const sph_ctx* c) {
 }
 
 // At precision 0 and 1 the step's density kernel also decides the outer parts
-// and appends the outer parts of the rows (k_density_df / k_density_mx with
-// OUTER); at precision 2 and outside a step, k_outer builds them before it.
+// of the rows and appends them (k_density_df / k_density_mx with OUTER); at
+// precision 2 and outside a step, k_outer builds them before it.
 inline bool fused_outer(const sph_ctx* c) { return c->prec == PREC_FP64 || c->prec == PREC_MIXED; }
 
 // Threads per block of a pair kernel that evaluates U neighbours at a time.
