@@ -89,18 +89,18 @@ FLOPS_PAIR_TABLE = 75
 # the files listed, in order); otherwise the bench reports null.
 NCU_EVIDENCE = {
     # k_forces_df<2, M4, 4>, the 1M patch, second step of the timed call
-    "df": {"sources": ("physics_df.cu", "df.cuh"), "sha1": "279e63614b6c9646fa4bdeee7f9a11388b3c453a",
-           "dram_bytes": (697.72 + 39.12) * 1e6, "warp_inst": 1617169777,
-           "issue_active": 76.42, "pairs": 100727656,
+    "df": {"sources": ("physics_df.cu", "df.cuh"), "sha1": "e38fd0d1b31e2c9c9202acbbe92464df379f0ece",
+           "dram_bytes": (697.86 + 39.18) * 1e6, "warp_inst": 1617169777,
+           "issue_active": 76.46, "pairs": 100727656,
            "profile": "profiles/forces_patch1m_evrard1m.md"},
     # k_forces_mx<2>, the 1M Evrard sphere, mixed precision
     "mixed": {"sources": ("physics_mixed.cu", "df.cuh"), "sha1": "12bc2039db6d1731a243379f82330ecb4d2c62e6",
-              "dram_bytes": (651.21 + 37.71) * 1e6, "warp_inst": 583622378,
-              "issue_active": 47.76, "pairs": 105700202,
+              "dram_bytes": (650.85 + 37.95) * 1e6, "warp_inst": 583622378,
+              "issue_active": 47.52, "pairs": 105700202,
               "profile": "profiles/forces_patch1m_evrard1m.md"},
     # k_forces<M4>, the 1M patch, native FP64 pair sums
     "fp64": {"sources": ("physics.cu",), "sha1": "12b17fe0c829156a517c097abcffbd823c552bce",
-             "dram_bytes": (654.10 + 37.59) * 1e6, "warp_inst": 1248069518,
+             "dram_bytes": (655.49 + 37.70) * 1e6, "warp_inst": 1248069518,
              "issue_active": 7.48, "pairs": 100727656,
              "profile": "profiles/forces_patch1m_evrard1m.md"},
 }

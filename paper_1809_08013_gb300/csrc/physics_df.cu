@@ -423,9 +423,9 @@ void launch_density_df(sph_ctx* c, bool fuse_eos, cudaStream_t s, bool outer) {
 // U: neighbours evaluated at a time, their terms added in the order of the row
 // (the same bits for every U); with U > 1 the viscosity is evaluated for every
 // pair and selected, so that no branch keeps the U evaluations apart.
-// Bound: instruction dispatch (550 warp instructions a pair, mostly FP32 with
+// Bound: instruction dispatch (514 lane instructions a pair, mostly FP32 with
 // three register operands, which this GPU issues at 0.62 of the rate of the
-// others). U = 4 in blocks of 64 (160 registers, 12 warps an SM) against U = 1
+// others). U = 4 in blocks of 64 (168 registers, 12 warps an SM) against U = 1
 // in blocks of 256 (80 registers, 24 warps): 4,096 particles 44 us (91), 27,000
 // 70 (108), 104k 216 (247), 1M 1,795 (1,893); the Wendland kernel at 216,000
 // 427 (457). U = 3: 1,860 at 1M; 5 or 6: 2,330. The sinc shapes, with a loop
